@@ -491,7 +491,30 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
       return PIMPC_EINVAL;
     }
     e = admm_configure(precision, s->smem_admm, &bps);
+    RegLaunch reg;
     if (sc.family == 3 && e == cudaSuccess) {
+      // Stage data in registers where every instance has n <= 16 and fits: with item_scale = 0
+      // the fewest CTAs whose lanes stay within a target while the whole batch fits the SMs
+      // (FP64: four warps, one per scheduler, because a fifth shares the FP64 pipe; FP32: eight),
+      // else the fewest that hold an instance.
+      const int target = precision == PIMPC_F32 ? 256 : 128;
+      for (int cand : {1, 2, 4, 8, 16}) {
+        if (sc.item_scale > 0 && cand != sc.item_scale) continue;
+        RegLaunch t;
+        t.C = cand;
+        pimpc::reg_plan(batch, nx.data(), nu.data(), N.data(), precision, cand, &t.threads,
+                        &t.region, &t.nmax);
+        if (t.threads == 0) continue;
+        if (reg.threads > 0 && (int64_t)batch * cand > nsm) break;
+        reg = t;
+        if (t.threads <= target) break;
+      }
+    }
+    s->reg_plan = reg;
+    if (sc.family == 3 && e == cudaSuccess && reg.threads > 0) {
+      P.threads = reg.threads;
+      s->smem_admm = (size_t)4 * reg.region * ts;
+    } else if (sc.family == 3 && e == cudaSuccess) {
       // One CTA or a cluster per instance: the fewest CTAs whose shared memory holds a slice.
       const int thr = res_threads(precision);
       int plan[6];
@@ -731,6 +754,7 @@ int run_solve(pimpc_solver *s, const double *dx0, const double *dup, const doubl
     return fail(s, PIMPC_ESTATE, "temporal blocking (schedule 7) runs the plain iteration: accel must be 0");
   PIMPC_CHECK(s, s->tiled == 2 ? launch_tile(a, st)
                  : s->tiled == 3 ? launch_blk(a, s->prec, s->smem_admm, st)
+                 : s->sched.family == 3 && s->reg_plan.threads > 0 ? launch_reg(a, s->prec, s->reg_plan, st)
                  : s->sched.family == 3 ? launch_resident(a, s->prec, s->res_plan, s->smem_admm, st)
                  : s->sched.family == 4 ? launch_gemm(a, s->prec, s->gemm_plan, st)
                  : s->sched.family == 6 ? launch_tc(a, s->tc_mat, s->tc_off, s->smem_admm, st)

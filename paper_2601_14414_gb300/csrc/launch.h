@@ -87,6 +87,15 @@ size_t res_plan(int batch, const int *nx, const int *nu, const int *N, const int
 cudaError_t launch_resident(const AdmmLaunch &s, int precision, const int *plan, size_t smem,
                             cudaStream_t stream);
 
+// The same for n <= 16 with the stage data in registers: threads (0: does not fit) and vector
+// region of one CTA for C CTAs per instance.
+struct RegLaunch {
+  int C = 0, threads = 0, region = 0, nmax = 0;  // threads == 0: the shared-memory kernel runs
+};
+void reg_plan(int batch, const int *nx, const int *nu, const int *N, int precision, int C,
+              int *threads, int *region, int *nmax);
+cudaError_t launch_reg(const AdmmLaunch &s, int precision, const RegLaunch &rl, cudaStream_t stream);
+
 // Stage-invariant instances as dense contractions (register-tiled products over stage blocks).
 int gemm_threads();
 int gemm_plan(int max_n, int max_nx, int max_nu, int precision, size_t budget, int *plan);
