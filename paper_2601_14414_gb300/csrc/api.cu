@@ -127,6 +127,35 @@ cudaError_t lalloc(pimpc_solver *s, P **p, size_t bytes) {
 
 namespace pimpc {
 
+// The resident schedule in registers (n <= 16): CTAs per instance, 0 threads if it does not fit.
+// With item_scale = 0 one CTA as long as its threads stay within `one`: an exchange in a cluster
+// costs about what 200 more FP32 threads do (n 16, N 20: 1.36 us per iteration on one CTA of 320
+// threads, 1.60 on four), and four warps, one per scheduler, are what the FP64 pipe takes before
+// a warp's instructions queue (n 6, N 20: 3.23 us on one CTA, 3.48 on two; N 60: 7.98 and 3.54
+// on four). Else the smallest cluster whose CTAs stay within `few` threads, the cluster of 16
+// within `most`, and beyond that (FP64, whose iterations are long enough to pay for an exchange
+// through global memory, or instances that no cluster holds) the fewest CTAs within `grid`
+// (n 16, N 200, FP64: 7.09 us on a cluster of 16, 5.71 on 32 CTAs; N 100: 4.72 and 5.76). Batches
+// larger than the SMs take the fewest CTAs that hold an instance.
+static RegLaunch choose_reg(const Schedule &sc, int batch, const std::vector<int> &nx,
+                            const std::vector<int> &nu, const std::vector<int> &N, int precision,
+                            int nsm) {
+  const bool f32 = precision == PIMPC_F32;
+  const int one = f32 ? 320 : 128, few = f32 ? 160 : 128, most = f32 ? 1024 : 160, grid = f32 ? 512 : 160;
+  RegLaunch best;
+  for (int cand : {1, 2, 4, 8, 16, 24, 32, 48, 64, 80, 96}) {
+    if (sc.item_scale > 0 && cand != sc.item_scale) continue;
+    RegLaunch t;
+    t.C = cand;
+    reg_plan(batch, nx.data(), nu.data(), N.data(), precision, &t);
+    if (t.threads == 0) continue;
+    if ((best.threads > 0 || cand > 16) && (int64_t)batch * cand > nsm) break;
+    best = t;
+    if (t.threads <= (cand == 1 ? one : cand < 16 ? few : cand == 16 ? most : grid)) break;
+  }
+  return best;
+}
+
 // Lays out the stage blocks and iterates for a schedule, plans the solve kernel's launch and
 // work items, and (re)allocates the buffers that depend on them. The iterates restart from zero
 // and the factorisation is redone at the next solve.
@@ -493,28 +522,6 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
     e = admm_configure(precision, s->smem_admm, &bps);
     RegLaunch reg;
     if (sc.family == 3 && e == cudaSuccess) {
-      // Stage data in registers where every instance has n <= 16 and fits: with item_scale = 0
-      // the fewest CTAs whose lanes stay within a target while the whole batch fits the SMs
-      // (FP64: four warps, one per scheduler, because a fifth shares the FP64 pipe; FP32: eight),
-      // else the fewest that hold an instance.
-      const int target = precision == PIMPC_F32 ? 256 : 128;
-      for (int cand : {1, 2, 4, 8, 16}) {
-        if (sc.item_scale > 0 && cand != sc.item_scale) continue;
-        RegLaunch t;
-        t.C = cand;
-        pimpc::reg_plan(batch, nx.data(), nu.data(), N.data(), precision, cand, &t.threads,
-                        &t.region, &t.nmax);
-        if (t.threads == 0) continue;
-        if (reg.threads > 0 && (int64_t)batch * cand > nsm) break;
-        reg = t;
-        if (t.threads <= target) break;
-      }
-    }
-    s->reg_plan = reg;
-    if (sc.family == 3 && e == cudaSuccess && reg.threads > 0) {
-      P.threads = reg.threads;
-      s->smem_admm = (size_t)4 * reg.region * ts;
-    } else if (sc.family == 3 && e == cudaSuccess) {
       // One CTA or a cluster per instance: the fewest CTAs whose shared memory holds a slice.
       const int thr = res_threads(precision);
       int plan[6];
@@ -549,7 +556,14 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
       std::copy(plan, plan + 6, s->res_plan);
       P.threads = thr;
       s->smem_admm = bytes;
+      // what the shared-memory kernel accepts, in registers where n <= 16 allows it
+      reg = choose_reg(sc, batch, nx, nu, N, precision, nsm);
+      if (reg.threads > 0) {
+        P.threads = reg.threads;
+        s->smem_admm = (size_t)4 * reg.region * ts;
+      }
     }
+    s->reg_plan = reg;
     if (e == cudaSuccess && bps >= 1) {
       const int64_t max_grid = (int64_t)bps * nsm;
       // Sub-chunks per item: enough items for about 4 per CTA, at most 16 sub-chunks per item.
@@ -639,6 +653,8 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
   chk(lalloc(s, &d_W, sizeof(int) * batch));
   chk(lalloc(s, &d_tw, sizeof(int) * batch));
   chk(lalloc(s, &d_grp, sizeof(int) * batch));
+  if (sc.family == 3 && s->reg_plan.xch_bytes > 0)
+    chk(lalloc(s, (char **)&s->reg_plan.xch, s->reg_plan.xch_bytes));
   s->tc_mat = nullptr;
   s->tc_off = nullptr;
   if (sc.family == 6) {

@@ -1,100 +1,104 @@
 // detsum.cuh -- sums of non-negative floating-point values across a warp in integer arithmetic
-// (internal). A double-precision add takes 64 cycles on this part (one warp, measured; a
-// five-step butterfly with its shuffles about 570), and the sum of c^{i+1} sits on the critical
-// path of every iteration of a single-instance solve. Here the lanes agree on the largest
-// exponent, shift their significands to it and add them as integers (redux.sync on 22-bit limbs):
-// no FP64 instruction, and a result that does not depend on the order of the lanes. What is cut
-// off by the shifts is at most 2^-55 of the largest value per summand, below the rounding of a
-// chain of double additions.
+// (internal). A double-precision add takes 64 cycles on this part (one warp, measured; a five-step
+// butterfly with its shuffles about 570), and the sum of c^{i+1} sits on the critical path of
+// every iteration of a single-instance solve. Here the lanes agree on the largest exponent, shift
+// their significands to it and add them as integers (redux.sync on limbs): no FP64 instruction,
+// and a result that does not depend on the order of the lanes. What the shifts cut off is below
+// 2^-56 of the largest value per summand, less than the rounding of a chain of double additions.
 #pragma once
 #include <cuda_runtime.h>
 
 namespace pimpc {
 namespace detsum {
 
-// A non-negative value as significand and exponent: v = sig 2^e up to a constant of the format.
-// Infinities and NaN carry e = kSpecial, with sig = 0 for infinity.
-constexpr int kSpecial = 1 << 20;
+constexpr int kSpecial = 1 << 20;   // exponent of infinity (sig 0) and NaN (sig 1)
+constexpr int kZero = -(1 << 20);   // exponent of zero
+constexpr int kBias = 1080;
 
-struct Term {
-  unsigned long long sig;  // 53 significant bits at most
+// A non-negative value sig 2^(e - kBias).
+struct Fx {
+  unsigned long long sig;
   int e;
 };
 
-__device__ __forceinline__ Term term(double v) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const int e = (int)(b >> 52) & 0x7ff;
-  const unsigned long long m = b & 0xfffffffffffffull;
-  Term t;
-  t.sig = e ? (e == 0x7ff ? (m ? 1ull : 0ull) : (m | (1ull << 52))) : m;
-  t.e = e == 0x7ff ? kSpecial : (e ? e : 1);
-  return t;
+__device__ __forceinline__ Fx special_sum(Fx t) {
+  return Fx{__any_sync(0xffffffffu, t.e == kSpecial && t.sig != 0) ? 1ull : 0ull, kSpecial};
 }
 
-// A float, in the scale of the doubles: its 24-bit significand moved up by 29 bits.
-__device__ __forceinline__ Term term(float v) {
-  const unsigned b = __float_as_uint(v);
-  const int e = (int)(b >> 23) & 0xff;
+// Sum over the warp of one float per lane (the same Fx in every lane).
+__device__ __forceinline__ Fx warp_sum(float v) {
+  const unsigned b = __float_as_uint(v) & 0x7fffffffu;
+  const int x = (int)(b >> 23);
   const unsigned m = b & 0x7fffffu;
-  Term t;
-  t.sig = e == 0xff ? (m ? 1ull : 0ull) : ((unsigned long long)(e ? (m | 0x800000u) : m) << 29);
-  t.e = e == 0xff ? kSpecial : (e ? e : 1) + 1023 - 127;
-  return t;
+  const int e = x == 0xff ? 1 << 10 : (x ? x : 1);
+  const int em = __reduce_max_sync(0xffffffffu, e);
+  if (em == 1 << 10) return special_sum(Fx{m ? 1ull : 0ull, x == 0xff ? kSpecial : 0});
+  const int sh = em - e;
+  const unsigned long long q =
+      sh < 64 ? ((unsigned long long)(x ? (m | 0x800000u) : m) << 27) >> sh : 0ull;
+  const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)q & 0x3ffffffu);
+  const unsigned l1 = __reduce_add_sync(0xffffffffu, (unsigned)(q >> 26));
+  // v = (24-bit m) 2^(x - 150), q = m 2^27
+  return Fx{(unsigned long long)l0 + ((unsigned long long)l1 << 26), em - 177 + kBias};
 }
 
-// The sum over the warp of every lane's cnt terms (cnt <= kMax <= 4, compile-time unrolled), the
-// same double in every lane.
-template <int kMax>
-__device__ __forceinline__ double warp_sum(const Term (&t)[kMax]) {
-  int e = t[0].e;
-#pragma unroll
-  for (int i = 1; i < kMax; ++i) e = max(e, t[i].e);
-  const int em = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
-  if (em == kSpecial) {
-    bool nan = false;
-#pragma unroll
-    for (int i = 0; i < kMax; ++i) nan |= t[i].e == kSpecial && t[i].sig != 0;
-    return __any_sync(0xffffffffu, nan) ? __longlong_as_double(0x7ff8000000000000ll)
-                                        : __longlong_as_double(0x7ff0000000000000ll);
+__device__ __forceinline__ Fx add_limbs(unsigned long long q, int e) {
+  const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)q & 0x3fffffu);
+  const unsigned l1 = __reduce_add_sync(0xffffffffu, (unsigned)(q >> 22) & 0x3fffffu);
+  const unsigned l2 = __reduce_add_sync(0xffffffffu, (unsigned)(q >> 44));
+  return Fx{(unsigned long long)l0 + ((unsigned long long)l1 << 22) + ((unsigned long long)l2 << 44),
+            e};
+}
+
+// Sum over the warp of one double per lane.
+__device__ __forceinline__ Fx warp_sum(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+  const int x = (int)(b >> 52);
+  const unsigned long long m = b & 0xfffffffffffffull;
+  const int e = x == 0x7ff ? 1 << 12 : (x ? x : 1);
+  const int em = __reduce_max_sync(0xffffffffu, e);
+  if (em == 1 << 12) return special_sum(Fx{m ? 1ull : 0ull, x == 0x7ff ? kSpecial : 0});
+  const int sh = em - e;
+  const unsigned long long q = sh < 64 ? ((x ? m | (1ull << 52) : m) << 5) >> sh : 0ull;
+  return add_limbs(q, em - 1080 + kBias);  // v = m 2^(x - 1075), q = m 2^5
+}
+
+// Sum over the warp of one Fx per lane ({0, kZero} where a lane has none).
+__device__ __forceinline__ Fx warp_sum(Fx t) {
+  if (t.e != kSpecial) {
+    if (t.sig == 0) {
+      t.e = kZero;
+    } else {
+      const int lz = __clzll((long long)t.sig);
+      t.sig <<= lz;
+      t.e -= lz;
+    }
   }
-  unsigned l0 = 0, l1 = 0, l2 = 0;
-#pragma unroll
-  for (int i = 0; i < kMax; ++i) {
-    const int sh = em - t[i].e;
-    const unsigned long long q = sh < 64 ? (t[i].sig << 3) >> sh : 0ull;
-    l0 += (unsigned)q & 0x3fffffu;
-    l1 += (unsigned)(q >> 22) & 0x3fffffu;
-    l2 += (unsigned)(q >> 44);
-  }
-  l0 = __reduce_add_sync(0xffffffffu, l0);
-  l1 = __reduce_add_sync(0xffffffffu, l1);
-  l2 = __reduce_add_sync(0xffffffffu, l2);
-  // 56-bit terms, at most 128 of them: the total fits 63 bits
-  const unsigned long long tot =
-      (unsigned long long)l0 + ((unsigned long long)l1 << 22) + ((unsigned long long)l2 << 44);
-  if (tot == 0) return 0.0;
+  const int em = __reduce_max_sync(0xffffffffu, t.e);
+  if (em == kSpecial) return special_sum(t);
+  const int sh = em - t.e;
+  return add_limbs(sh < 57 ? (t.sig >> 6) >> sh : 0ull, em + 6);
+}
+
+__device__ __forceinline__ double to_double(Fx t) {
+  if (t.e == kSpecial)
+    return __longlong_as_double(t.sig ? 0x7ff8000000000000ll : 0x7ff0000000000000ll);
+  if (t.sig == 0) return 0.0;
   // normalise to bit 63, round to nearest (ties away) at 53 bits
-  const int lz = __clzll((long long)tot);
-  const unsigned long long m = tot << lz;
-  const int ef = em - 3 + 11 - lz;  // biased exponent of the result
-  if (ef <= 0) {                    // below the normal range: truncate
+  const int lz = __clzll((long long)t.sig);
+  const unsigned long long m = t.sig << lz;
+  const int ef = t.e - kBias + 63 - lz + 1023;  // biased exponent
+  if (ef <= 0) {                                // below the normal range: truncate
     const int sh = 12 - ef;
     return __longlong_as_double((long long)(sh < 64 ? m >> sh : 0ull));
   }
   const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);  // may carry into the exponent
   const unsigned long long bits = ((unsigned long long)ef << 52) + (r - (1ull << 52));
-  if (bits >= 0x7ff0000000000000ull) return __longlong_as_double(0x7ff0000000000000ll);
-  return __longlong_as_double((long long)bits);
+  return __longlong_as_double((long long)(bits < 0x7ff0000000000000ull ? bits : 0x7ff0000000000000ull));
 }
 
-template <typename T>
-__device__ __forceinline__ double warp_sum1(T v) {
-  const Term t[1] = {term(v)};
-  return warp_sum<1>(t);
-}
-
-// a <= b for doubles that are non-negative or whose right side may be negative (eps < 0 never
-// holds); both not NaN. Integer comparison: the bit patterns of non-negative doubles are ordered.
+// a <= b for a >= 0 (not NaN) and any b but -0 and NaN: bit patterns of non-negative doubles are
+// ordered, and a negative b compares below all of them.
 __device__ __forceinline__ bool le_nonneg(double a, double b) {
   return __double_as_longlong(a) <= __double_as_longlong(b);
 }

@@ -91,9 +91,10 @@ cudaError_t launch_resident(const AdmmLaunch &s, int precision, const int *plan,
 // region of one CTA for C CTAs per instance.
 struct RegLaunch {
   int C = 0, threads = 0, region = 0, nmax = 0;  // threads == 0: the shared-memory kernel runs
+  size_t xch_bytes = 0;                          // C > 16: exchange records in global memory
+  void *xch = nullptr;
 };
-void reg_plan(int batch, const int *nx, const int *nu, const int *N, int precision, int C,
-              int *threads, int *region, int *nmax);
+void reg_plan(int batch, const int *nx, const int *nu, const int *N, int precision, RegLaunch *rl);
 cudaError_t launch_reg(const AdmmLaunch &s, int precision, const RegLaunch &rl, cudaStream_t stream);
 
 // Stage-invariant instances as dense contractions (register-tiled products over stage blocks).

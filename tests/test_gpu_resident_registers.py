@@ -67,6 +67,35 @@ def test_cstr_long_horizon_exchanges_in_two_stages():
     check([W.random_ltv(7200, 2, 1, 5000)], pimpc.F32, 16, 40, 1)
 
 
+@pytest.mark.parametrize("precision", [pimpc.F32, pimpc.F64])
+@pytest.mark.parametrize("accel", [0, 1])
+def test_more_than_a_cluster(precision, accel):
+    # FP64 instances too long for a cluster's four warps, and an FP32 one no cluster holds: CTAs
+    # of a cooperative launch exchange through global memory (24 to 96 CTAs, ragged last ones)
+    for nx, nu, N in ((12, 4, 200), (3, 2, 1009), (7, 5, 331)) if precision == pimpc.F64 else (
+            (3, 2, 3001),):
+        check([W.random_ltv(7400 + N, nx, nu, N)], precision, 0, 50, accel)
+    if precision == pimpc.F64:
+        check([W.random_ltv(7450 + j, 12, 4, 160 + j) for j in range(3)], precision, 0, 50, accel)
+
+
+@pytest.mark.parametrize("mode", [1, 2])
+def test_warm_start_of_long_instances(mode):
+    inst = W.random_ltv(7460, 6, 3, 400)
+    s = pimpc.Solver([inst], precision=pimpc.F64, eps=-1.0, max_iters=40, accel=1)
+    s.set_schedule(pimpc.FAMILY_RESIDENT)
+    s.solve()
+    warm = {k: v.copy() for k, v in s.iterates()[0].items()}
+    if mode == 2:
+        warm = {k: np.concatenate([v[1:], v[-1:]], axis=0) for k, v in warm.items()}
+    s.solve(warm_start=mode)
+    got = s.iterates()[0]
+    o = oracle.solve(inst, eps=-1.0, max_iters=40, accel=1, warm=warm)
+    for key in ("z", "v", "th", "be", "la"):
+        assert relerr(got[key], o[key]) <= 1e-10, key
+    s.close()
+
+
 def test_non_finite_dynamics_are_reported():
     inst = W.plain_lti(7300, 4, 2, 20)
     inst["x0"] = np.array([np.inf, 0.0, 0.0, 0.0])
