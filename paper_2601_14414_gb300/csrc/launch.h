@@ -4,7 +4,6 @@
 
 namespace pimpc {
 
-int factorise_smem_words(int max_nx, int max_n);
 cudaError_t launch_factorise(const Layout &L, const double *A, const double *B, const double *e,
                              const double *qd, const double *rdu, double rho, const int *binst,
                              const int64_t *bbase, int64_t nblocks, int max_nx, int max_n,
