@@ -1,611 +1,9 @@
-// admm_reg.cu -- the resident schedule (family 3) for instances with n <= 16: the stage matrices
-// and the iterates of an instance live in the registers of one CTA, or of a cluster of C CTAs.
-//
-// What bounds a resident solve is the latency of one iteration: a few hundred multiply-adds per
-// stage between synchronisations, the cross-CTA exchange, and the FP64 decision of steps 5-7.
-// Thread (slot, c) owns component c of one stage, so that a CTA's warps are full whatever n is,
-// and holds in registers its column of G_{k+1}, its rows of G_k, of H_k and of
-//   P_k = Bbar_k M_k Bbar_k^T   (du is only ever used as Bbar_k du_k = P_k (v - beta)),
-// so that an iteration loads only vectors from shared memory (broadcast 16-byte reads). The
-// lambda of Algorithm 1 needs no state of its own: steps 2-3 give
-//   v = (z + gamma) / 2 with gamma = Bbar du + beta - Abar xbar - ebar + lambda, hence
-//   beta' + lambda' = gamma + z - 2 v = 0,
-// and the hats are linear, so lambda = -beta throughout (the zero start included).
-// One iteration: hats, y and w | Abar^T y, h, P w | xbar = H h | Abar xbar, steps 2-4 | one
-// exchange. The slots of a CTA are its stages and the two neighbouring ones, whose x-update it
-// repeats, so that the CTAs of an instance meet once per iteration: each sends its share of c to
-// all and its boundary iterates to its neighbours, and every CTA sums the shares and takes the
-// decision of steps 5-7 by itself (identical inputs, a sum that has no order), in integer
-// arithmetic (detsum.cuh) off the 64-cycle FP64 pipe. Within a cluster the data go by st.async
-// into the others' shared memory and complete on their mbarriers (520-660 cycles per exchange,
-// measured; remote stores and a cluster barrier 890 and more); beyond 16 CTAs they go through
-// global memory as 16-byte records that carry their iteration number (1400-1600 cycles for up
-// to 96 CTAs; a barrier on an atomic counter takes 2500 before any data are read).
-// The launch also makes the starting iterates and the outputs: one kernel per solve.
-// FP64 is bound by its pipe (a warp issues one FP64 instruction per 64 cycles, an SM one per 19),
-// so the FP64 code counts instructions: one chain per dot product, with the sums around it folded
-// into its start; x / 3 as two operations; the clamp on bit patterns.
-// Per iteration, measured, against the shared-memory kernel of admm_res.cu (which keeps the
-// instances with n > 16): plain LTI n 6, N 20, FP64 7.9 -> 3.2 us; quadrotor n 16, N 200 FP32
-// 6.8 -> 1.8 us, FP64 18.6 -> 5.7 us; CSTR n 3, N 5000 FP32 22.8 -> 3.2 us, FP64 102 -> 5.9 us.
-#include <cooperative_groups.h>
-#include <algorithm>
-#include <math.h>
-
-#include "detsum.cuh"
-#include "lockstep.cuh"
-
-namespace cg = cooperative_groups;
+// admm_reg.cu -- planning of the register-resident schedule and its FP32 kernels (admm_reg.cuh).
+#include "admm_reg.cuh"
 
 namespace pimpc {
 
-namespace {
-
-template <typename T>
-using Args = ls::Args<T>;
-
-constexpr int kMaxN = 16;
-constexpr int kMaxC = 96;            // CTAs of one instance (grid scope)
-constexpr int kWaitPolls = 1 << 22;  // bounded waits: polls of a record in global memory ...
-constexpr long long kWaitCycles = 1ll << 31;  // ... and cycles at an mbarrier (about a second)
-
-// Who runs an instance: one CTA, a cluster of up to 16, or up to kMaxC CTAs of a cooperative
-// launch that exchange through global memory.
-enum { kCta = 0, kCluster = 1, kGrid = 2 };
-
-// Threads of one CTA by the register bound: 4 n-vectors of matrix rows per thread.
-__host__ __device__ constexpr int reg_max_threads(int tsize, int NM) {
-  return tsize == 4 ? (NM <= 4 ? 1024 : 512) : (NM <= 4 ? 512 : (NM <= 8 ? 512 : 256));
-}
-
-struct RegPlan {
-  int C;              // CTAs per instance
-  int region;         // elements of each of the four vector regions
-  ulonglong2 *xch;    // grid scope: the exchange records
-  double *u_out, *x_out;
-  int warm;
-};
-
-// Exchange records of one instance (grid scope): by parity, C shares, then per CTA two sides of
-// kHaloRecs halo records. Every record carries the iteration in its upper 32 bits and is written
-// and read as one 16-byte access, so a reader that sees the iteration sees the payload.
-constexpr int kHaloRecs = 3 * kMaxN;
-__host__ __device__ inline size_t xch_records(int C) { return (size_t)2 * C * (1 + 2 * kHaloRecs); }
-
-__host__ __device__ inline int reg_nv(int n, int tsize) {
-  const int w = tsize == 4 ? 4 : 2;
-  return (n + w - 1) / w * w;
-}
-
-// init + sum_j m[j] v[j] over j < cnt, v in shared memory (16-byte aligned, zero-padded to whole
-// vectors), m in registers with zeros beyond its length. FP64 runs one chain: a warp issues an
-// FP64 instruction every 64 cycles, which is also its latency, so a second chain gains nothing.
-template <int NM>
-__device__ __forceinline__ float dot(const float (&m)[NM], const float *v, int cnt, float init) {
-  float a0 = init, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
-#pragma unroll
-  for (int j = 0; j < NM; j += 4)
-    if (j < cnt) {
-      const float4 q = *reinterpret_cast<const float4 *>(v + j);
-      a0 = fmaf(m[j], q.x, a0);
-      a1 = fmaf(m[j + 1], q.y, a1);
-      a2 = fmaf(m[j + 2], q.z, a2);
-      a3 = fmaf(m[j + 3], q.w, a3);
-    }
-  return (a0 + a1) + (a2 + a3);
-}
-template <int NM>
-__device__ __forceinline__ double dot(const double (&m)[NM], const double *v, int cnt, double init) {
-  double a = init;
-#pragma unroll
-  for (int j = 0; j < NM; j += 2)
-    if (j < cnt) {
-      const double2 q = *reinterpret_cast<const double2 *>(v + j);
-      a = fma(m[j], q.x, a);
-      a = fma(m[j + 1], q.y, a);
-    }
-  return a;
-}
-
-// x / 3 to within a rounding of the correctly rounded quotient: 1/3 as the sum of its rounding
-// and the rounding of what is left (two operations instead of a division; infinities pass).
-__device__ __forceinline__ float third(float x) {
-  constexpr float hi = 1.0f / 3.0f;
-  constexpr float lo = (float)(1.0 / 3.0 - (double)hi);
-  return fmaf(x, hi, x * lo);
-}
-__device__ __forceinline__ double third(double x) {
-  constexpr double hi = 1.0 / 3.0;         // (1 - 2^-54) / 3
-  constexpr double lo = hi * 0x1p-54;      // 1/3 - hi = 2^-54 / 3
-  return fma(x, hi, x * lo);
-}
-
-// min(max(w, lo), hi), NaN passing through. FP64 by the order of the bit patterns: two FP64
-// comparisons would cost 128 cycles.
-__device__ __forceinline__ float clamp(float w, float lo, float hi) {
-  return w < lo ? lo : (w > hi ? hi : w);
-}
-__device__ __forceinline__ long long order_key(double v) {
-  const long long b = __double_as_longlong(v);
-  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
-}
-__device__ __forceinline__ double clamp(double w, double lo, double hi) {
-  const long long k = order_key(w);
-  const bool nan = (__double_as_longlong(w) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
-  const double z = k < order_key(lo) ? lo : (k > order_key(hi) ? hi : w);
-  return nan ? w : z;
-}
-
-template <typename T>
-__device__ __forceinline__ T sym_at(const T *Wp, int m, int r, int c) {
-  int d = c - r;
-  if (d < 0) d += m;
-  return (2 * d <= m) ? Wp[d * m + r] : Wp[(m - d) * m + c];
-}
-
-// ---- exchange primitives ---------------------------------------------------------------------
-
-__device__ __forceinline__ unsigned smem_addr(const void *p) {
-  return (unsigned)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ unsigned remote(unsigned addr, int rank) {
-  unsigned r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-// Store to a CTA of the cluster that counts its bytes on that CTA's mbarrier.
-__device__ __forceinline__ void push(unsigned dst, unsigned bar, float v) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(dst),
-               "r"(__float_as_uint(v)), "r"(bar)
-               : "memory");
-}
-__device__ __forceinline__ void push(unsigned dst, unsigned bar, double v) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(dst),
-               "l"(__double_as_longlong(v)), "r"(bar)
-               : "memory");
-}
-__device__ __forceinline__ void push(unsigned dst, unsigned bar, detsum::Fx v) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(
-                   dst),
-               "l"(v.sig), "l"((long long)v.e), "r"(bar)
-               : "memory");
-}
-__device__ __forceinline__ bool bar_wait(unsigned bar, unsigned parity) {
-  const long long t0 = clock64();
-  do {
-    unsigned ok;
-    asm volatile(
-        "{\n\t.reg .pred q;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  } while (clock64() - t0 < kWaitCycles);
-  return false;
-}
-// One 16-byte record, written and read in a single access.
-__device__ __forceinline__ void put_rec(ulonglong2 *p, unsigned long long a, unsigned long long b) {
-  asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\t"
-               "st.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
-               "l"(a), "l"(b)
-               : "memory");
-}
-__device__ __forceinline__ void get_rec(const ulonglong2 *p, unsigned long long &a,
-                                        unsigned long long &b) {
-  asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\t"
-               "mov.b128 {%0, %1}, t;\n\t}"
-               : "=l"(a), "=l"(b)
-               : "l"(p)
-               : "memory");
-}
-__device__ __forceinline__ unsigned long long with_tag(unsigned lo, unsigned tag) {
-  return (unsigned long long)lo | ((unsigned long long)tag << 32);
-}
-// Boundary values through global memory. FP32: one record of up to three values per component;
-// FP64: one record per value.
-__device__ __forceinline__ void put_halo(ulonglong2 *p, int n, int c, unsigned tag, float x, float y,
-                                         float w) {
-  put_rec(p + c, (unsigned long long)__float_as_uint(x) | ((unsigned long long)__float_as_uint(y) << 32),
-          with_tag(__float_as_uint(w), tag));
-}
-__device__ __forceinline__ void put_halo(ulonglong2 *p, int n, int c, unsigned tag, double x, double y,
-                                         double w) {
-  put_rec(p + c, (unsigned long long)__double_as_longlong(x), with_tag(0, tag));
-  put_rec(p + n + c, (unsigned long long)__double_as_longlong(y), with_tag(0, tag));
-  put_rec(p + 2 * n + c, (unsigned long long)__double_as_longlong(w), with_tag(0, tag));
-}
-__device__ __forceinline__ bool get_halo(const ulonglong2 *p, int n, int c, unsigned tag, float &x,
-                                         float &y, float &w) {
-  unsigned long long a, b;
-  for (int i = 0; i < kWaitPolls; ++i) {
-    get_rec(p + c, a, b);
-    if ((unsigned)(b >> 32) != tag) continue;
-    x = __uint_as_float((unsigned)a);
-    y = __uint_as_float((unsigned)(a >> 32));
-    w = __uint_as_float((unsigned)b);
-    return true;
-  }
-  return false;
-}
-__device__ __forceinline__ bool get_halo(const ulonglong2 *p, int n, int c, unsigned tag, double &x,
-                                         double &y, double &w) {
-  unsigned long long a[3], b[3];
-  for (int i = 0; i < kWaitPolls; ++i) {
-#pragma unroll
-    for (int q = 0; q < 3; ++q) get_rec(p + q * n + c, a[q], b[q]);
-    if ((unsigned)(b[0] >> 32) != tag || (unsigned)(b[1] >> 32) != tag || (unsigned)(b[2] >> 32) != tag)
-      continue;
-    x = __longlong_as_double((long long)a[0]);
-    y = __longlong_as_double((long long)a[1]);
-    w = __longlong_as_double((long long)a[2]);
-    return true;
-  }
-  return false;
-}
-
-// Data of the cluster and grid exchanges in shared memory.
-template <typename T>
-struct Shared {
-  ulonglong2 share[2][16];      // cluster: shares of c by parity (sig, e)
-  ulonglong2 warp[32];          // warp sums (sig, e)
-  T land[2][2][3][kMaxN];       // cluster: boundary iterates by parity and side
-  unsigned long long bar[2];    // cluster: mbarriers by parity
-  ulonglong2 total;             // grid: the sum (sig, e)
-  int fail;                     // a wait gave up
-};
-
-template <typename T, int NM, int SC, int kMinCtas>
-__global__ void __launch_bounds__(reg_max_threads((int)sizeof(T), NM), kMinCtas)
-    reg_kernel(Args<T> a, RegPlan pl) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ Shared<T> sh;
-  const int C = SC == kCta ? 1 : pl.C;
-  const int r = SC == kCta ? 0 : (int)(blockIdx.x % C);  // the rank in the cluster: C divides grid
-  const int j = blockIdx.x / C;
-  const int tid = threadIdx.x, nthreads = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  const int nw = nthreads >> 5;
-  const int nx = a.L.nx[j], nu = a.L.nu[j], N = a.L.N[j], n = nx + nu;
-  const int nv = reg_nv(n, (int)sizeof(T));
-  const int k0 = (int)((int64_t)r * N / C), k1 = (int)((int64_t)(r + 1) * N / C);
-  const int kb = k0 - (r > 0 ? 1 : 0);                       // stage of slot 0
-  const int ke = k1 + (k1 < N ? 1 : 0);                      // one past the last slot's stage
-  const int slot = tid / n, c = tid - slot * n, k = kb + slot;
-  const bool active = k < ke;
-  const bool owned = active && k >= k0 && k < k1;
-  const bool has_h = active && k < k1;                       // owned, or the stage before them
-  const bool more = k + 1 < N;
-  T *sW = reinterpret_cast<T *>(smem_raw), *sY = sW + pl.region, *sH = sY + pl.region,
-    *sX = sH + pl.region;                                    // sX: row q = xbar_{kb + q}
-  for (int i = tid; i < 4 * pl.region; i += nthreads) sW[i] = (T)0;
-  if (tid < 32) sh.warp[tid] = make_ulonglong2(0, (unsigned long long)(long long)detsum::kZero);
-  if (tid == 0) {
-    sh.fail = 0;
-    if (SC == kCluster) {
-      for (int p = 0; p < 2; ++p)
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&sh.bar[p])));
-      asm volatile("fence.mbarrier_init.release.cluster;");
-    }
-  }
-
-  // ---- the thread's rows and columns, once ----
-  T Gn[NM], Gr[NM], Hr[NM], Pr[NM];
-#pragma unroll
-  for (int q = 0; q < NM; ++q) Gn[q] = Gr[q] = Hr[q] = Pr[q] = (T)0;
-  T zc = 0, vc = 0, tc = 0, bc = 0, zp = 0, vp = 0, tp = 0, bp = 0;  // iterate, and the one before
-  T ee = 0, qref = 0, lo = 0, hi = 0;
-  const T rho = (T)a.rho;
-  const int n5p = ls::iter_stride_plain(n, (int)sizeof(T));
-  T *const gits = a.it[a.base[j]] + a.L.Ni[j];
-  if (active) {
-    const int lti = a.L.lti, W = a.L.W[j], ldg = odd_ld(n);
-    const int oE = nx * ldg, oH = oE + nx, oM = oH + wrapped_size(n);
-    const T *blk = a.blk + a.L.blk[j];
-    const T *Gk = blk + (lti ? 0 : (int64_t)k * W);
-    const T *Gk1 = lti ? blk : Gk + W;
-    const T *Hk = (lti ? blk + (more ? 0 : W) : Gk) + oH;
-    if (pl.warm != 0) {  // the previous solve's iterate, shifted by a stage for warm == 2
-      const T *git = gits + (int64_t)(pl.warm == 2 && more ? k + 1 : k) * n5p;
-      zc = git[c];
-      vc = git[n + c];
-      tc = git[2 * n + c];
-      bc = git[3 * n + c];
-    }
-    ee = c < nx ? Gk[oE + c] : (T)0;
-    lo = a.lo[a.L.off_n[j] + c];
-    hi = a.hi[a.L.off_n[j] + c];
-    if (a.ref) {
-      const T *ref = a.ref + (a.ref_per_stage ? a.L.Nn[j] + (int64_t)k * n : a.L.off_n[j]);
-      qref = a.qd[a.L.off_n[j] + c] * ref[c];
-    }
-    if (has_h) {
-#pragma unroll
-      for (int q = 0; q < NM; ++q) {
-        if (q < n) Hr[q] = sym_at(Hk, n, c, q);
-        if (q < nx && more) Gn[q] = Gk1[q * ldg + c];
-      }
-    }
-    if (owned) {
-#pragma unroll
-      for (int q = 0; q < NM; ++q)
-        if (q < n) Gr[q] = c < nx ? Gk[c * ldg + q] : (q == c ? (T)1 : (T)0);
-      // P row c: sum_i (sum_q Bbar[c][q] M[q][i]) Bbar[q'][i], Bbar = [B; I]
-      const T *M = Gk + oM;
-      for (int i = 0; i < nu; ++i) {
-        T t = (T)0;
-        if (c < nx) {
-          for (int q = 0; q < nu; ++q) t += Gk[c * ldg + nx + q] * sym_at(M, nu, q, i);
-        } else {
-          t = sym_at(M, nu, c - nx, i);
-        }
-#pragma unroll
-        for (int q = 0; q < NM; ++q)
-          if (q < n) Pr[q] += t * (q < nx ? Gk[q * ldg + nx + i] : (q - nx == i ? (T)1 : (T)0));
-      }
-    }
-  }
-  double cval = 0.0, cbest = INFINITY;
-  double etac = a.eta;  // eta times the last c (1 at the start), formed off the critical path
-  int itbest = 0, itfirst = -1, streak = 0, momentum = 0, status = kMaxIter, iters = 0;
-  T f = (T)0;
-  bool use_prev = false;
-  const double eps = a.eps;
-  const bool unit_rho = a.rho == 1.0, watch = a.stall_win > 0 || a.mask != nullptr;
-  ulonglong2 *xs = nullptr, *xh = nullptr;  // grid: this instance's share and halo records
-  if (SC == kGrid) {
-    xs = pl.xch + (size_t)j * xch_records(C);
-    xh = xs + 2 * C;
-  }
-  const unsigned my_bytes =
-      SC == kCluster ? (unsigned)(16 * C + (int)sizeof(T) * n * ((r > 0 ? 2 : 0) + (k1 < N ? 3 : 0))) : 0;
-  __syncthreads();
-  if (r == 0 && tid < n) sX[tid] = a.xb0[a.L.off_n[j] + tid];
-  if (SC == kCluster) cg::this_cluster().sync();  // every mbarrier is ready
-  else __syncthreads();
-
-  for (int it = 0; it < a.max_iters; ++it) {
-    const int par = it & 1;
-    const unsigned tag = (unsigned)it + 1;
-    if (SC == kCluster && tid == 0)
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&sh.bar[par])),
-                   "r"(my_bytes)
-                   : "memory");
-    // the momentum factor this iteration's decision would take, fetched ahead
-    double ctab;
-    asm volatile("ld.global.f64 %0, [%1];" : "=d"(ctab) : "l"(a.coef_tab + (a.accel ? streak : 0)));
-    const T fnext = (T)ctab;
-    // ---- hats, y, w ----
-    T zh = zc, vh = vc, th = tc, bh = bc;
-    if (use_prev) {
-      zh = zc + f * (zc - zp);
-      vh = vc + f * (vc - vp);
-      th = tc + f * (tc - tp);
-      bh = bc + f * (bc - bp);
-    }
-    const T be = bh + ee;  // ebar - lambda
-    if (active) {
-      sW[slot * nv + c] = vh - bh;
-      sY[slot * nv + c] = (zh - vh) - be;
-    }
-    __syncthreads();
-    if (SC != kCta && sh.fail) break;  // set before this barrier, if at all: uniform
-    // ---- Abar_{k+1}^T y_{k+1}, h_k; p = beta + P_k w_k ----
-    T p = (T)0;
-    if (has_h) {
-      const T *y = sY + (slot + 1) * nv;
-      T acc = zh - th;
-      if (more) {
-        if (c >= nx) acc += y[c];
-        acc = dot(Gn, y, nx, acc);
-      }
-      sH[slot * nv + c] = qref + rho * acc;
-    }
-    if (owned) p = dot(Pr, sW + slot * nv, n, bh);
-    __syncthreads();
-    // ---- xbar_{k+1} = H_k h_k ----
-    T xb = (T)0;
-    if (has_h) {
-      xb = dot(Hr, sH + slot * nv, n, (T)0);
-      sX[(slot + 1) * nv + c] = xb;
-    }
-    __syncthreads();
-    // ---- steps 2-4 ----
-    T cacc = (T)0;
-    T zn = (T)0, vn = (T)0, tn = (T)0, bn = (T)0;
-    if (owned) {
-      const T q = dot(Gr, sX + slot * nv, n, be);  // Abar xbar + ebar - lambda
-      const T s = xb + th;
-      const T w = third((T)2 * s + (p + q));
-      zn = clamp(w, lo, hi);
-      vn = (T)0.5 * (zn + (p - q));
-      tn = s - zn;
-      bn = p - vn;
-      if (SC == kCluster) {  // boundary iterates: the first stage to CTA r - 1, the last to r + 1
-        if (k == k0 && r > 0) {
-          const unsigned bar = remote(smem_addr(&sh.bar[par]), r - 1);
-          const unsigned d = remote(smem_addr(&sh.land[par][1][0][c]), r - 1);
-          push(d, bar, zn);
-          push(d + kMaxN * sizeof(T), bar, vn);
-          push(d + 2 * kMaxN * sizeof(T), bar, bn);
-        }
-        if (k == k1 - 1 && k1 < N) {
-          const unsigned bar = remote(smem_addr(&sh.bar[par]), r + 1);
-          const unsigned d = remote(smem_addr(&sh.land[par][0][0][c]), r + 1);
-          push(d, bar, zn);
-          push(d + kMaxN * sizeof(T), bar, tn);
-        }
-      }
-      if (SC == kGrid) {
-        if (k == k0 && r > 0)
-          put_halo(xh + ((size_t)(par * C + r - 1) * 2 + 1) * kHaloRecs, n, c, tag, zn, vn, bn);
-        if (k == k1 - 1 && k1 < N)
-          put_halo(xh + (size_t)(par * C + r + 1) * 2 * kHaloRecs, n, c, tag, zn, tn, (T)0);
-      }
-      const T d1 = tn - th, d2 = bn - bh, d4 = zn - zh, d5 = vn - vh;
-      // d1^2 + d2^2 + d3^2 + d4^2 + d5^2 + (d4 - d5)^2 with d3 = -d2
-      const T g = d2 * d2 + (d4 * d4 + d5 * (d5 - d4));
-      cacc = (T)2 * g + d1 * d1;
-    }
-    // ---- the exchange: shares of c and boundary iterates ----
-    detsum::Fx sum = detsum::warp_sum(cacc);
-    if (nw > 1) {
-      if (lane == 0) sh.warp[warp] = make_ulonglong2(sum.sig, (unsigned long long)(long long)sum.e);
-      __syncthreads();
-      if (SC == kCta || warp == 0) {
-        const ulonglong2 t = sh.warp[lane];  // {0, kZero} beyond the CTA's warps
-        sum = detsum::warp_sum(detsum::Fx{t.x, (int)t.y});
-      }
-    }
-    if (SC == kCluster) {
-      if (warp == 0 && lane < C)
-        push(remote(smem_addr(&sh.share[par][r]), lane), remote(smem_addr(&sh.bar[par]), lane), sum);
-      if (!bar_wait(smem_addr(&sh.bar[par]), (unsigned)(it >> 1) & 1u)) sh.fail = 1;
-      detsum::Fx t{0ull, detsum::kZero};
-      if (lane < C) {
-        const ulonglong2 q = sh.share[par][lane];
-        t = detsum::Fx{q.x, (int)q.y};
-      }
-      sum = detsum::warp_sum(t);
-    }
-    if (SC == kGrid) {
-      if (warp == 0) {
-        if (lane == 0) put_rec(xs + par * C + r, sum.sig, with_tag((unsigned)sum.e, tag));
-        detsum::Fx t[3];  // C <= 96 shares, three per lane, all in flight
-        bool ok = false;
-        for (int n_ = 0; n_ < kWaitPolls && !ok; ++n_) {
-          bool mine = true;
-#pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            unsigned long long b = with_tag((unsigned)detsum::kZero, tag);
-            t[q].sig = 0;
-            if (lane + 32 * q < C) get_rec(xs + par * C + lane + 32 * q, t[q].sig, b);
-            t[q].e = (int)(unsigned)b;
-            mine = mine && (unsigned)(b >> 32) == tag;
-          }
-          ok = __all_sync(0xffffffffu, mine);
-        }
-        if (!ok && lane == 0) sh.fail = 1;
-        sum = detsum::warp_sum(t[0]);
-        if (C > 32) {
-          const detsum::Fx s1 = detsum::warp_sum(t[1]), s2 = detsum::warp_sum(t[2]);
-          sum = detsum::warp_sum(lane == 0 ? sum : lane == 1 ? s1 : lane == 2 ? s2
-                                                                  : detsum::Fx{0ull, detsum::kZero});
-        }
-        if (lane == 0) sh.total = make_ulonglong2(sum.sig, (unsigned long long)(long long)sum.e);
-      }
-      if (active && !owned) {  // boundary iterates of the neighbours
-        T x, y, w;
-        const bool before = k < k0;
-        if (!get_halo(xh + ((size_t)(par * C + r) * 2 + (before ? 0 : 1)) * kHaloRecs, n, c, tag, x, y, w))
-          sh.fail = 1;
-        zn = x;
-        if (before) {
-          tn = y;
-        } else {
-          vn = y;
-          bn = w;
-        }
-      }
-      __syncthreads();
-      const ulonglong2 q = sh.total;
-      sum = detsum::Fx{q.x, (int)q.y};
-    }
-    // ---- steps 5-7, by every thread alike ----
-    double cn = detsum::to_double(sum);
-    if (!unit_rho) cn *= a.rho;
-    cval = cn;
-    iters = it + 1;
-    bool stop = false, take;
-    if (detsum::le_nonneg(cn, eps) || !detsum::finite(cn) || it + 1 >= a.max_iters || watch) {
-      take = false;
-      if (!detsum::finite(cn)) {
-        status = kNonFinite; stop = true;
-      } else if (detsum::le_nonneg(cn, eps)) {
-        status = kConverged; stop = true;
-      } else if (a.stall_win > 0 && cn <= a.stall_below && !(cn < a.stall_fac * cbest) &&
-                 (double)(it - itbest) >=
-                     fmax((double)a.stall_win, a.stall_rel * (double)(itfirst < 0 ? it : itfirst))) {
-        status = kStalled; stop = true;
-      } else if (it + 1 >= a.max_iters) {
-        status = kMaxIter; stop = true;
-      } else if (a.accel) {
-        if (a.mask && it < a.mask_len) take = a.mask[(int64_t)j * a.mask_len + it] != 0;
-        else take = detsum::le_nonneg(cn, etac);
-      }
-      if (a.stall_win > 0 && cn <= a.stall_below) {
-        if (itfirst < 0) itfirst = it;
-        if (cn < a.stall_fac * cbest) {
-          cbest = cn;
-          itbest = it;
-        }
-      }
-    } else {
-      take = a.accel && detsum::le_nonneg(cn, etac);
-    }
-    // (alpha_m - 1) / alpha_{m+1}, alpha_0 = 1, from the precomputed table; 0 after a restart
-    use_prev = take && streak > 0;
-    momentum += use_prev;
-    f = take ? fnext : (T)0;
-    streak = take ? streak + 1 : 0;
-    etac = a.eta * cn;
-    // ---- the new iterate becomes the current one; halo slots take theirs from the landing ----
-    if (SC == kCluster && active && !owned) {
-      const T *d = &sh.land[par][k < k0 ? 0 : 1][0][c];
-      zn = d[0];
-      if (k < k0) {
-        tn = d[kMaxN];
-      } else {
-        vn = d[kMaxN];
-        bn = d[2 * kMaxN];
-      }
-    }
-    zp = zc; vp = vc; tp = tc; bp = bc;
-    zc = zn; vc = vn; tc = tn; bc = bn;
-    if (stop) break;
-  }
-  if (SC != kCta) {
-    __syncthreads();
-    if (sh.fail) status = kTimeout;
-  }
-  if (owned) {
-    T *git = gits + (int64_t)k * n5p;
-    git[c] = zc;
-    git[n + c] = vc;
-    git[2 * n + c] = tc;
-    git[3 * n + c] = bc;
-    git[4 * n + c] = -bc;
-    if (c < nx) {
-      if (pl.x_out) pl.x_out[a.L.Nnx[j] + (int64_t)k * nx + c] = (double)zc;
-    } else if (pl.u_out) {
-      pl.u_out[a.L.Nnu[j] + (int64_t)k * nu + (c - nx)] = (double)zc;
-    }
-  }
-  if (r == 0 && tid == 0) {
-    InstState s;
-    s.iters = iters;
-    s.status = a.ferr && a.ferr[j] ? kFactorFailed : status;
-    s.momentum = momentum;
-    s.pad = 0;
-    s.c = cval;
-    a.st[j] = s;
-    a.stop[j] = 1;
-  }
-  if (SC == kCluster) cg::this_cluster().sync();  // no CTA leaves with a push to it in flight
-}
-
-template <typename T, int SC>
-const void *pick_kernel(int NM, bool crowded) {
-  if constexpr (sizeof(T) == 4 && SC == kCta)
-    if (crowded && NM == 8) return (const void *)reg_kernel<T, 8, SC, 2>;
-  return NM == 4   ? (const void *)reg_kernel<T, 4, SC, 1>
-         : NM == 8 ? (const void *)reg_kernel<T, 8, SC, 1>
-                   : (const void *)reg_kernel<T, 16, SC, 1>;
-}
-
-int reg_class(int n) { return n <= 4 ? 4 : (n <= 8 ? 8 : 16); }
-
-}  // namespace
+cudaError_t launch_reg64(const AdmmLaunch &s, const RegLaunch &rl, cudaStream_t stream);
 
 // Threads and shared memory of one CTA for C CTAs per instance; 0 threads: the batch does not fit
 // (an n above 16, fewer stages than CTAs, or more stages per CTA than its threads hold).
@@ -630,64 +28,69 @@ void reg_plan(int batch, const int *nx, const int *nu, const int *N, int precisi
   rl->xch_bytes = C > 16 ? sizeof(ulonglong2) * xch_records(C) * (size_t)batch : 0;
 }
 
-template <typename T>
-static cudaError_t reg_launch_t(const AdmmLaunch &s, const RegLaunch &rl, cudaStream_t stream) {
-  Args<T> a = ls::make_args<T>(s);
-  a.eps = s.eps + 0.0;  // -0 becomes +0: the stop test compares bit patterns
-  cudaError_t rc;
-  if (s.max_iters <= 0) {  // nothing to iterate: the starting iterates are the result
-    rc = cudaMemcpyAsync(s.old_base, s.base, sizeof(int) * s.L.batch, cudaMemcpyDeviceToDevice, stream);
-    if (rc != cudaSuccess) return rc;
-    const int n_init = s.L.batch > s.nitems ? s.L.batch : s.nitems;
-    ls::solve_init_kernel<T><<<(n_init + 255) / 256, 256, 0, stream>>>(a, s.warm);
-    if ((rc = cudaGetLastError()) != cudaSuccess) return rc;
-    if (s.warm != 1) {
-      ls::prepare_kernel<T><<<dim3(8, s.L.batch), 256, 0, stream>>>(a, s.warm, s.old_base);
-      if ((rc = cudaGetLastError()) != cudaSuccess) return rc;
-    }
-    ls::output_kernel<T><<<dim3(4, s.L.batch), 256, 0, stream>>>(a, s.u_out, s.x_out);
-    return cudaGetLastError();
+// The resident schedule in registers (n <= 16): CTAs per instance, 0 threads if it does not fit.
+// With item_scale = 0 one CTA as long as its threads stay within `one`: an exchange in a cluster
+// costs about what 200 more FP32 threads do (n 16, N 20: 1.36 us per iteration on one CTA of 320
+// threads, 1.60 on four), and four warps, one per scheduler, are what the FP64 pipe takes before
+// a warp's instructions queue (n 6, N 20: 3.23 us on one CTA, 3.48 on two; N 60: 7.98 and 3.54
+// on four). Else the smallest cluster whose CTAs stay within `few` threads, the cluster of 16
+// within `most`, and beyond that (FP64, whose iterations are long enough to pay for an exchange
+// through global memory, or instances that no cluster holds) the fewest CTAs within `grid`
+// (n 16, N 200, FP64: 7.09 us on a cluster of 16, 5.71 on 32 CTAs; N 100: 4.72 and 5.76). Batches
+// larger than the SMs take the fewest CTAs that hold an instance.
+static RegLaunch choose_reg(int item_scale, int batch, const int *nx, const int *nu, const int *N,
+                            int precision, int nsm) {
+  const bool f32 = precision == 0;
+  const int one = f32 ? 320 : 128, few = f32 ? 160 : 128, most = f32 ? 1024 : 160, grid = f32 ? 512 : 160;
+  RegLaunch best;
+  for (int cand : {1, 2, 4, 8, 16, 24, 32, 48, 64, 80, 96}) {
+    if (item_scale > 0 && cand != item_scale) continue;
+    RegLaunch t;
+    t.C = cand;
+    reg_plan(batch, nx, nu, N, precision, &t);
+    if (t.threads == 0) continue;
+    if ((best.threads > 0 || cand > 16) && (int64_t)batch * cand > nsm) break;
+    best = t;
+    if (t.threads <= (cand == 1 ? one : cand < 16 ? few : cand == 16 ? most : grid)) break;
   }
-  int dev = 0, nsm = 0;
-  if ((rc = cudaGetDevice(&dev)) != cudaSuccess) return rc;
-  if ((rc = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return rc;
-  const int cls = reg_class(rl.nmax);
-  const void *kernel = rl.C == 1    ? pick_kernel<T, kCta>(cls, (int64_t)s.L.batch > nsm)
-                       : rl.C <= 16 ? pick_kernel<T, kCluster>(cls, false)
-                                    : pick_kernel<T, kGrid>(cls, false);
-  const size_t smem = (size_t)4 * rl.region * sizeof(T);
-  rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (rc != cudaSuccess) return rc;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(s.L.batch * rl.C);
-  cfg.blockDim = dim3(rl.threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  cfg.attrs = attr;
-  cfg.numAttrs = rl.C > 1 ? 1 : 0;
-  if (rl.C > 16) {  // all CTAs resident at once; records of an earlier solve are cleared
-    rc = cudaMemsetAsync(rl.xch, 0, rl.xch_bytes, stream);
-    if (rc != cudaSuccess) return rc;
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-  } else if (rl.C > 1) {
-    if (rl.C > 8) {
-      rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (rc != cudaSuccess) return rc;
+  return best;
+}
+
+// Plans the resident schedule (family 3): the shared-memory kernel's cluster size, regions and
+// bytes per CTA, and the register kernel's launch where every instance has n <= 16. False if the
+// instances do not fit the shared memory of a cluster (of item_scale CTAs, if that is not 0), or
+// one has fewer stages than its CTAs.
+// With item_scale = 0: the fewest CTAs that fit, or, when the whole batch occupies few SMs (latency,
+// not throughput, is what a small batch needs), the most CTAs (up to 16) that still give every
+// CTA four stages or more.
+bool plan_resident(int item_scale, int batch, const int *nx, const int *nu, const int *N,
+                   const int *W, int lti, int precision, int nsm, size_t optin, int *res,
+                   size_t *smem, RegLaunch *reg) {
+  const int thr = res_threads(precision), ts = precision == 0 ? 4 : 8;
+  const int nmin = *std::min_element(N, N + batch);
+  int fewest = 0, most = 0, plan[6], p_few[6], p_most[6];
+  size_t b_few = 0, b_most = 0;
+  for (int cand : {1, 2, 4, 8, 16}) {
+    if (item_scale > 0 && cand != item_scale) continue;
+    const size_t b = res_plan(batch, nx, nu, N, W, lti, precision, thr, cand, plan);
+    if (b == 0 || b + 1024 > optin - 256) continue;
+    if (fewest == 0) { fewest = cand; b_few = b; std::copy(plan, plan + 6, p_few); }
+    if (item_scale > 0 || (nmin >= 4 * cand && (int64_t)batch * cand <= nsm)) {
+      most = cand; b_most = b; std::copy(plan, plan + 6, p_most);
     }
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = rl.C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
   }
-  RegPlan pl{rl.C, rl.region, (ulonglong2 *)rl.xch, s.u_out, s.x_out, s.warm};
-  void *params[] = {&a, &pl};
-  return cudaLaunchKernelExC(&cfg, kernel, params);
+  if (fewest == 0) return false;
+  const bool wide = most >= fewest;
+  std::copy(wide ? p_most : p_few, (wide ? p_most : p_few) + 6, res);
+  *smem = wide ? b_most : b_few;
+  // what the shared-memory kernel accepts, in registers where n <= 16 allows it
+  *reg = choose_reg(item_scale, batch, nx, nu, N, precision, nsm);
+  if (reg->threads > 0) *smem = (size_t)4 * reg->region * ts;
+  return true;
 }
 
 cudaError_t launch_reg(const AdmmLaunch &s, int precision, const RegLaunch &rl, cudaStream_t stream) {
-  return precision == 0 ? reg_launch_t<float>(s, rl, stream) : reg_launch_t<double>(s, rl, stream);
+  return precision == 0 ? reg_launch_t<float>(s, rl, stream) : launch_reg64(s, rl, stream);
 }
 
 }  // namespace pimpc

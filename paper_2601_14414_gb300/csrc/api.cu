@@ -127,35 +127,6 @@ cudaError_t lalloc(pimpc_solver *s, P **p, size_t bytes) {
 
 namespace pimpc {
 
-// The resident schedule in registers (n <= 16): CTAs per instance, 0 threads if it does not fit.
-// With item_scale = 0 one CTA as long as its threads stay within `one`: an exchange in a cluster
-// costs about what 200 more FP32 threads do (n 16, N 20: 1.36 us per iteration on one CTA of 320
-// threads, 1.60 on four), and four warps, one per scheduler, are what the FP64 pipe takes before
-// a warp's instructions queue (n 6, N 20: 3.23 us on one CTA, 3.48 on two; N 60: 7.98 and 3.54
-// on four). Else the smallest cluster whose CTAs stay within `few` threads, the cluster of 16
-// within `most`, and beyond that (FP64, whose iterations are long enough to pay for an exchange
-// through global memory, or instances that no cluster holds) the fewest CTAs within `grid`
-// (n 16, N 200, FP64: 7.09 us on a cluster of 16, 5.71 on 32 CTAs; N 100: 4.72 and 5.76). Batches
-// larger than the SMs take the fewest CTAs that hold an instance.
-static RegLaunch choose_reg(const Schedule &sc, int batch, const std::vector<int> &nx,
-                            const std::vector<int> &nu, const std::vector<int> &N, int precision,
-                            int nsm) {
-  const bool f32 = precision == PIMPC_F32;
-  const int one = f32 ? 320 : 128, few = f32 ? 160 : 128, most = f32 ? 1024 : 160, grid = f32 ? 512 : 160;
-  RegLaunch best;
-  for (int cand : {1, 2, 4, 8, 16, 24, 32, 48, 64, 80, 96}) {
-    if (sc.item_scale > 0 && cand != sc.item_scale) continue;
-    RegLaunch t;
-    t.C = cand;
-    reg_plan(batch, nx.data(), nu.data(), N.data(), precision, &t);
-    if (t.threads == 0) continue;
-    if ((best.threads > 0 || cand > 16) && (int64_t)batch * cand > nsm) break;
-    best = t;
-    if (t.threads <= (cand == 1 ? one : cand < 16 ? few : cand == 16 ? most : grid)) break;
-  }
-  return best;
-}
-
 // Lays out the stage blocks and iterates for a schedule, plans the solve kernel's launch and
 // work items, and (re)allocates the buffers that depend on them. The iterates restart from zero
 // and the factorisation is redone at the next solve.
@@ -522,46 +493,12 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
     e = admm_configure(precision, s->smem_admm, &bps);
     RegLaunch reg;
     if (sc.family == 3 && e == cudaSuccess) {
-      // One CTA or a cluster per instance: the fewest CTAs whose shared memory holds a slice.
-      const int thr = res_threads(precision);
-      int plan[6];
-      size_t bytes = 0;
-      int C = 0;
-      // With item_scale = 0: the fewest CTAs that fit, or, when the whole batch occupies few
-      // SMs (latency, not throughput, is what a small batch needs), the most CTAs (up to 16)
-      // that still give every CTA four stages or more.
-      const int nmin = *std::min_element(N.begin(), N.end());
-      int fewest = 0, most = 0;
-      size_t b_few = 0, b_most = 0;
-      int p_few[6], p_most[6];
-      for (int cand : {1, 2, 4, 8, 16}) {
-        if (sc.item_scale > 0 && cand != sc.item_scale) continue;
-        const size_t b = res_plan(batch, nx.data(), nu.data(), N.data(), W.data(), lti, precision,
-                                  thr, cand, plan);
-        if (b == 0 || b + 1024 > (size_t)optin - 256) continue;
-        if (fewest == 0) { fewest = cand; b_few = b; std::copy(plan, plan + 6, p_few); }
-        if (sc.item_scale > 0 || (nmin >= 4 * cand && (int64_t)batch * cand <= nsm)) {
-          most = cand; b_most = b; std::copy(plan, plan + 6, p_most);
-        }
-      }
-      if (most > 0 && most >= fewest) {
-        C = most; bytes = b_most; std::copy(p_most, p_most + 6, plan);
-      } else if (fewest > 0) {
-        C = fewest; bytes = b_few; std::copy(p_few, p_few + 6, plan);
-      }
-      if (C == 0) {
+      if (!plan_resident(sc.item_scale, batch, nx.data(), nu.data(), N.data(), W.data(), lti,
+                         precision, nsm, (size_t)optin, s->res_plan, &s->smem_admm, &reg)) {
         why = "the instances do not fit the shared memory of a cluster of that size (or N < cluster size)";
         return PIMPC_EINVAL;
       }
-      std::copy(plan, plan + 6, s->res_plan);
-      P.threads = thr;
-      s->smem_admm = bytes;
-      // what the shared-memory kernel accepts, in registers where n <= 16 allows it
-      reg = choose_reg(sc, batch, nx, nu, N, precision, nsm);
-      if (reg.threads > 0) {
-        P.threads = reg.threads;
-        s->smem_admm = (size_t)4 * reg.region * ts;
-      }
+      P.threads = reg.threads > 0 ? reg.threads : res_threads(precision);
     }
     s->reg_plan = reg;
     if (e == cudaSuccess && bps >= 1) {

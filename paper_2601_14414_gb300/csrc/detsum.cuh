@@ -107,5 +107,15 @@ __device__ __forceinline__ bool finite(double v) {
   return ((unsigned)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u;
 }
 
+__device__ __forceinline__ bool finite(float v) {
+  return (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u;
+}
+
+// Whether a sum of v with others may leave the finite range (NaN and infinity included).
+__device__ __forceinline__ bool may_overflow(double v) {
+  return ((unsigned)__double2hiint(v) & 0x7ff00000u) >= (2047u - 16u) << 20;
+}
+__device__ __forceinline__ bool may_overflow(float v) { return !finite(v); }
+
 }  // namespace detsum
 }  // namespace pimpc

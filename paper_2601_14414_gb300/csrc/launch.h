@@ -94,6 +94,9 @@ struct RegLaunch {
   void *xch = nullptr;
 };
 void reg_plan(int batch, const int *nx, const int *nu, const int *N, int precision, RegLaunch *rl);
+bool plan_resident(int item_scale, int batch, const int *nx, const int *nu, const int *N,
+                   const int *W, int lti, int precision, int nsm, size_t optin, int *res,
+                   size_t *smem, RegLaunch *reg);
 cudaError_t launch_reg(const AdmmLaunch &s, int precision, const RegLaunch &rl, cudaStream_t stream);
 
 // Stage-invariant instances as dense contractions (register-tiled products over stage blocks).
