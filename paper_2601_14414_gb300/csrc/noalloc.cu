@@ -15,12 +15,18 @@
 // cudaGetSymbolAddress (once per device); make that first call before any stream capture.
 //
 // The arithmetic is that of pimpc_solve: the same factorisation, solve and output kernels run
-// on the same memory layout, with their buffers carved out of the static array.
+// on the same memory layout, with their buffers carved out of the static array. An instance that
+// the resident schedule holds (registers or shared memory of one CTA, a cluster or a few dozen
+// CTAs; see plan_resident) runs on it: one instance leaves the lock-step frame waiting on its grid
+// barrier (n 16, N 200, 100 FP32 iterations: 8.6 ms there, 0.2 ms resident). Its momentum factors
+// come from a constant table, filled once per device together with the array's address; longer
+// runs, and instances too long for a cluster, use one thread per stage on tiles.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <mutex>
 #include <string>
+#include <vector>
 
 #include "launch.h"
 #include "pimpc.h"
@@ -38,12 +44,20 @@ namespace {
 constexpr size_t kStaticBytes = (size_t)16 << 20;  // 16 MiB, documented in include/pimpc.h
 __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
+// Momentum factors (alpha_m - 1) / alpha_{m+1} of Algorithm 1 step 6 after m consecutive momentum
+// steps, alpha_0 = 1, alpha_{m+1} = (1 + sqrt(1 + 4 alpha_m^2)) / 2, rounded as the device rounds
+// them (multiply-adds fused).
+constexpr int kCoefs = 4096;
+__device__ double g_coef_table[kCoefs];
+
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void *g_scratch_ptr[kMaxDevices] = {};
+double *g_coef_ptr[kMaxDevices] = {};
 
-// Device address of the static array on the current device (looked up once per device).
-cudaError_t scratch_address(void **out) {
+// Device addresses of the static array and of the momentum table on the current device (looked
+// up, and the table filled, once per device).
+cudaError_t scratch_address(void **out, const double **coefs) {
   int dev = 0;
   cudaError_t rc = cudaGetDevice(&dev);
   if (rc != cudaSuccess) return rc;
@@ -53,9 +67,23 @@ cudaError_t scratch_address(void **out) {
     void *p = nullptr;
     rc = cudaGetSymbolAddress(&p, g_static_scratch);
     if (rc != cudaSuccess) return rc;
+    void *t = nullptr;
+    rc = cudaGetSymbolAddress(&t, g_coef_table);
+    if (rc != cudaSuccess) return rc;
+    std::vector<double> tab(kCoefs);
+    double al = 1.0;
+    for (int m = 0; m < kCoefs; ++m) {
+      const double an = std::fma(0.5, std::sqrt(std::fma(4.0 * al, al, 1.0)), 0.5);
+      tab[m] = (al - 1.0) / an;
+      al = an;
+    }
+    rc = cudaMemcpy(t, tab.data(), sizeof(double) * kCoefs, cudaMemcpyHostToDevice);
+    if (rc != cudaSuccess) return rc;
+    g_coef_ptr[dev] = (double *)t;
     g_scratch_ptr[dev] = p;
   }
   *out = g_scratch_ptr[dev];
+  *coefs = g_coef_ptr[dev];
   return cudaSuccess;
 }
 
@@ -83,8 +111,8 @@ struct Views {
 };
 
 // Fills the single-instance layout and work list (all offsets 0, one instance).
-__global__ void static_setup_kernel(Views v, int nx, int nu, int N, int W, int64_t Ni_total,
-                                    int item_stages, int nitems) {
+__global__ void static_setup_kernel(Views v, int nx, int nu, int N, int W, int item_stages,
+                                    int nitems) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t == 0) {
     v.nx[0] = nx;
@@ -95,7 +123,6 @@ __global__ void static_setup_kernel(Views v, int nx, int nu, int N, int W, int64
     v.base[0] = 0;
     v.nitems_inst[0] = nitems;
     v.ferr[0] = 0;
-    (void)Ni_total;
   }
   for (int k = t; k < N; k += gridDim.x * blockDim.x) v.binst[k] = 0;
   for (int i = t; i < nitems; i += gridDim.x * blockDim.x) {
@@ -137,50 +164,83 @@ extern "C" int pimpc_solve_static(int nx, int nu, int N, int precision, const do
     return fail_static(PIMPC_EINVAL, "pimpc_solve_static: eta must be finite and >= 0");
   cudaStream_t st = (cudaStream_t)stream;
   const size_t ts = precision == PIMPC_F32 ? 4 : 8;
-  const int64_t ntiles = (N + 31) / 32;
-  const int W = nx * n + nx + n * (n + 1) / 2 + nu * (nu + 1) / 2;
-  const int64_t blk_elems = (ntiles * 32 * W + 31) / 32 * 32;
-  const int64_t it_elems = ntiles * 32 * 5 * n;
   const int S = tps_stages_per_subchunk();
   const int item_stages = S;
   const int nitems = (N + item_stages - 1) / item_stages;
 
   void *raw = nullptr;
-  cudaError_t rc = scratch_address(&raw);
+  const double *coefs = nullptr;
+  cudaError_t rc = scratch_address(&raw, &coefs);
   if (rc != cudaSuccess)
-    return fail_static(PIMPC_ECUDA, std::string("pimpc_solve_static: cudaGetSymbolAddress: ") +
+    return fail_static(PIMPC_ECUDA, std::string("pimpc_solve_static: static array: ") +
                                         cudaGetErrorString(rc));
-  Carver cv{(unsigned char *)raw};
+  int nsm = 0, dev = 0, optin = 0;
+  if ((rc = cudaGetDevice(&dev)) != cudaSuccess ||
+      (rc = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+      (rc = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
+    return fail_static(PIMPC_ECUDA, std::string("pimpc_solve_static: device: ") + cudaGetErrorString(rc));
   Views v;
-  v.nx = cv.take<int>(1); v.nu = cv.take<int>(1); v.N = cv.take<int>(1); v.W = cv.take<int>(1);
-  for (int i = 0; i < 13; ++i) v.off[i] = cv.take<int64_t>(1);
-  v.binst = cv.take<int>(N);
-  v.item_inst = cv.take<int>(nitems); v.item_a = cv.take<int>(nitems); v.item_b = cv.take<int>(nitems);
-  v.nitems_inst = cv.take<int>(1);
-  v.list0 = cv.take<int>(nitems); v.list1 = cv.take<int>(nitems);
-  v.base = cv.take<int>(1); v.old_base = cv.take<int>(1); v.ndone = cv.take<int>(1);
-  v.stop = cv.take<int>(1); v.ferr = cv.take<int>(1);
-  v.alpha = cv.take<double>(1); v.cprev = cv.take<double>(1); v.coef = cv.take<double>(1);
-  v.cacc = cv.take<double>(1); v.qd64 = cv.take<double>(n);
-  v.st = cv.take<InstState>(1);
-  v.ctl = cv.take<Ctl>(1);
-  unsigned char *blk = cv.take<unsigned char>(blk_elems * ts);
-  unsigned char *its[3];
-  for (int b = 0; b < 3; ++b) its[b] = cv.take<unsigned char>(it_elems * ts);
-  unsigned char *qd_T = cv.take<unsigned char>(n * ts), *ref_T = cv.take<unsigned char>(n * ts);
-  unsigned char *lo_T = cv.take<unsigned char>(n * ts), *hi_T = cv.take<unsigned char>(n * ts);
-  unsigned char *xb0_T = cv.take<unsigned char>(n * ts);
-  if (cv.used > kStaticBytes) {
+  unsigned char *blk = nullptr, *its[3] = {nullptr, nullptr, nullptr};
+  unsigned char *qd_T = nullptr, *ref_T = nullptr, *lo_T = nullptr, *hi_T = nullptr, *xb0_T = nullptr;
+  int W = 0, res[6];
+  int64_t blk_elems = 0;
+  size_t smem = 0, used = 0;
+  RegLaunch reg;
+  // Carves the working memory; `resident`: the plain layout with one iterate buffer (the other
+  // two are not touched), else tiles of 32 stages with three.
+  auto carve = [&](bool resident) {
+    Carver cv{(unsigned char *)raw};
+    v.nx = cv.take<int>(1); v.nu = cv.take<int>(1); v.N = cv.take<int>(1); v.W = cv.take<int>(1);
+    for (int i = 0; i < 13; ++i) v.off[i] = cv.take<int64_t>(1);
+    v.binst = cv.take<int>(N);
+    v.item_inst = cv.take<int>(nitems); v.item_a = cv.take<int>(nitems); v.item_b = cv.take<int>(nitems);
+    v.nitems_inst = cv.take<int>(1);
+    v.list0 = cv.take<int>(nitems); v.list1 = cv.take<int>(nitems);
+    v.base = cv.take<int>(1); v.old_base = cv.take<int>(1); v.ndone = cv.take<int>(1);
+    v.stop = cv.take<int>(1); v.ferr = cv.take<int>(1);
+    v.alpha = cv.take<double>(1); v.cprev = cv.take<double>(1); v.coef = cv.take<double>(1);
+    v.cacc = cv.take<double>(1); v.qd64 = cv.take<double>(n);
+    v.st = cv.take<InstState>(1);
+    v.ctl = cv.take<Ctl>(1);
+    const int64_t ntiles = (N + 31) / 32;
+    int64_t it_elems;
+    if (resident) {
+      W = block_words(nx, nu);
+      blk_elems = (int64_t)N * W;
+      it_elems = (int64_t)N * admm_iter_stride(n, precision);
+    } else {
+      W = nx * n + nx + n * (n + 1) / 2 + nu * (nu + 1) / 2;
+      blk_elems = (ntiles * 32 * W + 31) / 32 * 32;
+      it_elems = ntiles * 32 * 5 * n;
+    }
+    blk = cv.take<unsigned char>(blk_elems * ts);
+    for (int b = 0; b < 3; ++b)
+      its[b] = resident && b > 0 ? its[0] : cv.take<unsigned char>(it_elems * ts);
+    qd_T = cv.take<unsigned char>(n * ts); ref_T = cv.take<unsigned char>(n * ts);
+    lo_T = cv.take<unsigned char>(n * ts); hi_T = cv.take<unsigned char>(n * ts);
+    xb0_T = cv.take<unsigned char>(n * ts);
+    if (resident && reg.xch_bytes > 0) reg.xch = cv.take<unsigned char>(reg.xch_bytes);
+    used = cv.used;
+  };
+  const int Wp = block_words(nx, nu);
+  bool resident = max_iters < kCoefs &&
+                  plan_resident(0, 1, &nx, &nu, &N, &Wp, 0, precision, nsm, (size_t)optin, res, &smem, &reg);
+  if (resident) {
+    carve(true);
+    resident = used <= kStaticBytes;
+  }
+  if (!resident) carve(false);
+  if (used > kStaticBytes) {
     char msg[200];
     snprintf(msg, sizeof msg,
              "pimpc_solve_static: this instance needs %zu bytes of working memory, more than the "
              "%zu-byte static array",
-             cv.used, kStaticBytes);
+             used, kStaticBytes);
     return fail_static(PIMPC_EINVAL, msg);
   }
 
   Layout L{};
-  L.batch = 1; L.lti = 0; L.tiled = 1;
+  L.batch = 1; L.lti = 0; L.tiled = resident ? 0 : 1;
   L.nx = v.nx; L.nu = v.nu; L.N = v.N; L.W = v.W;
   L.off_nx = v.off[0]; L.off_nu = v.off[1]; L.off_n = v.off[2];
   L.Nnx = v.off[3]; L.Nnu = v.off[4]; L.Nn = v.off[5];
@@ -193,10 +253,12 @@ extern "C" int pimpc_solve_static(int nx, int nu, int N, int precision, const do
                                         cudaGetErrorString(e2));
   };
   int ret;
-  static_setup_kernel<<<1, 128, 0, st>>>(v, nx, nu, N, W, it_elems, item_stages, nitems);
+  static_setup_kernel<<<1, 128, 0, st>>>(v, nx, nu, N, W, item_stages, nitems);
   if ((ret = check(cudaGetLastError(), "setup"))) return ret;
   // Everything the kernels read before writing starts from a known state on every call.
-  if ((ret = check(cudaMemsetAsync(blk, 0, blk_elems * ts, st), "clear stage blocks"))) return ret;
+  // (The factorisation writes every word of a plain block; tiles hold stages beyond N.)
+  if (!resident && (ret = check(cudaMemsetAsync(blk, 0, blk_elems * ts, st), "clear stage blocks")))
+    return ret;
   if ((ret = check(launch_gather_n64(L, q, r, n, v.qd64, st), "weights"))) return ret;
   if ((ret = check(launch_gather_n(L, q, r, n, precision, qd_T, st), "weights"))) return ret;
   if ((ret = check(launch_gather_n(L, xmin, umin, n, precision, lo_T, st), "bounds"))) return ret;
@@ -224,15 +286,21 @@ extern "C" int pimpc_solve_static(int nx, int nu, int N, int precision, const do
   a.u_out = u_out; a.x_out = x_out;
   a.warm = 0;  // cold start: the iterate buffer is cleared by the launch sequence
   a.ferr = v.ferr;
-  a.threads = tps_threads();
-  a.nv_max = n;
-  const size_t smem = tps_smem_bytes(n, precision);
-  int bps = 0, nsm = 0, dev = 0;
-  if ((ret = check(tps_configure(precision, smem, &bps), "configure"))) return ret;
-  if ((ret = check(cudaGetDevice(&dev), "device"))) return ret;
-  if ((ret = check(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev), "device"))) return ret;
-  a.grid = std::min(nitems, std::max(1, bps * nsm));
-  if ((ret = check(launch_tps(a, precision, st), "solve"))) return ret;
+  a.coef_tab = coefs;
+  if (resident) {
+    a.threads = reg.threads > 0 ? reg.threads : res_threads(precision);
+    ret = check(reg.threads > 0 ? launch_reg(a, precision, reg, st)
+                                : launch_resident(a, precision, res, smem, st), "solve");
+  } else {
+    a.threads = tps_threads();
+    a.nv_max = n;
+    const size_t tps_smem = tps_smem_bytes(n, precision);
+    int bps = 0;
+    if ((ret = check(tps_configure(precision, tps_smem, &bps), "configure"))) return ret;
+    a.grid = std::min(nitems, std::max(1, bps * nsm));
+    ret = check(launch_tps(a, precision, st), "solve");
+  }
+  if (ret) return ret;
   if (iters || c || status)
     if ((ret = check(launch_unpack_state(v.st, 1, iters, c, status, nullptr, st), "results"))) return ret;
   return PIMPC_OK;
