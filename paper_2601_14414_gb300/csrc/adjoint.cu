@@ -35,6 +35,7 @@
 
 #include "launch.h"
 #include "pimpc.h"
+#include "regvec.cuh"
 #include "solver.h"
 
 namespace pimpc {
@@ -485,6 +486,328 @@ __global__ void __launch_bounds__(256) adjoint_kernel(AdjArgs a) {
   (void)nu;
 }
 
+// ---- the same sweep with an instance in the registers of one CTA (n <= 16) ---------------------
+//
+// The sweep above reads every matrix element and every vector component from memory; one cart-pole
+// batch (1024 instances, N 100, 150 iterations) took it 12.5 ms. Here thread (k, c) holds component
+// c of stage k and its rows of G_k, H_k, P_k = Bbar_k M_k Bbar_k^T and its column of G_{k+1}, as in
+// the register-resident solve (admm_reg.cuh, whose reduced iteration with lambda = -beta this
+// reverses), and the vectors cross threads through shared memory. With bars for adjoints, an
+// iteration
+//   w = v - beta, y = z - v - beta - ebar, h = Qbar ref + rho (z - theta + Abar_{k+1}^T y_{k+1}),
+//   xb = H h, p = beta + P w, q = Abar xb_{k-1} + beta + ebar, s = xb + theta,
+//   z' = clamp((2 s + p + q) / 3), v' = (z' + p - q) / 2, theta' = s - z', beta' = p - v'
+// reverses to
+//   vt = v'bar - beta'bar, zt = z'bar - theta'bar + vt / 2, wb = zt / 3 where w was inside the box,
+//   pb = beta'bar + vt / 2 + wb, qb = wb - vt / 2, sb = theta'bar + 2 wb,
+//   xbbar = sb + Abar_{k+1}^T qb_{k+1}, hbar = H xbbar, yb = Abar_k rho hbar_{k-1},
+//   zbar = rho hbar + yb, vbar = P pb - yb, thetabar = sb - rho hbar, betabar = pb + qb - yb - P pb:
+// linear but for the clamp, so all it needs of the forward iteration is which side each component
+// was clamped to (two bits) and, for the weights' gradient, xb. Both are kept for a whole segment
+// (every iteration at once when that takes no more memory than the checkpoints and states of the
+// sweep above), in place of K full states. Gradient sums run in FP64 for FP64 iterations and as
+// unevaluated float pairs (48 bits, error-free additions) for FP32 ones: three FP64 additions per
+// thread and iteration would take longer than the iteration.
+struct RegAdj {
+  int region;       // elements of each of the four vector regions in shared memory
+  int K, nck;       // iterations per segment, segments
+  int keep_xb;      // the gradients need xb
+  const int64_t *off;  // per-instance workspace offset (bytes)
+  unsigned char *ws;   // per instance: nck states of 4 vectors, K x xb, K x clamp bits
+};
+
+template <typename T>
+struct Sum;
+template <>
+struct Sum<double> {
+  double v = 0.0;
+  __device__ __forceinline__ void add(double x) { v += x; }
+  __device__ __forceinline__ void add_product(double x, double y) { v = fma(x, y, v); }
+  __device__ __forceinline__ double value() const { return v; }
+};
+template <>
+struct Sum<float> {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float x) {  // Knuth's two-sum
+    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+    hi = s;
+  }
+  __device__ __forceinline__ void add_product(float x, float y) {
+    const float p = __fmul_rn(x, y);
+    add(p);
+    lo = __fadd_rn(lo, fmaf(x, y, -p));
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
+__host__ __device__ constexpr int adj_max_threads(int tsize, int NM) {
+  return tsize == 4 ? 512 : (NM <= 8 ? 512 : 256);
+}
+
+template <typename T, int NM>
+__global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_reg_kernel(AdjArgs a, RegAdj ra) {
+  extern __shared__ __align__(128) unsigned char adj_smem[];
+  __shared__ T sG0[NM][NM];  // G_0, for the adjoint of x_0
+  const int j = a.order[blockIdx.x];
+  Inst<T> I;
+  make_inst(a, j, I);
+  const int n = I.n, N = I.N, nx = I.nx, nu = I.nu;
+  const int nv = reg_nv(n, (int)sizeof(T));
+  const int tid = threadIdx.x, nthreads = blockDim.x;
+  const int k = tid / n, c = tid - k * n;
+  const bool on = k < N, more = on && k + 1 < N;
+  T *s0 = reinterpret_cast<T *>(adj_smem), *s1 = s0 + ra.region, *s2 = s1 + ra.region, *s3 = s2 + ra.region;
+  const int row = k * nv, at = row + c;
+  for (int i = tid; i < 4 * ra.region; i += nthreads) s0[i] = (T)0;
+  for (int i = tid; i < nx * nx; i += nthreads) sG0[i / nx][i % nx] = I.Gv(0, i / nx, i % nx);
+
+  T Gn[NM], Gr[NM], Hr[NM], Pr[NM];
+#pragma unroll
+  for (int q = 0; q < NM; ++q) Gn[q] = Gr[q] = Hr[q] = Pr[q] = (T)0;
+  T ee = 0, qref = 0, rv = 0, lo = 0, hi = 0;
+  if (on) {
+    ee = c < nx ? I.Ev(k, c) : (T)0;
+    lo = I.lo[c];
+    hi = I.hi[c];
+    if (I.refk(k)) rv = I.refk(k)[c];
+    qref = I.qd[c] * rv;
+#pragma unroll
+    for (int q = 0; q < NM; ++q)
+      if (q < n) {
+        Hr[q] = I.Hv(k, c, q);
+        Gr[q] = c < nx ? I.Gv(k, c, q) : (q == c ? (T)1 : (T)0);
+        if (q < nx && more) Gn[q] = I.Gv(k + 1, q, c);
+      }
+    for (int i = 0; i < nu; ++i) {  // P row c = sum_i (Bbar M)_{c,i} (row i of Bbar^T)
+      T t = (T)0;
+      if (c < nx) {
+        for (int q = 0; q < nu; ++q) t += I.Gv(k, c, nx + q) * I.Mv(k, q, i);
+      } else {
+        t = I.Mv(k, c - nx, i);
+      }
+#pragma unroll
+      for (int q = 0; q < NM; ++q)
+        if (q < n) Pr[q] += t * (q < nx ? I.Gv(k, q, nx + i) : (q - nx == i ? (T)1 : (T)0));
+    }
+  }
+  const T rho = I.rho;
+  const int64_t nt = (n * N + 31) & ~31;  // this instance's stride in the workspace
+  const bool kept = tid < nt;
+  T *ck = reinterpret_cast<T *>(ra.ws + ra.off[j]);                    // [nck][4][nt]
+  T *xbs = ck + (int64_t)ra.nck * 4 * nt;                               // [K][nt]
+  uint2 *bits = reinterpret_cast<uint2 *>(xbs + (ra.keep_xb ? (int64_t)ra.K * nt : 0));  // [K][warps]
+  const int nw = (int)(nt >> 5), warp = tid >> 5, lane = tid & 31;
+  const T x0 = tid < n ? I.xb0[tid] : (T)0;
+
+  T z = 0, v = 0, t = 0, b = 0;
+  // One forward iteration; m >= 0: keep its clamp bits and xb as the segment's m-th.
+  auto forward = [&](int m) {
+    const T be = b + ee;
+    if (on) {
+      s0[at] = v - b;
+      s1[at] = (z - v) - be;
+    }
+    if (tid < n) s3[tid] = x0;  // row 0: xbar_0; row k + 1: xbar_{k+1}
+    __syncthreads();
+    T p = (T)0;
+    if (on) {
+      T acc = z - t;
+      if (more) {
+        if (c >= nx) acc += s1[at + nv];
+        acc = dot(Gn, s1 + row + nv, nx, acc);
+      }
+      s2[at] = qref + rho * acc;
+      p = dot(Pr, s0 + row, n, b);
+    }
+    __syncthreads();
+    T xb = (T)0;
+    if (on) {
+      xb = dot(Hr, s2 + row, n, (T)0);
+      s3[at + nv] = xb;
+    }
+    __syncthreads();
+    bool below = false, above = false;
+    if (on) {
+      const T q = dot(Gr, s3 + row, n, be);
+      const T s = xb + t;
+      const T w = third((T)2 * s + (p + q));
+      below = w <= lo;
+      above = !below && w >= hi;
+      z = w < lo ? lo : (w > hi ? hi : w);
+      v = (T)0.5 * (z + (p - q));
+      t = s - z;
+      b = p - v;
+    }
+    if (m >= 0) {
+      const unsigned bl = __ballot_sync(0xffffffffu, below), ab = __ballot_sync(0xffffffffu, above);
+      if (lane == 0 && kept) bits[(int64_t)m * nw + warp] = make_uint2(bl, ab);
+      if (ra.keep_xb && kept) xbs[(int64_t)m * nt + tid] = xb;
+    }
+  };
+  auto checkpoint = [&](int seg) {
+    if (!kept) return;
+    T *o = ck + (int64_t)seg * 4 * nt + tid;
+    o[0] = z; o[nt] = v; o[2 * nt] = t; o[3 * nt] = b;
+  };
+
+  __syncthreads();
+  const int last = ra.nck - 1;  // the last segment's states need no checkpoint of their own
+  for (int seg = 0; seg < last; ++seg) {
+    checkpoint(seg);
+    for (int m = 0; m < ra.K; ++m) forward(-1);
+  }
+
+  // Adjoint of the last iterate: z = (x, u).
+  T zb = 0, vb = 0, tb = 0, bb = 0;
+  if (on) {
+    if (c < nx) zb = a.dL_dx ? (T)a.dL_dx[a.L.Nnx[j] + (int64_t)k * nx + c] : (T)0;
+    else zb = a.dL_du ? (T)a.dL_du[a.L.Nnu[j] + (int64_t)k * nu + c - nx] : (T)0;
+  }
+  Sum<T> hs, hx, los, his, x0s;
+  for (int seg = last; seg >= 0; --seg) {
+    const int len = min(ra.K, a.iters - seg * ra.K);
+    if (seg < last && kept) {
+      const T *o = ck + (int64_t)seg * 4 * nt + tid;
+      z = o[0]; v = o[nt]; t = o[2 * nt]; b = o[3 * nt];
+    }
+    for (int m = 0; m < len; ++m) forward(m);
+    __syncthreads();  // the bits of this segment (written by lane 0), and the regions' last reads
+    for (int m = len - 1; m >= 0; --m) {
+      const uint2 side = kept ? bits[(int64_t)m * nw + warp] : make_uint2(0u, 0u);
+      const T xb = ra.keep_xb && kept ? xbs[(int64_t)m * nt + tid] : (T)0;
+      const bool below = side.x >> lane & 1u, above = side.y >> lane & 1u;
+      const T half = (T)0.5 * (vb - bb);
+      const T zt = (zb - tb) + half;
+      T wb = (T)0;
+      if (below) los.add(zt);
+      else if (above) his.add(zt);
+      else wb = third(zt);
+      const T pb = (bb + half) + wb, qb = wb - half, sb = tb + (T)2 * wb;
+      if (on) {
+        s0[at] = pb;
+        s1[at] = qb;
+      }
+      __syncthreads();
+      T ab = (T)0;
+      if (on) {
+        T acc = sb;
+        if (more) {
+          if (c >= nx) acc += s1[at + nv];
+          acc = dot(Gn, s1 + row + nv, nx, acc);
+        }
+        s2[at] = acc;
+        ab = dot(Pr, s0 + row, n, (T)0);
+        if (k == 0 && c < nx) {
+          T g = (T)0;
+          for (int r = 0; r < nx; ++r) g += sG0[r][c] * s1[r];
+          x0s.add(g);
+        }
+      }
+      __syncthreads();
+      T rh = (T)0;
+      if (on) {
+        const T hb = dot(Hr, s2 + row, n, (T)0);
+        hs.add(hb);
+        hx.add_product(hb, xb);
+        rh = rho * hb;
+        s3[at + nv] = rh;  // row k + 1, read by stage k + 1
+      }
+      __syncthreads();
+      T yb = (T)0;
+      if (on && k > 0) yb = dot(Gr, s3 + row, n, (T)0);
+      zb = rh + yb;
+      vb = ab - yb;
+      tb = sb - rh;
+      bb = (pb + qb) - (yb + ab);
+    }
+  }
+
+  // Gradients: sums over the stages, pairwise.
+  const double qd = on ? (double)I.qd[c] : 0.0, h = hs.value();
+  double *sd = reinterpret_cast<double *>(adj_smem);
+  if (on && a.g_ref && a.ref_per_stage) a.g_ref[a.L.Nn[j] + (int64_t)k * n + c] = qd * h;
+  int top = 1;
+  while (2 * top < N) top *= 2;
+  auto total = [&](double x) {  // of component c, in thread (0, c)
+    __syncthreads();
+    if (on) sd[tid] = x;
+    for (int s = top; s > 0; s >>= 1) {
+      __syncthreads();
+      if (k < s && k + s < N) sd[tid] += sd[tid + s * n];
+    }
+    return sd[tid < n ? tid : 0];
+  };
+  const double gq = total((double)rv * h - hx.value());
+  const double glo = total(los.value());
+  const double ghi = total(his.value());
+  const double gref = total(qd * h);
+  if (tid < n) {
+    if (a.g_ref && !a.ref_per_stage) a.g_ref[a.L.off_n[j] + c] = gref;
+    if (c < nx) {
+      if (a.g_q) a.g_q[a.L.off_nx[j] + c] = gq;
+      if (a.g_xmin) a.g_xmin[a.L.off_nx[j] + c] = glo;
+      if (a.g_xmax) a.g_xmax[a.L.off_nx[j] + c] = ghi;
+      if (a.g_x0) a.g_x0[a.L.off_nx[j] + c] = x0s.value();
+    } else {
+      const int q = c - nx;
+      if (a.g_r) a.g_r[a.L.off_nu[j] + q] = gq;
+      if (a.g_umin) a.g_umin[a.L.off_nu[j] + q] = glo;
+      if (a.g_umax) a.g_umax[a.L.off_nu[j] + q] = ghi;
+    }
+  }
+}
+
+// Plan of the register sweep: threads (0: some instance has n > 16 or more components than a CTA
+// holds threads), the segment length, and the workspace offsets.
+struct RegAdjPlan {
+  int threads = 0, NM = 0;
+  RegAdj ra{};
+  std::vector<int64_t> off;
+  int64_t bytes = 0;
+};
+
+RegAdjPlan plan_reg_adjoint(const pimpc_solver *s, int Tn, int K, int nck, int slots, bool keep_xb) {
+  RegAdjPlan p;
+  const int ts = (int)tsize(s->prec);
+  int nmax = 1, thr = 0, reg = 0;
+  for (int j = 0; j < s->batch; ++j) nmax = std::max(nmax, s->nx[j] + s->nu[j]);
+  if (nmax > 16 || Tn < 1) return p;
+  p.NM = nmax <= 4 ? 4 : (nmax <= 8 ? 8 : 16);
+  for (int j = 0; j < s->batch; ++j) {
+    const int n = s->nx[j] + s->nu[j];
+    if ((int64_t)n * s->N[j] > adj_max_threads(ts, p.NM)) return p;
+    thr = std::max(thr, n * s->N[j]);
+    reg = std::max(reg, (s->N[j] + 1) * reg_nv(n, ts));
+  }
+  p.threads = (thr + 31) / 32 * 32;
+  p.ra.region = (reg + 3) / 4 * 4;
+  p.ra.keep_xb = keep_xb;
+  // words per component: what the other sweep takes, and what keeping every iteration takes
+  const double theirs = 5.0 * (nck + slots + 1) + 4.0 + 32.0 / ts;
+  const double whole = 4.0 + Tn * ((keep_xb ? 1.0 : 0.0) + 0.25 / ts);
+  p.ra.K = whole <= theirs ? Tn : K;
+  p.ra.nck = whole <= theirs ? 1 : nck;
+  for (int j = 0; j < s->batch; ++j) {
+    const int64_t nt = ((int64_t)(s->nx[j] + s->nu[j]) * s->N[j] + 31) / 32 * 32;
+    p.off.push_back(p.bytes);
+    p.bytes += ((int64_t)p.ra.nck * 4 + (keep_xb ? p.ra.K : 0)) * nt * ts +
+               (int64_t)p.ra.K * (nt / 32) * (int64_t)sizeof(uint2);
+    p.bytes = (p.bytes + 255) & ~(int64_t)255;
+  }
+  return p;
+}
+
+template <typename T>
+cudaError_t launch_reg_adjoint(const AdjArgs &a, const RegAdjPlan &p, int batch, cudaStream_t st) {
+  auto kernel = p.NM == 4 ? adjoint_reg_kernel<T, 4> : (p.NM == 8 ? adjoint_reg_kernel<T, 8> : adjoint_reg_kernel<T, 16>);
+  const size_t smem = (size_t)4 * p.ra.region * sizeof(T);
+  const cudaError_t rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (rc != cudaSuccess) return rc;
+  kernel<<<batch, p.threads, smem, st>>>(a, p.ra);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 }  // namespace pimpc
@@ -515,21 +838,24 @@ extern "C" int pimpc_backward(pimpc_solver *s, const double *dL_du, const double
   const int slots = std::max(K - 1, 2);
   const size_t ts = tsize(s->prec);
 
+  RegAdjPlan rp = plan_reg_adjoint(s, Tn, K, nck, slots, g_q != nullptr || g_r != nullptr);
+  const bool in_regs = rp.threads > 0;
   // Workspace: per-instance T region and FP64 accumulators, the CTA order, host staging.
   std::vector<int64_t> offT(s->batch), offD(s->batch);
   int64_t totT = 0, totD = 0;
   int maxN = 1;
   for (int j = 0; j < s->batch; ++j) {
     const int64_t n = s->nx[j] + s->nu[j], N = s->N[j], nu = s->nu[j];
+    maxN = std::max(maxN, (int)N);
     offT[j] = totT;
     // checkpoints, recompute slots and the adjoint state (5 n N each); xb, p, yb, xbp (n N);
     // du, dubar (nu N)
+    if (in_regs) continue;
     totT += (5 * n * N) * (nck + slots + 1) + 4 * n * N + 2 * nu * N;
     totT = (totT + 31) & ~(int64_t)31;
     offD[j] = totD;
     totD += 4 * n * N + s->nx[j];
     totD = (totD + 3) & ~(int64_t)3;
-    maxN = std::max(maxN, (int)N);
   }
   const int64_t n_ref = s->last_ref_per_stage ? s->tot_Nn : s->tot_n;
   const int64_t stage_in = s->tot_Nnu + s->tot_Nnx;
@@ -538,7 +864,7 @@ extern "C" int pimpc_backward(pimpc_solver *s, const double *dL_du, const double
   const size_t parts[7] = {sizeof(int64_t) * s->batch, sizeof(int64_t) * s->batch,
                            sizeof(int) * s->batch,     sizeof(double) * totD,
                            sizeof(double) * stage_in,  sizeof(double) * stage_out,
-                           ts * totT};
+                           in_regs ? (size_t)rp.bytes : ts * totT};
   size_t bytes = 0;
   for (size_t b : parts) bytes += rounded(b);
   if (bytes > s->adj_ws_bytes) {
@@ -575,6 +901,7 @@ extern "C" int pimpc_backward(pimpc_solver *s, const double *dL_du, const double
     const double cy = (double)s->N[y] * (s->nx[y] + s->nu[y]) * (s->nx[y] + s->nu[y]);
     return cx > cy;
   });
+  if (in_regs) offT = rp.off;
   PIMPC_CHECK(s, cudaMemcpyAsync(d_offT, offT.data(), sizeof(int64_t) * s->batch, cudaMemcpyHostToDevice, st), "adjoint offsets");
   PIMPC_CHECK(s, cudaMemcpyAsync(d_offD, offD.data(), sizeof(int64_t) * s->batch, cudaMemcpyHostToDevice, st), "adjoint offsets");
   PIMPC_CHECK(s, cudaMemcpyAsync(d_order, order.data(), sizeof(int) * s->batch, cudaMemcpyHostToDevice, st), "adjoint order");
@@ -621,7 +948,13 @@ extern "C" int pimpc_backward(pimpc_solver *s, const double *dL_du, const double
     a.g_r = g_r; a.g_umin = g_umin; a.g_umax = g_umax; a.g_ref = g_ref;
   }
   const int threads = std::min(256, std::max(32, (maxN + 31) / 32 * 32));
-  if (s->prec == PIMPC_F32) adjoint_kernel<float><<<s->batch, threads, 0, st>>>(a);
+  if (in_regs) {
+    rp.ra.off = d_offT;
+    rp.ra.ws = (unsigned char *)d_T;
+    PIMPC_CHECK(s, s->prec == PIMPC_F32 ? launch_reg_adjoint<float>(a, rp, s->batch, st)
+                                        : launch_reg_adjoint<double>(a, rp, s->batch, st),
+                "adjoint launch");
+  } else if (s->prec == PIMPC_F32) adjoint_kernel<float><<<s->batch, threads, 0, st>>>(a);
   else adjoint_kernel<double><<<s->batch, threads, 0, st>>>(a);
   PIMPC_CHECK(s, cudaGetLastError(), "adjoint launch");
   if (host) {

@@ -1,0 +1,57 @@
+// regvec.cuh -- products of a register-resident matrix row with a vector in shared memory, and x / 3,
+// as the register-resident solve and adjoint use them (internal).
+#pragma once
+#include <cuda_runtime.h>
+
+namespace pimpc {
+
+// Elements of a vector of n in shared memory: whole 16-byte pieces.
+__host__ __device__ inline int reg_nv(int n, int tsize) {
+  const int w = tsize == 4 ? 4 : 2;
+  return (n + w - 1) / w * w;
+}
+
+// init + sum_j m[j] v[j] over j < cnt, v in shared memory (16-byte aligned, zero-padded to whole
+// vectors), m in registers with zeros beyond its length. FP64 runs one chain: a warp issues an
+// FP64 instruction every 64 cycles, which is also its latency, so a second chain gains nothing.
+template <int NM>
+__device__ __forceinline__ float dot(const float (&m)[NM], const float *v, int cnt, float init) {
+  float a0 = init, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
+#pragma unroll
+  for (int j = 0; j < NM; j += 4)
+    if (j < cnt) {
+      const float4 q = *reinterpret_cast<const float4 *>(v + j);
+      a0 = fmaf(m[j], q.x, a0);
+      a1 = fmaf(m[j + 1], q.y, a1);
+      a2 = fmaf(m[j + 2], q.z, a2);
+      a3 = fmaf(m[j + 3], q.w, a3);
+    }
+  return (a0 + a1) + (a2 + a3);
+}
+template <int NM>
+__device__ __forceinline__ double dot(const double (&m)[NM], const double *v, int cnt, double init) {
+  double a = init;
+#pragma unroll
+  for (int j = 0; j < NM; j += 2)
+    if (j < cnt) {
+      const double2 q = *reinterpret_cast<const double2 *>(v + j);
+      a = fma(m[j], q.x, a);
+      a = fma(m[j + 1], q.y, a);
+    }
+  return a;
+}
+
+// x / 3 to within a rounding of the correctly rounded quotient: 1/3 as the sum of its rounding
+// and the rounding of what is left (two operations instead of a division; infinities pass).
+__device__ __forceinline__ float third(float x) {
+  constexpr float hi = 1.0f / 3.0f;
+  constexpr float lo = (float)(1.0 / 3.0 - (double)hi);
+  return fmaf(x, hi, x * lo);
+}
+__device__ __forceinline__ double third(double x) {
+  constexpr double hi = 1.0 / 3.0;         // (1 - 2^-54) / 3
+  constexpr double lo = hi * 0x1p-54;      // 1/3 - hi = 2^-54 / 3
+  return fma(x, hi, x * lo);
+}
+
+}  // namespace pimpc
