@@ -80,22 +80,6 @@ struct RegPlan {
 constexpr int kHaloRecs = 3 * kMaxN;
 __host__ __device__ inline size_t xch_records(int C) { return (size_t)2 * C * (1 + 2 * kHaloRecs); }
 
-// min(max(w, lo), hi), NaN passing through. FP64 by the order of the bit patterns: two FP64
-// comparisons would cost 128 cycles.
-__device__ __forceinline__ float clamp(float w, float lo, float hi) {
-  return w < lo ? lo : (w > hi ? hi : w);
-}
-__device__ __forceinline__ long long order_key(double v) {
-  const long long b = __double_as_longlong(v);
-  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
-}
-__device__ __forceinline__ double clamp(double w, double lo, double hi) {
-  const long long k = order_key(w);
-  const bool nan = (__double_as_longlong(w) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
-  const double z = k < order_key(lo) ? lo : (k > order_key(hi) ? hi : w);
-  return nan ? w : z;
-}
-
 template <typename T>
 __device__ __forceinline__ T sym_at(const T *Wp, int m, int r, int c) {
   int d = c - r;

@@ -501,15 +501,26 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
       P.threads = reg.threads > 0 ? reg.threads : res_threads(precision);
     }
     s->reg_plan = reg;
+    // FP64 iterations: the full-warp kernel (the lane groups stay for non-box input sets).
+    int dense_bps = 0;
+    if (sc.family == 0 && precision == PIMPC_F64 && e == cudaSuccess &&
+        dense_plan(batch, nx.data(), nu.data(), W.data(), lti, smem_sm, optin, grp.data(),
+                   s->dense_plan, &s->dense_smem))
+      e = dense_configure(s->dense_smem, &dense_bps);
+    s->dense_grid = dense_bps * nsm;
+    if (dense_bps > 0) {
+      total_sub = 0;
+      for (int j = 0; j < batch; ++j) total_sub += (N[j] + grp[j] - 2) / (grp[j] - 1);
+    }
     if (e == cudaSuccess && bps >= 1) {
-      const int64_t max_grid = (int64_t)bps * nsm;
+      const int64_t max_grid = dense_bps > 0 ? s->dense_grid : (int64_t)bps * nsm;
       // Sub-chunks per item: enough items for about 4 per CTA, at most 16 sub-chunks per item.
       int64_t m = sc.item_scale > 0 ? sc.item_scale : total_sub / (4 * max_grid);
       m = std::max<int64_t>(1, std::min<int64_t>(sc.item_scale > 0 ? 64 : 16, m));
       for (int oi = 0; oi < batch; ++oi) {
         const int j = order[oi];
         const int n = nx[j] + nu[j];
-        const int S = threads / admm_group_size(n);
+        const int S = dense_bps > 0 ? grp[j] - 1 : threads / admm_group_size(n);
         int is = (int)(S * m);
         if (lti) is = std::max(is, std::min(N[j], (256 + S - 1) / S * S));
         if (!lti && m > fine_sub) fine_len[j] = S * fine_sub;
@@ -529,6 +540,8 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
   }
   const int nitems = (int)item_inst.size();
   const int grid = (int)std::min<int64_t>((int64_t)bps * nsm, nitems);
+  if (sc.family != 0) s->dense_grid = 0;
+  s->dense_grid = std::min(s->dense_grid, nitems);
   for (int oi = 0; oi < batch; ++oi) {
     const int j = order[oi];
     if (fine_len[j] <= 0) continue;
@@ -583,7 +596,7 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
   chk(lalloc(s, &s->item_first, sizeof(int) * 2 * batch));
   chk(lalloc(s, &s->cpart, sizeof(double) * nall));
   chk(lalloc(s, &s->list_init, sizeof(int) * std::max(nitems, 1)));
-  chk(lalloc(s, &s->ccount, sizeof(int) * std::max(grid, 1)));
+  chk(lalloc(s, &s->ccount, sizeof(int) * std::max({grid, s->dense_grid, 1})));
   chk(lalloc(s, &s->pos_of, sizeof(int) * nall));
   chk(lalloc(s, &d_blk, sizeof(int64_t) * batch));
   chk(lalloc(s, &d_Ni, sizeof(int64_t) * batch));
@@ -705,7 +718,13 @@ int run_solve(pimpc_solver *s, const double *dx0, const double *dup, const doubl
     return fail(s, PIMPC_ESTATE, "momentum table shorter than max_iters");
   if (s->sched.family == 7 && s->accel)
     return fail(s, PIMPC_ESTATE, "temporal blocking (schedule 7) runs the plain iteration: accel must be 0");
-  PIMPC_CHECK(s, s->tiled == 2 ? launch_tile(a, st)
+  const bool dense = s->sched.family == 0 && s->dense_grid > 0 && !s->any_uset;
+  if (dense) {
+    a.grid = s->dense_grid;
+    a.threads = dense_threads();
+  }
+  PIMPC_CHECK(s, dense ? launch_dense(a, s->dense_plan, s->dense_smem, st)
+                 : s->tiled == 2 ? launch_tile(a, st)
                  : s->tiled == 3 ? launch_blk(a, s->prec, s->smem_admm, st)
                  : s->sched.family == 3 && s->reg_plan.threads > 0 ? launch_reg(a, s->prec, s->reg_plan, st)
                  : s->sched.family == 3 ? launch_resident(a, s->prec, s->res_plan, s->smem_admm, st)

@@ -72,6 +72,13 @@ size_t admm_smem_bytes(const AdmmLaunch &s, int precision);
 cudaError_t admm_configure(int precision, size_t smem, int *blocks_per_sm);
 cudaError_t launch_admm(const AdmmLaunch &a, int precision, cudaStream_t stream);
 
+// FP64 iterations on box constraints with full warps (schedule family 0; the plain layout).
+bool dense_plan(int batch, const int *nx, const int *nu, const int *W, int lti, int64_t smem_sm,
+                int64_t optin, int *slots, int *plan, size_t *smem);
+int dense_threads();
+cudaError_t dense_configure(size_t smem, int *blocks_per_sm);
+cudaError_t launch_dense(const AdmmLaunch &s, const int *plan, size_t smem, cudaStream_t stream);
+
 // One thread per stage on halo tiles (stage-varying FP32 instances).
 int tile_threads();
 int tile_warps();

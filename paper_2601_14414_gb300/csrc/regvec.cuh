@@ -1,5 +1,5 @@
-// regvec.cuh -- products of a register-resident matrix row with a vector in shared memory, and x / 3,
-// as the register-resident solve and adjoint use them (internal).
+// regvec.cuh -- products of a register-resident matrix row with a vector in shared memory, x / 3 and
+// the clamp, as the kernels that count FP64 instructions use them (internal).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -52,6 +52,27 @@ __device__ __forceinline__ double third(double x) {
   constexpr double hi = 1.0 / 3.0;         // (1 - 2^-54) / 3
   constexpr double lo = hi * 0x1p-54;      // 1/3 - hi = 2^-54 / 3
   return fma(x, hi, x * lo);
+}
+
+// min(max(w, lo), hi), NaN passing through. FP64 by the order of the bit patterns: two FP64
+// comparisons would cost 128 cycles.
+__device__ __forceinline__ float clamp(float w, float lo, float hi) {
+  return w < lo ? lo : (w > hi ? hi : w);
+}
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double clamp(double w, double lo, double hi) {
+  const long long k = order_key(w);
+  const bool nan = (__double_as_longlong(w) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+  const double z = k < order_key(lo) ? lo : (k > order_key(hi) ? hi : w);
+  return nan ? w : z;
+}
+
+// -v without an FP64 instruction.
+__device__ __forceinline__ double negated(double v) {
+  return __hiloint2double(__double2hiint(v) ^ (int)0x80000000, __double2loint(v));
 }
 
 }  // namespace pimpc

@@ -11,6 +11,9 @@ struct pimpc_solver {
   std::vector<int> nx, nu, N, W, tw;
   pimpc::Schedule sched{};
   int res_plan[6] = {0, 0, 0, 0, 0, 0};   // resident schedule: cluster size and smem regions
+  int dense_plan[3] = {0, 0, 0};          // FP64 full-warp kernel: regions, grid (0: not used)
+  int dense_grid = 0;
+  size_t dense_smem = 0;
   pimpc::RegLaunch reg_plan;              // resident schedule in registers (threads 0: not used)
   int gemm_plan[5] = {0, 0, 0, 0, 0};     // contraction schedule: stages per item, padding
   double *coef_tab = nullptr;             // momentum factors by streak length (resident)
