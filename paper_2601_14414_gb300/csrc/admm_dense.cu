@@ -257,16 +257,16 @@ __global__ void __launch_bounds__(kThreads, 3) dense_kernel(ls::Args<double> a, 
         // ---- steps 2-4 ----
         if (owned) {
           const double *xk = sX + slot * nv, *du = sD + slot * nuv;
-          double p, qv;  // beta + Bbar du, Abar xbar + ebar - lambda
+          double bd, qv;  // Bbar du, Abar xbar + ebar - lambda
           if (c < nx) {
             const double *row = Gk + c * ldg;  // odd stride: the lanes' rows hit distinct banks
             qv = dot_strided(row, 1, xk, n, be);
-            p = dot_strided(row + nx, 1, du, nu, bh);
+            bd = dot_strided(row + nx, 1, du, nu, 0.0);
           } else {
             qv = be + xk[c];
-            p = bh + du[c - nx];
+            bd = du[c - nx];
           }
-          const double s = xb + th;
+          const double s = xb + th, p = bh + bd;
           const double z = clamp(third(2.0 * s + (p + qv)), lo, hi);
           const double v = 0.5 * (z + (p - qv));
           const double t = s - z, b = p - v;
@@ -276,7 +276,8 @@ __global__ void __launch_bounds__(kThreads, 3) dense_kernel(ls::Args<double> a, 
           o[2 * n] = t;
           o[3 * n] = b;
           o[4 * n] = negated(b);
-          const double d1 = t - th, d2 = b - bh, d4 = z - zh, d5 = v - vh;
+          // theta' - theta = xbar - z' and beta' - beta = Bbar du - v', without the duals' own rounding
+          const double d1 = xb - z, d2 = bd - v, d4 = z - zh, d5 = v - vh;
           // d1^2 + d2^2 + d3^2 + d4^2 + d5^2 + (d4 - d5)^2 with d3 = -d2
           const double g = d2 * d2 + (d4 * d4 + d5 * (d5 - d4));
           cacc = fma(d1, d1, fma(2.0, g, cacc));

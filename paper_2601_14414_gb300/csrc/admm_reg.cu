@@ -13,7 +13,8 @@ void reg_plan(int batch, const int *nx, const int *nu, const int *N, int precisi
   for (int j = 0; j < batch; ++j) nm = std::max(nm, nx[j] + nu[j]);
   rl->threads = 0;
   if (nm > kMaxN || C > kMaxC) return;
-  const int cap = reg_max_threads(ts, reg_class(nm));
+  const int cls = reg_class(nm);  // more CTAs than a cluster: with the deciding warp
+  const int cap = C > 16 ? spec_max_threads(ts, cls) - 32 : reg_max_threads(ts, cls);
   for (int j = 0; j < batch; ++j) {
     const int n = nx[j] + nu[j];
     if (N[j] < C) return;
@@ -29,19 +30,19 @@ void reg_plan(int batch, const int *nx, const int *nu, const int *N, int precisi
 }
 
 // The resident schedule in registers (n <= 16): CTAs per instance, 0 threads if it does not fit.
-// With item_scale = 0 one CTA as long as its threads stay within `one`: an exchange in a cluster
-// costs about what 200 more FP32 threads do (n 16, N 20: 1.36 us per iteration on one CTA of 320
-// threads, 1.60 on four), and four warps, one per scheduler, are what the FP64 pipe takes before
-// a warp's instructions queue (n 6, N 20: 3.23 us on one CTA, 3.48 on two; N 60: 7.98 and 3.54
-// on four). Else the smallest cluster whose CTAs stay within `few` threads, the cluster of 16
-// within `most`, and beyond that (FP64, whose iterations are long enough to pay for an exchange
-// through global memory, or instances that no cluster holds) the fewest CTAs within `grid`
-// (n 16, N 200, FP64: 7.09 us on a cluster of 16, 5.71 on 32 CTAs; N 100: 4.72 and 5.76). Batches
-// larger than the SMs take the fewest CTAs that hold an instance.
+// With item_scale = 0 one CTA as long as its threads stay within `one`: in FP32 what the kernel with a
+// deciding warp holds (n 6, N 60: 0.83 us per iteration on one CTA of 384 threads, 1.13 on two), in
+// FP64 four warps, one per scheduler, because a fifth queues for the FP64 pipe (n 6, N 60: 8.0 us on
+// one CTA, 3.3 on four; N 20, four warps: 3.03 on one and on two). Else the smallest cluster whose CTAs
+// stay within `few` threads (FP32, n 16, N 50: 1.25 us with 256 threads, 1.19 with 160, 1.18 with 96),
+// the cluster of 16 within `most`, and beyond that (FP64, whose iterations are long enough to pay for
+// an exchange through global memory, or instances that no cluster holds) the fewest CTAs within
+// `grid` (n 16, N 200, FP64: 7.15 us on a cluster of 16, 4.93 on 32 CTAs; N 100: 4.67 on the cluster).
+// Batches larger than the SMs take the fewest CTAs that hold an instance.
 static RegLaunch choose_reg(int item_scale, int batch, const int *nx, const int *nu, const int *N,
                             int precision, int nsm) {
   const bool f32 = precision == 0;
-  const int one = f32 ? 320 : 128, few = f32 ? 160 : 128, most = f32 ? 1024 : 160, grid = f32 ? 512 : 160;
+  const int one = f32 ? 480 : 128, few = f32 ? 160 : 128, most = f32 ? 1024 : 160, grid = f32 ? 512 : 160;
   RegLaunch best;
   for (int cand : {1, 2, 4, 8, 16, 24, 32, 48, 64, 80, 96}) {
     if (item_scale > 0 && cand != item_scale) continue;

@@ -25,9 +25,12 @@
 // FP64 is bound by its pipe (a warp issues one FP64 instruction per 64 cycles, an SM one per 19),
 // so the FP64 code counts instructions: one chain per dot product, with the sums around it folded
 // into its start; x / 3 as two operations; the clamp on bit patterns.
+// What is left of an exchange and a decision (about 2000 cycles in a cluster of 16, half of an FP32
+// iteration) runs beside the next iteration, in a warp of its own (spec_kernel).
 // Per iteration, measured, against the shared-memory kernel of admm_res.cu (which keeps the
-// instances with n > 16): plain LTI n 6, N 20, FP64 7.9 -> 3.2 us; quadrotor n 16, N 200 FP32
-// 6.8 -> 1.8 us, FP64 18.6 -> 5.7 us; CSTR n 3, N 5000 FP32 22.8 -> 3.2 us, FP64 102 -> 5.9 us.
+// instances with n > 16) and, in brackets, without the deciding warp: plain LTI n 6, N 20, FP64
+// 7.9 -> 3.0 us (3.2); quadrotor n 16, N 200 FP32 6.8 -> 1.26 us (1.80), FP64 18.6 -> 4.9 us (5.6);
+// CSTR n 3, N 5000 FP32 22.8 -> 1.80 us (2.59), FP64 102 -> 4.1 us (5.9).
 #pragma once
 #include <cooperative_groups.h>
 #include <algorithm>
@@ -55,15 +58,21 @@ constexpr long long kWaitCycles = 1ll << 31;  // ... and cycles at an mbarrier (
 // launch that exchange through global memory.
 enum { kCta = 0, kCluster = 1, kGrid = 2 };
 
-// How c is found: by every warp alike; by warp 0 alone, the others reading it (kSolo: with many
-// warps their integer sums take longer than one more barrier); or not before the last iteration
-// (kLazy: the plain iteration with a fixed count, where no decision depends on it but that a
+// kSpec: a warp of its own finds c and takes the decisions while the others run the next iteration
+// on the hats that a momentum step would give (latency: CTAs that have an SM each). kSolo: warp 0
+// finds c between two iterations (batches that crowd the SMs). kLazy: c is not formed before the last
+// iteration (the plain iteration with a fixed count, where no decision depends on it but that a
 // non-finite c ends the solve, so a share that is non-finite or near overflow has it formed).
-enum { kEach = 0, kSolo = 1, kLazy = 2 };
+enum { kSpec = 0, kSolo = 1, kLazy = 2 };
 
 // Threads of one CTA by the register bound: 4 n-vectors of matrix rows per thread.
 __host__ __device__ constexpr int reg_max_threads(int tsize, int NM) {
   return tsize == 4 ? (NM <= 4 ? 1024 : 512) : (NM <= 4 ? 512 : (NM <= 8 ? 512 : 256));
+}
+
+// With the deciding warp (kSpec), whose iterations have an SM to themselves: FP64 keeps more registers.
+__host__ __device__ constexpr int spec_max_threads(int tsize, int NM) {
+  return tsize == 4 ? reg_max_threads(tsize, NM) : 256;
 }
 
 struct RegPlan {
@@ -189,68 +198,59 @@ __device__ __forceinline__ bool get_halo(const ulonglong2 *p, int n, int c, unsi
   return false;
 }
 
-// Data of the cluster and grid exchanges in shared memory.
+// Data of the exchanges in shared memory.
 template <typename T>
 struct Shared {
   ulonglong2 share[2][16];      // cluster: shares of c by parity (sig, e)
   ulonglong2 warp[32];          // warp sums (sig, e)
   T land[2][2][3][kMaxN];       // cluster: boundary iterates by parity and side
-  unsigned long long bar[2];    // cluster: mbarriers by parity
-  double cn;                    // c / rho, as found by warp 0
+  unsigned long long bar[2];    // cluster: mbarriers by parity: boundary iterates (and shares)
+  unsigned long long sbar[2];   // cluster, kSpec: mbarriers by parity: shares
+  double cn;                    // kSolo: c / rho, as found by warp 0
+  T fnext;                      // kSpec: the decision: momentum factor of the iteration after the
+  int stop, take, use_next;     // next, stop, momentum step (else restart), whether fnext applies
   int fail;                     // a wait gave up
 };
 
-template <typename T, int NM, int SC, int kMode, int kMinCtas>
-__global__ void __launch_bounds__(reg_max_threads((int)sizeof(T), NM), kMinCtas)
-    reg_kernel(Args<T> a, RegPlan pl) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ Shared<T> sh;
-  const int C = SC == kCta ? 1 : pl.C;
-  const int r = SC == kCta ? 0 : (int)(blockIdx.x % C);  // the rank in the cluster: C divides grid
-  const int j = blockIdx.x / C;
-  const int tid = threadIdx.x, nthreads = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  const int nw = nthreads >> 5;
-  const int nx = a.L.nx[j], nu = a.L.nu[j], N = a.L.N[j], n = nx + nu;
-  const int nv = reg_nv(n, (int)sizeof(T));
-  const int k0 = (int)((int64_t)r * N / C), k1 = (int)((int64_t)(r + 1) * N / C);
-  const int kb = k0 - (r > 0 ? 1 : 0);                       // stage of slot 0
-  const int ke = k1 + (k1 < N ? 1 : 0);                      // one past the last slot's stage
-  const int slot = tid / n, c = tid - slot * n, k = kb + slot;
-  const bool active = k < ke;
-  const bool owned = active && k >= k0 && k < k1;
-  const bool has_h = active && k < k1;                       // owned, or the stage before them
-  const bool more = k + 1 < N;
-  T *sW = reinterpret_cast<T *>(smem_raw), *sY = sW + pl.region, *sH = sY + pl.region,
-    *sX = sH + pl.region;                                    // sX: row q = xbar_{kb + q}
-  for (int i = tid; i < 4 * pl.region; i += nthreads) sW[i] = (T)0;
-  if (tid < 32) sh.warp[tid] = make_ulonglong2(0, (unsigned long long)(long long)detsum::kZero);
-  if (tid == 0) {
-    sh.fail = 0;
-    if (SC == kCluster) {
-      for (int p = 0; p < 2; ++p)
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&sh.bar[p])));
-      asm volatile("fence.mbarrier_init.release.cluster;");
-    }
-  }
-
-  // ---- the thread's rows and columns, once ----
+// One thread's component of one stage: its matrix rows, its iterate and the one before.
+template <typename T, int NM>
+struct Lane {
   T Gn[NM], Gr[NM], Hr[NM], Pr[NM];
+  T zc, vc, tc, bc, zp, vp, tp, bp;
+  T ee, qref, lo, hi, rho;
+  int nx, n, nv, slot, c, k, k0, k1;
+  bool active, owned, has_h, more, below, above;  // below / above: a CTA of the instance on that side
+
+  __device__ __forceinline__ void setup(const Args<T> &a, int warm, int j, int r, int C, int tid) {
+    const int nu = a.L.nu[j], N = a.L.N[j];
+    nx = a.L.nx[j];
+    n = nx + nu;
+    nv = reg_nv(n, (int)sizeof(T));
+    k0 = (int)((int64_t)r * N / C);
+    k1 = (int)((int64_t)(r + 1) * N / C);
+    below = r > 0;
+    above = k1 < N;
+    slot = tid / n;
+    c = tid - slot * n;
+    k = k0 - (below ? 1 : 0) + slot;            // slot 0 is the stage before the CTA's, if any
+    active = k < k1 + (above ? 1 : 0);          // the last slot the stage after them
+    owned = active && k >= k0 && k < k1;
+    has_h = active && k < k1;                   // owned, or the stage before them
+    more = k + 1 < N;
 #pragma unroll
-  for (int q = 0; q < NM; ++q) Gn[q] = Gr[q] = Hr[q] = Pr[q] = (T)0;
-  T zc = 0, vc = 0, tc = 0, bc = 0, zp = 0, vp = 0, tp = 0, bp = 0;  // iterate, and the one before
-  T ee = 0, qref = 0, lo = 0, hi = 0;
-  const T rho = (T)a.rho;
-  const int n5p = ls::iter_stride_plain(n, (int)sizeof(T));
-  T *const gits = a.it[a.base[j]] + a.L.Ni[j];
-  if (active) {
+    for (int q = 0; q < NM; ++q) Gn[q] = Gr[q] = Hr[q] = Pr[q] = (T)0;
+    zc = vc = tc = bc = zp = vp = tp = bp = (T)0;
+    ee = qref = lo = hi = (T)0;
+    rho = (T)a.rho;
+    if (!active) return;
     const int lti = a.L.lti, W = a.L.W[j], ldg = odd_ld(n);
     const int oE = nx * ldg, oH = oE + nx, oM = oH + wrapped_size(n);
     const T *blk = a.blk + a.L.blk[j];
     const T *Gk = blk + (lti ? 0 : (int64_t)k * W);
     const T *Gk1 = lti ? blk : Gk + W;
     const T *Hk = (lti ? blk + (more ? 0 : W) : Gk) + oH;
-    if (pl.warm != 0) {  // the previous solve's iterate, shifted by a stage for warm == 2
-      const T *git = gits + (int64_t)(pl.warm == 2 && more ? k + 1 : k) * n5p;
+    if (warm != 0) {  // the previous solve's iterate, shifted by a stage for warm == 2
+      const T *git = iterates(a, j) + (int64_t)(warm == 2 && more ? k + 1 : k) * stride();
       zc = git[c];
       vc = git[n + c];
       tc = git[2 * n + c];
@@ -289,41 +289,21 @@ __global__ void __launch_bounds__(reg_max_threads((int)sizeof(T), NM), kMinCtas)
       }
     }
   }
-  double cval = 0.0, cbest = INFINITY;
-  double etac = a.eta;  // eta times the last c (1 at the start), formed off the critical path
-  int itbest = 0, itfirst = -1, streak = 0, momentum = 0, status = kMaxIter, iters = 0;
-  T f = (T)0;
-  bool use_prev = false;
-  const double eps = a.eps;
-  const bool unit_rho = a.rho == 1.0, watch = a.stall_win > 0 || a.mask != nullptr;
-  constexpr bool solo = kMode == kSolo, lazy = kMode == kLazy;
-  ulonglong2 *xs = nullptr, *xh = nullptr;  // grid: this instance's share and halo records
-  if (SC == kGrid) {
-    xs = pl.xch + (size_t)j * xch_records(C);
-    xh = xs + 2 * C;
-  }
-  const unsigned my_bytes =
-      SC == kCluster ? (unsigned)(16 * C + (int)sizeof(T) * n * ((r > 0 ? 2 : 0) + (k1 < N ? 3 : 0))) : 0;
-  __syncthreads();
-  if (r == 0 && tid < n) sX[tid] = a.xb0[a.L.off_n[j] + tid];
-  if (SC == kCluster) cg::this_cluster().sync();  // every mbarrier is ready
-  else __syncthreads();
 
-  for (int it = 0; it < a.max_iters; ++it) {
-    const int par = it & 1;
-    const unsigned tag = (unsigned)it + 1;
-    if (SC == kCluster && tid == 0)
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&sh.bar[par])),
-                   "r"(my_bytes)
-                   : "memory");
-    // the momentum factor this iteration's decision would take, fetched ahead
-    double ctab = 0.0;
-    if (!lazy)
-      asm volatile("ld.global.f64 %0, [%1];" : "=d"(ctab) : "l"(a.coef_tab + (a.accel ? streak : 0)));
-    const T fnext = lazy ? (T)0 : (T)ctab;
+  __device__ __forceinline__ int stride() const { return ls::iter_stride_plain(n, (int)sizeof(T)); }
+  __device__ __forceinline__ T *iterates(const Args<T> &a, int j) const {
+    return a.it[a.base[j]] + a.L.Ni[j];
+  }
+
+  // Steps 1-4 with hats cur + f (cur - prev) (momentum) or cur: the new iterate of an owned component
+  // and its share of c. sW, sY, sH, sX: the CTA's vectors (sX: row q = xbar of slot q); sync: a barrier
+  // of its threads, after which earlier reads of the vectors are over.
+  template <typename Sync>
+  __device__ __forceinline__ void iterate(T *sW, T *sY, T *sH, T *sX, T f, bool momentum, Sync sync, T &zn,
+                                          T &vn, T &tn, T &bn, T &cacc) {
     // ---- hats, y, w ----
     T zh = zc, vh = vc, th = tc, bh = bc;
-    if (!lazy && use_prev) {
+    if (momentum) {
       zh = zc + f * (zc - zp);
       vh = vc + f * (vc - vp);
       th = tc + f * (tc - tp);
@@ -334,10 +314,9 @@ __global__ void __launch_bounds__(reg_max_threads((int)sizeof(T), NM), kMinCtas)
       sW[slot * nv + c] = vh - bh;
       sY[slot * nv + c] = (zh - vh) - be;
     }
-    __syncthreads();
-    if (SC != kCta && sh.fail) break;  // set before this barrier, if at all: uniform
-    // ---- Abar_{k+1}^T y_{k+1}, h_k; p = beta + P_k w_k ----
-    T p = (T)0;
+    sync();
+    // ---- Abar_{k+1}^T y_{k+1}, h_k; Bbar du = P_k w_k ----
+    T bd = (T)0;
     if (has_h) {
       const T *y = sY + (slot + 1) * nv;
       T acc = zh - th;
@@ -347,139 +326,102 @@ __global__ void __launch_bounds__(reg_max_threads((int)sizeof(T), NM), kMinCtas)
       }
       sH[slot * nv + c] = qref + rho * acc;
     }
-    if (owned) p = dot(Pr, sW + slot * nv, n, bh);
-    __syncthreads();
+    if (owned) bd = dot(Pr, sW + slot * nv, n, (T)0);
+    sync();
     // ---- xbar_{k+1} = H_k h_k ----
     T xb = (T)0;
     if (has_h) {
       xb = dot(Hr, sH + slot * nv, n, (T)0);
       sX[(slot + 1) * nv + c] = xb;
     }
-    __syncthreads();
+    sync();
     // ---- steps 2-4 ----
-    T cacc = (T)0;
-    T zn = (T)0, vn = (T)0, tn = (T)0, bn = (T)0;
+    cacc = (T)0;
+    zn = vn = tn = bn = (T)0;
     if (owned) {
       const T q = dot(Gr, sX + slot * nv, n, be);  // Abar xbar + ebar - lambda
-      const T s = xb + th;
+      const T s = xb + th, p = bh + bd;
       const T w = third((T)2 * s + (p + q));
       zn = clamp(w, lo, hi);
       vn = (T)0.5 * (zn + (p - q));
       tn = s - zn;
       bn = p - vn;
-      if (SC == kCluster) {  // boundary iterates: the first stage to CTA r - 1, the last to r + 1
-        if (k == k0 && r > 0) {
-          const unsigned bar = remote(smem_addr(&sh.bar[par]), r - 1);
-          const unsigned d = remote(smem_addr(&sh.land[par][1][0][c]), r - 1);
-          push(d, bar, zn);
-          push(d + kMaxN * sizeof(T), bar, vn);
-          push(d + 2 * kMaxN * sizeof(T), bar, bn);
-        }
-        if (k == k1 - 1 && k1 < N) {
-          const unsigned bar = remote(smem_addr(&sh.bar[par]), r + 1);
-          const unsigned d = remote(smem_addr(&sh.land[par][0][0][c]), r + 1);
-          push(d, bar, zn);
-          push(d + kMaxN * sizeof(T), bar, tn);
-        }
-      }
-      if (SC == kGrid) {
-        if (k == k0 && r > 0)
-          put_halo(xh + ((size_t)(par * C + r - 1) * 2 + 1) * kHaloRecs, n, c, tag, zn, vn, bn);
-        if (k == k1 - 1 && k1 < N)
-          put_halo(xh + (size_t)(par * C + r + 1) * 2 * kHaloRecs, n, c, tag, zn, tn, (T)0);
-      }
-      const T d1 = tn - th, d2 = bn - bh, d4 = zn - zh, d5 = vn - vh;
+      // theta' - theta = xbar - z' and beta' - beta = Bbar du - v', without the duals' own rounding
+      const T d1 = xb - zn, d2 = bd - vn, d4 = zn - zh, d5 = vn - vh;
       // d1^2 + d2^2 + d3^2 + d4^2 + d5^2 + (d4 - d5)^2 with d3 = -d2
       const T g = d2 * d2 + (d4 * d4 + d5 * (d5 - d4));
       cacc = (T)2 * g + d1 * d1;
     }
-    // ---- the exchange: shares of c and boundary iterates ----
-    double cn = 0.0;
-    if (lazy && it + 1 < a.max_iters && !__syncthreads_or(detsum::may_overflow(cacc))) {
-      zc = zn; vc = vn; tc = tn; bc = bn;
-      continue;
+  }
+
+  // Cluster: the first stage's new iterate to CTA r - 1, the last one's to CTA r + 1.
+  __device__ __forceinline__ void push_boundary(Shared<T> &sh, int par, int r, T zn, T vn, T tn, T bn) const {
+    if (owned && k == k0 && below) {
+      const unsigned bar = remote(smem_addr(&sh.bar[par]), r - 1);
+      const unsigned d = remote(smem_addr(&sh.land[par][1][0][c]), r - 1);
+      push(d, bar, zn);
+      push(d + kMaxN * sizeof(T), bar, vn);
+      push(d + 2 * kMaxN * sizeof(T), bar, bn);
     }
-    detsum::Fx sum = detsum::warp_sum(cacc);
-    if (nw > 1) {
-      if (lane == 0) sh.warp[warp] = make_ulonglong2(sum.sig, (unsigned long long)(long long)sum.e);
-      __syncthreads();
-      if ((SC == kCta && !solo) || warp == 0) {
-        const ulonglong2 t = sh.warp[lane];  // {0, kZero} beyond the CTA's warps
-        sum = detsum::warp_sum(detsum::Fx{t.x, (int)t.y});
-      }
+    if (owned && k == k1 - 1 && above) {
+      const unsigned bar = remote(smem_addr(&sh.bar[par]), r + 1);
+      const unsigned d = remote(smem_addr(&sh.land[par][0][0][c]), r + 1);
+      push(d, bar, zn);
+      push(d + kMaxN * sizeof(T), bar, tn);
     }
-    if (SC == kCluster) {
-      if (warp == 0 && lane < C)
-        push(remote(smem_addr(&sh.share[par][r]), lane), remote(smem_addr(&sh.bar[par]), lane), sum);
-      if (!solo || warp == 0) {
-        if (!bar_wait(smem_addr(&sh.bar[par]), (unsigned)(it >> 1) & 1u)) sh.fail = 1;
-        detsum::Fx t{0ull, detsum::kZero};
-        if (lane < C) {
-          const ulonglong2 q = sh.share[par][lane];
-          t = detsum::Fx{q.x, (int)q.y};
-        }
-        sum = detsum::warp_sum(t);
-      }
-    }
-    if (SC == kGrid) {
-      if (warp == 0) {
-        if (lane == 0) put_rec(xs + par * C + r, sum.sig, with_tag((unsigned)sum.e, tag));
-        detsum::Fx t[3];  // C <= 96 shares, three per lane, all in flight
-        bool ok = false;
-        for (int n_ = 0; n_ < kWaitPolls && !ok; ++n_) {
-          bool mine = true;
-#pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            unsigned long long b = with_tag((unsigned)detsum::kZero, tag);
-            t[q].sig = 0;
-            if (lane + 32 * q < C) get_rec(xs + par * C + lane + 32 * q, t[q].sig, b);
-            t[q].e = (int)(unsigned)b;
-            mine = mine && (unsigned)(b >> 32) == tag;
-          }
-          ok = __all_sync(0xffffffffu, mine);
-        }
-        if (!ok && lane == 0) sh.fail = 1;
-        sum = detsum::warp_sum(t[0]);
-        if (C > 32) {
-          const detsum::Fx s1 = detsum::warp_sum(t[1]), s2 = detsum::warp_sum(t[2]);
-          sum = detsum::warp_sum(lane == 0 ? sum : lane == 1 ? s1 : lane == 2 ? s2
-                                                                  : detsum::Fx{0ull, detsum::kZero});
-        }
-      }
-      if (active && !owned) {  // boundary iterates of the neighbours
-        T x, y, w;
-        const bool before = k < k0;
-        if (!get_halo(xh + ((size_t)(par * C + r) * 2 + (before ? 0 : 1)) * kHaloRecs, n, c, tag, x, y, w))
-          sh.fail = 1;
-        zn = x;
-        if (before) {
-          tn = y;
-        } else {
-          vn = y;
-          bn = w;
-        }
-      }
-    }
-    if (SC == kGrid || solo) {
-      if (warp == 0) cn = detsum::to_double(sum);
-      if (tid == 0) sh.cn = cn;
-      __syncthreads();
-      cn = sh.cn;
+  }
+  __device__ __forceinline__ unsigned boundary_bytes() const {
+    return (unsigned)((int)sizeof(T) * n * ((below ? 2 : 0) + (above ? 3 : 0)));
+  }
+  // Cluster: what the neighbours pushed, for the slots of their stages.
+  __device__ __forceinline__ void land(const Shared<T> &sh, int par, T &zn, T &vn, T &tn, T &bn) const {
+    const T *d = &sh.land[par][k < k0 ? 0 : 1][0][c];
+    zn = d[0];
+    if (k < k0) {
+      tn = d[kMaxN];
     } else {
-      cn = detsum::to_double(sum);
+      vn = d[kMaxN];
+      bn = d[2 * kMaxN];
     }
-    // ---- steps 5-7, by every thread alike ----
-    if (!unit_rho) cn *= a.rho;
+  }
+
+  // The current iterate to the solver's buffer, and the outputs.
+  __device__ __forceinline__ void store(const Args<T> &a, const RegPlan &pl, int j) const {
+    if (!owned) return;
+    T *git = iterates(a, j) + (int64_t)k * stride();
+    git[c] = zc;
+    git[n + c] = vc;
+    git[2 * n + c] = tc;
+    git[3 * n + c] = bc;
+    git[4 * n + c] = -bc;
+    if (c < nx) {
+      if (pl.x_out) pl.x_out[a.L.Nnx[j] + (int64_t)k * nx + c] = (double)zc;
+    } else if (pl.u_out) {
+      pl.u_out[a.L.Nnu[j] + (int64_t)k * (n - nx) + (c - nx)] = (double)zc;
+    }
+  }
+};
+
+// Steps 5-7 of one instance: the stop tests and the momentum decision, from c^{i+1}.
+struct Decider {
+  double cval = 0.0, cbest = INFINITY, etac;  // etac: eta times the last c (1 at the start)
+  double eps, rho;
+  int itbest = 0, itfirst = -1, streak = 0, momentum = 0, status = kMaxIter, iters = 0;
+  bool unit_rho, watch;
+
+  template <typename T>
+  __device__ __forceinline__ explicit Decider(const Args<T> &a)
+      : etac(a.eta), eps(a.eps), rho(a.rho), unit_rho(a.rho == 1.0),
+        watch(a.stall_win > 0 || a.mask != nullptr) {}
+
+  // c from the sum of the shares: the stop flag, and whether the next hats take the momentum step.
+  template <typename T>
+  __device__ __forceinline__ bool step(const Args<T> &a, int j, int it, double cn, bool &take) {
+    if (!unit_rho) cn *= rho;
     cval = cn;
     iters = it + 1;
-    bool stop = false, take;
-    if (lazy) {  // here on the last iteration, or for a c that may not be finite
-      take = false;
-      stop = it + 1 >= a.max_iters;
-      if (!detsum::finite(cn)) {
-        status = kNonFinite; stop = true;
-      }
-    } else if (detsum::le_nonneg(cn, eps) || !detsum::finite(cn) || it + 1 >= a.max_iters || watch) {
+    bool stop = false;
+    if (detsum::le_nonneg(cn, eps) || !detsum::finite(cn) || it + 1 >= a.max_iters || watch) {
       take = false;
       if (!detsum::finite(cn)) {
         status = kNonFinite; stop = true;
@@ -505,49 +447,23 @@ __global__ void __launch_bounds__(reg_max_threads((int)sizeof(T), NM), kMinCtas)
     } else {
       take = a.accel && detsum::le_nonneg(cn, etac);
     }
-    if (!lazy) {
-      // (alpha_m - 1) / alpha_{m+1}, alpha_0 = 1, from the precomputed table; 0 after a restart
-      use_prev = take && streak > 0;
-      momentum += use_prev;
-      f = take ? fnext : (T)0;
-      streak = take ? streak + 1 : 0;
-      etac = a.eta * cn;
-    }
-    // ---- the new iterate becomes the current one; halo slots take theirs from the landing ----
-    if (SC == kCluster && active && !owned) {
-      const T *d = &sh.land[par][k < k0 ? 0 : 1][0][c];
-      zn = d[0];
-      if (k < k0) {
-        tn = d[kMaxN];
-      } else {
-        vn = d[kMaxN];
-        bn = d[2 * kMaxN];
-      }
-    }
-    if (!lazy) {
-      zp = zc; vp = vc; tp = tc; bp = bc;
-    }
-    zc = zn; vc = vn; tc = tn; bc = bn;
-    if (stop) break;
+    etac = a.eta * cn;
+    momentum += take && streak > 0;
+    streak = take ? streak + 1 : 0;
+    return stop;
   }
-  if (SC != kCta) {
-    __syncthreads();
-    if (sh.fail) status = kTimeout;
+
+  // The momentum factor (alpha_m - 1) / alpha_{m+1}, alpha_0 = 1, after m momentum steps in a row,
+  // from the precomputed table: loaded here and not where it is used.
+  template <typename T>
+  __device__ __forceinline__ double factor(const Args<T> &a, int m) const {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(a.coef_tab + (a.accel ? m : 0)));
+    return v;
   }
-  if (owned) {
-    T *git = gits + (int64_t)k * n5p;
-    git[c] = zc;
-    git[n + c] = vc;
-    git[2 * n + c] = tc;
-    git[3 * n + c] = bc;
-    git[4 * n + c] = -bc;
-    if (c < nx) {
-      if (pl.x_out) pl.x_out[a.L.Nnx[j] + (int64_t)k * nx + c] = (double)zc;
-    } else if (pl.u_out) {
-      pl.u_out[a.L.Nnu[j] + (int64_t)k * nu + (c - nx)] = (double)zc;
-    }
-  }
-  if (r == 0 && tid == 0) {
+
+  template <typename T>
+  __device__ __forceinline__ void store(const Args<T> &a, int j) const {
     InstState s;
     s.iters = iters;
     s.status = a.ferr && a.ferr[j] ? kFactorFailed : status;
@@ -557,6 +473,283 @@ __global__ void __launch_bounds__(reg_max_threads((int)sizeof(T), NM), kMinCtas)
     a.st[j] = s;
     a.stop[j] = 1;
   }
+};
+
+__device__ __forceinline__ ulonglong2 packed(detsum::Fx t) {
+  return make_ulonglong2(t.sig, (unsigned long long)(long long)t.e);
+}
+__device__ __forceinline__ detsum::Fx unpacked(ulonglong2 q) { return detsum::Fx{q.x, (int)q.y}; }
+
+// Zeroes the vectors, sets up the mbarriers and xbar_0 (every thread of the CTA).
+template <typename T, int SC>
+__device__ __forceinline__ void start_cta(const Args<T> &a, const RegPlan &pl, Shared<T> &sh, T *vec, T *sX,
+                                          int j, int r, int n) {
+  const int tid = threadIdx.x;
+  for (int i = tid; i < 4 * pl.region; i += blockDim.x) vec[i] = (T)0;
+  if (tid < 32) sh.warp[tid] = make_ulonglong2(0, (unsigned long long)(long long)detsum::kZero);
+  if (tid == 0) {
+    sh.fail = 0;
+    if (SC == kCluster) {
+      for (int p = 0; p < 2; ++p) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&sh.bar[p])));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&sh.sbar[p])));
+      }
+      asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+  }
+  __syncthreads();
+  if (r == 0 && tid < n) sX[tid] = a.xb0[a.L.off_n[j] + tid];
+  if (SC == kCluster) cg::this_cluster().sync();  // every mbarrier is ready
+  else __syncthreads();
+}
+
+__device__ __forceinline__ void expect(unsigned long long *bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
+               : "memory");
+}
+template <int kId>
+__device__ __forceinline__ void named_sync(int threads) {
+  asm volatile("bar.sync %0, %1;" ::"n"(kId), "r"(threads) : "memory");
+}
+template <int kId>
+__device__ __forceinline__ void named_arrive(int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"n"(kId), "r"(threads) : "memory");
+}
+
+// kSpec. The last warp of the CTA decides, the others iterate. Iteration i's warp sums are handed to the
+// decider, which sums them, exchanges shares with the other CTAs, takes the decision and hands it
+// back; meanwhile the others run iteration i + 1 on the hats that a momentum step would give, the
+// factor of which is known an iteration ahead. At its end they learn the decision of i: stop (the
+// iteration in hand is dropped), momentum (it stands), restart (it is run again on hats equal to the
+// iterates, unless it was without momentum anyway). Only then its boundary iterates and sums leave
+// the CTA, so a CTA is never more than one iteration ahead of another, which two buffers by parity
+// allow for.
+template <typename T, int NM, int SC>
+__global__ void __launch_bounds__(spec_max_threads((int)sizeof(T), NM), 1) spec_kernel(Args<T> a, RegPlan pl) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ Shared<T> sh;
+  const int C = SC == kCta ? 1 : pl.C;
+  const int r = SC == kCta ? 0 : (int)(blockIdx.x % C);  // the rank in the cluster: C divides grid
+  const int j = blockIdx.x / C;
+  const int all = blockDim.x, nct = all - 32;            // threads, and those that iterate
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = nct >> 5;
+  const bool decides = warp == nw;
+  T *sW = reinterpret_cast<T *>(smem_raw), *sY = sW + pl.region, *sH = sY + pl.region, *sX = sH + pl.region;
+  ulonglong2 *xs = nullptr, *xh = nullptr;  // grid: this instance's share and halo records
+  if (SC == kGrid) {
+    xs = pl.xch + (size_t)j * xch_records(C);
+    xh = xs + 2 * C;
+  }
+  start_cta<T, SC>(a, pl, sh, sW, sX, j, r, a.L.nx[j] + a.L.nu[j]);
+
+  if (decides) {
+    Decider d(a);
+    for (int it = 0;; ++it) {
+      const int par = it & 1;
+      const unsigned tag = (unsigned)it + 1;
+      if (SC == kCluster && lane == 0) expect(&sh.sbar[par], (unsigned)(16 * C));
+      const T fmore = (T)d.factor(a, d.streak + 1);
+      named_sync<2>(all);  // the warp sums of iteration it
+      bool ok = SC == kCta || *(volatile int *)&sh.fail == 0;
+      detsum::Fx sum = unpacked(sh.warp[nw == 1 ? 0 : lane]);  // {0, kZero} beyond the CTA's warps
+      if (nw > 1) sum = detsum::warp_sum(sum);
+      if (SC == kCluster && ok) {
+        if (lane < C)
+          push(remote(smem_addr(&sh.share[par][r]), lane), remote(smem_addr(&sh.sbar[par]), lane), sum);
+        ok = __all_sync(0xffffffffu, bar_wait(smem_addr(&sh.sbar[par]), (unsigned)(it >> 1) & 1u));
+        sum = detsum::warp_sum(lane < C ? unpacked(sh.share[par][lane]) : detsum::Fx{0ull, detsum::kZero});
+      }
+      if (SC == kGrid && ok) {
+        if (lane == 0) put_rec(xs + par * C + r, sum.sig, with_tag((unsigned)sum.e, tag));
+        detsum::Fx t[3];  // C <= 96 shares, three per lane, all in flight
+        ok = false;
+        for (int n_ = 0; n_ < kWaitPolls && !ok; ++n_) {
+          bool mine = true;
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            unsigned long long b = with_tag((unsigned)detsum::kZero, tag);
+            t[q].sig = 0;
+            if (lane + 32 * q < C) get_rec(xs + par * C + lane + 32 * q, t[q].sig, b);
+            t[q].e = (int)(unsigned)b;
+            mine = mine && (unsigned)(b >> 32) == tag;
+          }
+          ok = __all_sync(0xffffffffu, mine);
+        }
+        sum = detsum::warp_sum(t[0]);
+        if (C > 32) {
+          const detsum::Fx s1 = detsum::warp_sum(t[1]), s2 = detsum::warp_sum(t[2]);
+          sum = detsum::warp_sum(lane == 0 ? sum : lane == 1 ? s1 : lane == 2 ? s2
+                                                                  : detsum::Fx{0ull, detsum::kZero});
+        }
+      }
+      bool take = false;
+      bool stop = d.step(a, j, it, detsum::to_double(sum), take);
+      if (!ok) {  // a wait gave up, here or at a boundary: nothing leaves this CTA any more
+        stop = true;
+        d.status = kTimeout;
+      }
+      if (lane == 0) {
+        sh.stop = stop;
+        sh.take = take;
+        sh.fnext = take ? fmore : (T)0;
+        sh.use_next = take;  // after a restart the next factor is 0
+        if (!ok) sh.fail = 1;
+      }
+      __syncwarp();
+      named_arrive<3>(all);  // the decision of iteration it
+      if (stop) break;
+    }
+    if (r == 0 && lane == 0) d.store(a, j);
+  } else {
+    Lane<T, NM> L;
+    L.setup(a, pl.warm, j, r, C, tid);
+    auto sync = [&]() { named_sync<1>(nct); };
+    sync();
+    T f = (T)0;
+    bool momentum = false;
+    for (int it = 0;; ++it) {
+      const int par = it & 1, last = par ^ 1;
+      const unsigned tag = (unsigned)it + 1;
+      if (SC == kCluster && tid == 0) expect(&sh.bar[par], L.boundary_bytes());
+      if (SC != kCta && it > 0 && L.active && !L.owned) {  // the neighbours' iterate of it - 1
+        T zn = (T)0, vn = (T)0, tn = (T)0, bn = (T)0;
+        if (SC == kCluster) {
+          if (!bar_wait(smem_addr(&sh.bar[last]), (unsigned)((it - 1) >> 1) & 1u)) sh.fail = 1;
+          L.land(sh, last, zn, vn, tn, bn);
+        } else {
+          T x, y, w;
+          const bool before = L.k < L.k0;
+          if (!get_halo(xh + ((size_t)(last * C + r) * 2 + (before ? 0 : 1)) * kHaloRecs, L.n, L.c, tag - 1, x, y, w)) {
+            sh.fail = 1;
+            x = y = w = (T)0;
+          }
+          zn = x;
+          if (before) {
+            tn = y;
+          } else {
+            vn = y;
+            bn = w;
+          }
+        }
+        L.zp = L.zc; L.vp = L.vc; L.tp = L.tc; L.bp = L.bc;
+        L.zc = zn; L.vc = vn; L.tc = tn; L.bc = bn;
+      }
+      T zn, vn, tn, bn, cacc;
+      T fnext = (T)0;
+      bool mnext = false;
+      if (it < a.max_iters) {
+        L.iterate(sW, sY, sH, sX, f, momentum, sync, zn, vn, tn, bn, cacc);
+      }
+      if (it > 0) {
+        named_sync<3>(all);  // the decision of it - 1
+        if (*(volatile int *)&sh.stop) break;
+        fnext = *(volatile T *)&sh.fnext;
+        mnext = *(volatile int *)&sh.use_next != 0;
+        if (momentum && !*(volatile int *)&sh.take)
+          L.iterate(sW, sY, sH, sX, (T)0, false, sync, zn, vn, tn, bn, cacc);
+      }
+      if (SC == kCta || *(volatile int *)&sh.fail == 0) {
+        if (SC == kCluster) L.push_boundary(sh, par, r, zn, vn, tn, bn);
+        if (SC == kGrid && L.owned) {
+          if (L.k == L.k0 && L.below)
+            put_halo(xh + ((size_t)(par * C + r - 1) * 2 + 1) * kHaloRecs, L.n, L.c, tag, zn, vn, bn);
+          if (L.k == L.k1 - 1 && L.above)
+            put_halo(xh + (size_t)(par * C + r + 1) * 2 * kHaloRecs, L.n, L.c, tag, zn, tn, (T)0);
+        }
+      }
+      const detsum::Fx sum = detsum::warp_sum(cacc);
+      if (lane == 0) sh.warp[warp] = packed(sum);
+      named_arrive<2>(all);
+      if (L.owned) {
+        L.zp = L.zc; L.vp = L.vc; L.tp = L.tc; L.bp = L.bc;
+        L.zc = zn; L.vc = vn; L.tc = tn; L.bc = bn;
+      }
+      f = fnext;
+      momentum = mnext;
+    }
+    L.store(a, pl, j);
+  }
+  if (SC == kCluster) cg::this_cluster().sync();  // no CTA leaves with a push to it in flight
+}
+
+// kSolo and kLazy: one iteration after the other.
+template <typename T, int NM, int SC, int kMode, int kMinCtas>
+__global__ void __launch_bounds__(reg_max_threads((int)sizeof(T), NM), kMinCtas)
+    reg_kernel(Args<T> a, RegPlan pl) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ Shared<T> sh;
+  constexpr bool lazy = kMode == kLazy;
+  const int C = SC == kCta ? 1 : pl.C;
+  const int r = SC == kCta ? 0 : (int)(blockIdx.x % C);  // the rank in the cluster: C divides grid
+  const int j = blockIdx.x / C;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  T *sW = reinterpret_cast<T *>(smem_raw), *sY = sW + pl.region, *sH = sY + pl.region, *sX = sH + pl.region;
+  start_cta<T, SC>(a, pl, sh, sW, sX, j, r, a.L.nx[j] + a.L.nu[j]);
+  Lane<T, NM> L;
+  L.setup(a, pl.warm, j, r, C, tid);
+  Decider d(a);
+  auto sync = [&]() { __syncthreads(); };
+  sync();
+  T f = (T)0;
+  bool momentum = false;
+  for (int it = 0; it < a.max_iters; ++it) {
+    const int par = it & 1;
+    if (SC == kCluster && tid == 0) expect(&sh.bar[par], (unsigned)(16 * C) + L.boundary_bytes());
+    // the momentum factor this iteration's decision would take, fetched ahead
+    const T fnext = lazy ? (T)0 : (T)d.factor(a, d.streak);
+    T zn, vn, tn, bn, cacc;
+    L.iterate(sW, sY, sH, sX, f, !lazy && momentum, sync, zn, vn, tn, bn, cacc);
+    if (SC != kCta && sh.fail) break;  // set before the iteration's first barrier, if at all: uniform
+    if (SC == kCluster) L.push_boundary(sh, par, r, zn, vn, tn, bn);
+    if (lazy && it + 1 < a.max_iters && !__syncthreads_or(detsum::may_overflow(cacc))) {
+      L.zc = zn; L.vc = vn; L.tc = tn; L.bc = bn;
+      continue;
+    }
+    // ---- c: by warp 0, the others read it (their integer sums take longer than one more barrier) ----
+    detsum::Fx sum = detsum::warp_sum(cacc);
+    if (lane == 0) sh.warp[warp] = packed(sum);
+    __syncthreads();
+    if (warp == 0) {
+      sum = detsum::warp_sum(unpacked(sh.warp[lane]));  // {0, kZero} beyond the CTA's warps
+      if (SC == kCluster) {
+        if (lane < C)
+          push(remote(smem_addr(&sh.share[par][r]), lane), remote(smem_addr(&sh.bar[par]), lane), sum);
+        if (!bar_wait(smem_addr(&sh.bar[par]), (unsigned)(it >> 1) & 1u)) sh.fail = 1;
+        sum = detsum::warp_sum(lane < C ? unpacked(sh.share[par][lane]) : detsum::Fx{0ull, detsum::kZero});
+      }
+      const double cn = detsum::to_double(sum);
+      if (lane == 0) sh.cn = cn;
+    }
+    __syncthreads();
+    const double cn = sh.cn;
+    bool take = false, stop;
+    if (lazy) {  // here on the last iteration, or for a c that may not be finite
+      d.cval = d.unit_rho ? cn : cn * d.rho;
+      d.iters = it + 1;
+      stop = it + 1 >= a.max_iters;
+      if (!detsum::finite(d.cval)) {
+        d.status = kNonFinite; stop = true;
+      }
+    } else {
+      const bool high = d.streak > 0;
+      stop = d.step(a, j, it, cn, take);
+      momentum = take && high;
+      f = take ? fnext : (T)0;
+    }
+    // ---- the new iterate becomes the current one; halo slots take theirs from the landing ----
+    if (SC == kCluster && L.active && !L.owned) L.land(sh, par, zn, vn, tn, bn);
+    if (!lazy) {
+      L.zp = L.zc; L.vp = L.vc; L.tp = L.tc; L.bp = L.bc;
+    }
+    L.zc = zn; L.vc = vn; L.tc = tn; L.bc = bn;
+    if (stop) break;
+  }
+  if (SC != kCta) {
+    __syncthreads();
+    if (sh.fail) d.status = kTimeout;
+  }
+  L.store(a, pl, j);
+  if (r == 0 && tid == 0) d.store(a, j);
   if (SC == kCluster) cg::this_cluster().sync();  // no CTA leaves with a push to it in flight
 }
 
@@ -569,6 +762,13 @@ const void *pick_kernel(int NM, bool crowded) {
   return NM == 4   ? (const void *)reg_kernel<T, 4, SC, kMode, 1>
          : NM == 8 ? (const void *)reg_kernel<T, 8, SC, kMode, 1>
                    : (const void *)reg_kernel<T, 16, SC, kMode, 1>;
+}
+
+template <typename T, int SC>
+const void *pick_spec(int NM) {
+  return NM == 4   ? (const void *)spec_kernel<T, 4, SC>
+         : NM == 8 ? (const void *)spec_kernel<T, 8, SC>
+                   : (const void *)spec_kernel<T, 16, SC>;
 }
 
 // The launch of one solve.
@@ -594,25 +794,24 @@ cudaError_t reg_launch_t(const AdmmLaunch &s, const RegLaunch &rl, cudaStream_t 
   if ((rc = cudaGetDevice(&dev)) != cudaSuccess) return rc;
   if ((rc = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return rc;
   const int cls = reg_class(rl.nmax);
-  // Up to 4 warps (8 in a cluster) find c each by themselves (one CTA, n 6, N 20, FP64: 3.20 us per
-  // iteration, 3.41 by warp 0 alone; cluster of 16, n 16, N 200, FP32: 1.78 and 1.82), more leave it
-  // to warp 0 (CSTR N 5000 FP32, 30 warps: 3.18 and 2.94).
+  // A batch that leaves every CTA an SM runs the deciding warp beside the others; one that does not
+  // has other CTAs to run meanwhile.
   const bool watch = s.stall_win > 0 || s.mask != nullptr;
   const bool lazy = !s.accel && s.eps < 0.0 && !watch;
-  const bool crowded = (int64_t)s.L.batch > nsm;
-  const void *kernel =
-      rl.C == 1 ? (lazy                ? pick_kernel<T, kCta, kLazy>(cls, crowded)
-                   : rl.threads <= 128 ? pick_kernel<T, kCta, kEach>(cls, crowded)
-                                       : pick_kernel<T, kCta, kSolo>(cls, crowded))
-      : rl.C <= 16 ? (rl.threads <= 256 ? pick_kernel<T, kCluster, kEach>(cls, false)
-                                        : pick_kernel<T, kCluster, kSolo>(cls, false))
-                   : pick_kernel<T, kGrid, kSolo>(cls, false);
+  const bool crowded = (int64_t)s.L.batch * rl.C > nsm || rl.threads + 32 > spec_max_threads((int)sizeof(T), cls);
+  const bool spec = rl.C > 16 || (!crowded && !(lazy && rl.C == 1));
+  const void *kernel = spec ? (rl.C == 1    ? pick_spec<T, kCta>(cls)
+                               : rl.C <= 16 ? pick_spec<T, kCluster>(cls)
+                                            : pick_spec<T, kGrid>(cls))
+                       : rl.C > 1 ? pick_kernel<T, kCluster, kSolo>(cls, false)
+                       : lazy     ? pick_kernel<T, kCta, kLazy>(cls, crowded)
+                                  : pick_kernel<T, kCta, kSolo>(cls, crowded);
   const size_t smem = (size_t)4 * rl.region * sizeof(T);
   rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (rc != cudaSuccess) return rc;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(s.L.batch * rl.C);
-  cfg.blockDim = dim3(rl.threads);
+  cfg.blockDim = dim3(rl.threads + (spec ? 32 : 0));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
