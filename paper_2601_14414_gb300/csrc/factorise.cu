@@ -17,11 +17,14 @@
 // starts from the FP32 one and takes three FP64 instructions instead of a division's dozen or
 // so, signs and pivot tests work on bit patterns, and kLanes lanes work on one stage, so that a
 // warp's per-pivot instructions (reciprocal, scaled column) serve 32 / kLanes stages at once. A
-// small batch, which leaves schedulers idle, takes the whole warp per stage instead.
+// small batch, which leaves schedulers idle, takes two whole warps per stage instead, one for H and
+// one for M and the copies, with all rows of G at once: there the chain of one stage is what counts.
 // 1.13M stages of the batched workload (nx 4 .. 24, nu 2 .. 8): 56.5 ms with a warp per stage,
 // divisions and all of G in shared memory, 26.4 ms so (the FP64 pipe busy 83 % of its nominal
 // rate, which is what it sustains; the multiply-adds alone would take 17). 5000 stages of n = 3:
 // 27.9 and 9.6 us.
+#include <algorithm>
+
 #include "bl_slot.cuh"
 #include "launch.h"
 
@@ -38,7 +41,8 @@ struct FactArgs {
   const int *binst;          // instance of each global block
   const int64_t *bbase;      // first global block of each instance
   int64_t nblocks;
-  int words_per_stage;       // shared-memory doubles per stage
+  int words_per_stage;       // shared-memory doubles per stage (per part of one, kParts == 2)
+  int rows;                  // rows of G held at a time
   int tab_len, tab_words;    // entries of the triangle table, and its doubles
   int *err;                  // [batch]: set to 1 for an instance with a non-positive pivot
 };
@@ -143,18 +147,21 @@ __device__ void sweep_inverse(double *S, double *col, const unsigned short *tab,
   __syncwarp();
 }
 
-// Rows of G held at a time: with all of G, or with 8 rows, an SM holds too few warps to fill the
-// FP64 pipe (batched workload: 8 warps 68 % busy, 12 warps 75 %, 16 warps 83 %, which is its limit
-// at 19 cycles per instruction).
+// Rows of G held at a time by large batches: with all of G, or with 8 rows, an SM holds too few warps
+// to fill the FP64 pipe (batched workload: 8 warps 68 % busy, 12 warps 75 %, 16 warps 83 %, which is
+// its limit at 19 cycles per instruction).
 constexpr int kRows = 6;
 constexpr int kPad = 8;  // rows of G and columns: entries a last round may read past their end
 
-template <typename T, int kLanes>
+// kParts: 1, a group of lanes does all of a stage; 2, consecutive groups do H, and M and the copies.
+template <typename T, int kLanes, int kParts>
 __global__ void __launch_bounds__(128) factorise_kernel(FactArgs a, T *blk) {
   extern __shared__ double smem[];
   const int gl = threadIdx.x & (kLanes - 1);
   const int group = threadIdx.x / kLanes;
-  const int64_t b0 = (int64_t)blockIdx.x * (blockDim.x / kLanes) + group;
+  const bool do_H = kParts == 1 || (group & 1) == 0, do_M = kParts == 1 || (group & 1) == 1;
+  const int rows_max = a.rows;
+  const int64_t b0 = ((int64_t)blockIdx.x * (blockDim.x / kLanes) + group) / kParts;
   const bool valid = b0 < a.nblocks;  // the groups of a warp stay together: the last ones idle
   const int64_t b = valid ? b0 : a.nblocks - 1;
   unsigned short *tab = reinterpret_cast<unsigned short *>(smem);
@@ -164,8 +171,8 @@ __global__ void __launch_bounds__(128) factorise_kernel(FactArgs a, T *blk) {
   const int j = a.binst[b];
   const int kb = (int)(b - a.bbase[j]);
   const int nx = a.L.nx[j], nu = a.L.nu[j], N = a.L.N[j], n = nx + nu;
-  double *G = sh;                          // up to kRows rows of n
-  double *S = G + kRows * n + kPad;        // lower triangle, packed
+  double *G = sh;                          // up to rows_max rows of n
+  double *S = G + rows_max * n + kPad;       // lower triangle, packed
   double *col = S + n * (n + 1) / 2 + kLanes;  // 2 n
   const bool lti = a.L.lti != 0;
   const bool terminal = lti ? (kb == 1) : (kb == N - 1);
@@ -181,39 +188,41 @@ __global__ void __launch_bounds__(128) factorise_kernel(FactArgs a, T *blk) {
   const double *B = a.B + a.L.offB[j];
   const double *e = a.e ? a.e + a.L.offe[j] : nullptr;
 
-  // K = Qbar + rho I (+ rho (G^T G + diag(0, I))), lower triangle, kRows rows of G at a time.
-  const int tr = rounds<kLanes>(n * (n + 1) / 2);
   const int nxmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)nx);
-  for (int r0 = 0; r0 < nxmax; r0 += kRows) {
-    const int rows = terminal ? 0 : min(kRows, nx - r0);  // <= 0: this stage is done
-    const double *Ak = A + (size_t)kH * nx * nx, *Bk = B + (size_t)kH * nx * nu;
-    __syncwarp();
-    for (int w = gl; w < rows * n; w += kLanes) {
-      const int r = w / n, c = w - r * n;
-      G[w] = c < nx ? Ak[(r0 + r) * nx + c] : Bk[(r0 + r) * nu + (c - nx)];
+  if (do_H) {
+    // K = Qbar + rho I (+ rho (G^T G + diag(0, I))), lower triangle, rows_max rows of G at a time.
+    const int tr = rounds<kLanes>(n * (n + 1) / 2);
+    for (int r0 = 0; r0 < nxmax; r0 += rows_max) {
+      const int rows = terminal ? 0 : min(rows_max, nx - r0);  // <= 0: this stage is done
+      const double *Ak = A + (size_t)kH * nx * nx, *Bk = B + (size_t)kH * nx * nu;
+      __syncwarp();
+      for (int w = gl; w < rows * n; w += kLanes) {
+        const int r = w / n, c = w - r * n;
+        G[w] = c < nx ? Ak[(r0 + r) * nx + c] : Bk[(r0 + r) * nu + (c - nx)];
+      }
+      __syncwarp();
+      if (r0 == 0 || rows > 0)
+        for (int q = 0, t = gl; q < tr; ++q, t += kLanes) {  // every lane its own (i, c), c <= i
+          const int i = tab[t] >> 8, c = tab[t] & 0xff;
+          double s = r0 ? S[t] : 0.0;
+          for (int r = 0; r < rows; ++r) s = fma(G[r * n + i], G[r * n + c], s);
+          S[t] = s;
+        }
     }
     __syncwarp();
-    if (r0 == 0 || rows > 0)
-      for (int q = 0, t = gl; q < tr; ++q, t += kLanes) {  // every lane its own (i, c), c <= i
-        const int i = tab[t] >> 8, c = tab[t] & 0xff;
-        double s = r0 ? S[t] : 0.0;
-        for (int r = 0; r < rows; ++r) s = fma(G[r * n + i], G[r * n + c], s);
-        S[t] = s;
-      }
+    if (rho != 1.0) {  // the off-diagonal entries; the diagonal follows
+      for (int t = gl; t < n * (n + 1) / 2; t += kLanes)
+        if (tab[t] >> 8 != (tab[t] & 0xff)) S[t] *= rho;
+      __syncwarp();
+    }
+    for (int i = gl; i < n; i += kLanes) {  // the diagonal's own terms
+      double s = S[tri_slot(i, i)];
+      if (!terminal && i >= nx) s += 1.0;
+      s *= rho;
+      S[tri_slot(i, i)] = s + (qd[i] + rho);
+    }
+    sweep_inverse<kLanes>(S, col, tab, n, nmax, gl, a.err + j);
   }
-  __syncwarp();
-  if (rho != 1.0) {  // the off-diagonal entries; the diagonal follows
-    for (int t = gl; t < n * (n + 1) / 2; t += kLanes)
-      if (tab[t] >> 8 != (tab[t] & 0xff)) S[t] *= rho;
-    __syncwarp();
-  }
-  for (int i = gl; i < n; i += kLanes) {  // the diagonal's own terms
-    double s = S[tri_slot(i, i)];
-    if (!terminal && i >= nx) s += 1.0;
-    s *= rho;
-    S[tri_slot(i, i)] = s + (qd[i] + rho);
-  }
-  sweep_inverse<kLanes>(S, col, tab, n, nmax, gl, a.err + j);
 
   const int W = a.L.W[j];
   const int lay = a.L.tiled;
@@ -277,9 +286,12 @@ __global__ void __launch_bounds__(128) factorise_kernel(FactArgs a, T *blk) {
       }
     }
   };
-  if (blocked) put_sym_blocks(oH, n, S);
-  else put_sym(oH, n, S);
-  __syncwarp();
+  if (do_H) {
+    if (blocked) put_sym_blocks(oH, n, S);
+    else put_sym(oH, n, S);
+    __syncwarp();
+  }
+  if (!do_M) return;
 
   // Own-stage G_k, e_k and M_k = (B_k^T B_k + I + Wdu/rho)^{-1}.
   const double *Ak = A + (size_t)kS * nx * nx, *Bk = B + (size_t)kS * nx * nu;
@@ -296,8 +308,8 @@ __global__ void __launch_bounds__(128) factorise_kernel(FactArgs a, T *blk) {
     for (int r = nx + gl; r < bl_pad4(nx); r += kLanes) put(oE + r, 0.0);
   const double *rdu = a.rdu ? a.rdu + a.L.off_n[j] + nx : nullptr;
   const int tru = rounds<kLanes>(nu * (nu + 1) / 2);
-  for (int r0 = 0; r0 < nxmax; r0 += kRows) {
-    const int rows = min(kRows, nx - r0);
+  for (int r0 = 0; r0 < nxmax; r0 += rows_max) {
+    const int rows = min(rows_max, nx - r0);
     __syncwarp();
     for (int w = gl; w < rows * nu; w += kLanes) G[w] = Bk[r0 * nu + w];
     __syncwarp();
@@ -318,31 +330,33 @@ __global__ void __launch_bounds__(128) factorise_kernel(FactArgs a, T *blk) {
   }
 }
 
-template <typename T, int kLanes>
-cudaError_t launch_lanes(const FactArgs &a, T *blk, int warps, size_t per_stage, cudaStream_t stream) {
-  const int stages = warps * 32 / kLanes;
-  const size_t smem = per_stage * stages + sizeof(double) * a.tab_words;
-  cudaError_t rc = cudaFuncSetAttribute(factorise_kernel<T, kLanes>,
+template <typename T, int kLanes, int kParts>
+cudaError_t launch_lanes(const FactArgs &a, T *blk, int warps, size_t per_group, cudaStream_t stream) {
+  const int groups = warps * 32 / kLanes, stages = groups / kParts;
+  const size_t smem = per_group * groups + sizeof(double) * a.tab_words;
+  cudaError_t rc = cudaFuncSetAttribute(factorise_kernel<T, kLanes, kParts>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (rc != cudaSuccess) return rc;
-  factorise_kernel<T, kLanes><<<(unsigned)((a.nblocks + stages - 1) / stages), 32 * warps, smem, stream>>>(a, blk);
+  factorise_kernel<T, kLanes, kParts>
+      <<<(unsigned)((a.nblocks + stages - 1) / stages), 32 * warps, smem, stream>>>(a, blk);
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_t(const FactArgs &a, T *blk, int lanes, int warps, size_t per_stage,
+cudaError_t launch_t(const FactArgs &a, T *blk, int lanes, int parts, int warps, size_t per_group,
                      cudaStream_t stream) {
-  return lanes == 8    ? launch_lanes<T, 8>(a, blk, warps, per_stage, stream)
-         : lanes == 16 ? launch_lanes<T, 16>(a, blk, warps, per_stage, stream)
-                       : launch_lanes<T, 32>(a, blk, warps, per_stage, stream);
+  return lanes == 8    ? launch_lanes<T, 8, 1>(a, blk, warps, per_group, stream)
+         : lanes == 16 ? launch_lanes<T, 16, 1>(a, blk, warps, per_group, stream)
+         : parts == 1  ? launch_lanes<T, 32, 1>(a, blk, warps, per_group, stream)
+                       : launch_lanes<T, 32, 2>(a, blk, warps, per_group, stream);
 }
 
 }  // namespace
 
-// Shared-memory doubles of one stage: kRows rows of G, the packed lower triangle, the pivot
+// Shared-memory doubles of one stage: `rows` rows of G, the packed lower triangle, the pivot
 // column twice.
-static int factorise_stage_words(int max_n, int lanes) {
-  return kRows * max_n + kPad + max_n * (max_n + 1) / 2 + lanes + 2 * max_n + kPad;
+static int factorise_stage_words(int max_n, int lanes, int rows) {
+  return rows * max_n + kPad + max_n * (max_n + 1) / 2 + lanes + 2 * max_n + kPad;
 }
 
 cudaError_t launch_factorise(const Layout &L, const double *A, const double *B, const double *e,
@@ -358,18 +372,21 @@ cudaError_t launch_factorise(const Layout &L, const double *A, const double *B, 
   int dev = 0, nsm = 0;
   if ((rc = cudaGetDevice(&dev)) != cudaSuccess) return rc;
   if ((rc = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return rc;
-  // Few stages: a warp each, spread over the schedulers. Many: 8 or 16 lanes each.
+  // Few stages (up to two per SM): two warps each, spread over the schedulers (200 stages of n = 16:
+  // 31 us with a warp each, 24 with two). Up to eight per SM: a warp each. Many: 8 or 16 lanes each.
+  const int parts = nblocks <= 2 * (int64_t)nsm ? 2 : 1;
   int lanes = nblocks <= 8 * (int64_t)nsm ? 32 : (max_n <= 8 ? 8 : 16);
-  int warps = nblocks <= 4 * (int64_t)nsm ? 1 : 4;
-  auto bytes = [&](int l, int w) { return sizeof(double) * factorise_stage_words(max_n, l) * (32 / l) * w; };
+  int warps = parts == 2 ? 2 : (nblocks <= 4 * (int64_t)nsm ? 1 : 4);
+  a.rows = parts == 2 ? max_nx : std::min(kRows, max_nx);
+  auto bytes = [&](int l, int w) { return sizeof(double) * factorise_stage_words(max_n, l, a.rows) * (32 / l) * w; };
   while (lanes < 32 && bytes(lanes, warps) > 100 * 1024) lanes *= 2;
-  while (warps > 1 && bytes(lanes, warps) > 200 * 1024) warps >>= 1;
-  a.words_per_stage = factorise_stage_words(max_n, lanes);
+  while (warps > parts && bytes(lanes, warps) > 200 * 1024) warps >>= 1;
+  a.words_per_stage = factorise_stage_words(max_n, lanes, a.rows);
   a.tab_len = max_n * (max_n + 1) / 2 + lanes;
   a.tab_words = (a.tab_len + 3) / 4;
   const size_t per_stage = sizeof(double) * a.words_per_stage;
-  return precision == 0 ? launch_t<float>(a, (float *)blk, lanes, warps, per_stage, stream)
-                        : launch_t<double>(a, (double *)blk, lanes, warps, per_stage, stream);
+  return precision == 0 ? launch_t<float>(a, (float *)blk, lanes, parts, warps, per_stage, stream)
+                        : launch_t<double>(a, (double *)blk, lanes, parts, warps, per_stage, stream);
 }
 
 }  // namespace pimpc
