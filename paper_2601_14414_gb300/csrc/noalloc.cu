@@ -18,7 +18,7 @@
 // on the same memory layout, with their buffers carved out of the static array. An instance that
 // the resident schedule holds (registers or shared memory of one CTA, a cluster or a few dozen
 // CTAs; see plan_resident) runs on it: one instance leaves the lock-step frame waiting on its grid
-// barrier (n 16, N 200, 100 FP32 iterations: 8.6 ms there, 0.2 ms resident). Its momentum factors
+// barrier (n 16, N 200, 100 FP32 iterations: 8.81 ms there, 0.17 ms resident, all launches counted). Its momentum factors
 // come from a constant table, filled once per device together with the array's address; longer
 // runs, and instances too long for a cluster, use one thread per stage on tiles.
 #include <algorithm>
@@ -110,8 +110,16 @@ struct Views {
   Ctl *ctl;
 };
 
-// Fills the single-instance layout and work list (all offsets 0, one instance).
-__global__ void static_setup_kernel(Views v, int nx, int nu, int N, int W, int item_stages,
+// The caller's vectors (FP64) and where they go.
+struct Vectors {
+  const double *q, *r, *xmin, *xmax, *umin, *umax, *x0, *ref;
+  void *qd, *lo, *hi, *xb0, *refT;  // iteration precision
+};
+
+// Fills the single-instance layout and work list (all offsets 0, one instance), the weights, bounds,
+// xbar_0 and the reference: one launch.
+template <typename T>
+__global__ void static_setup_kernel(Views v, Vectors in, int nx, int nu, int N, int W, int item_stages,
                                     int nitems) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t == 0) {
@@ -123,6 +131,16 @@ __global__ void static_setup_kernel(Views v, int nx, int nu, int N, int W, int i
     v.base[0] = 0;
     v.nitems_inst[0] = nitems;
     v.ferr[0] = 0;
+  }
+  for (int c = t; c < nx + nu; c += gridDim.x * blockDim.x) {
+    const bool x = c < nx;
+    const double w = x ? in.q[c] : in.r[c - nx];
+    v.qd64[c] = w;
+    ((T *)in.qd)[c] = (T)w;
+    ((T *)in.lo)[c] = (T)(x ? in.xmin[c] : in.umin[c - nx]);
+    ((T *)in.hi)[c] = (T)(x ? in.xmax[c] : in.umax[c - nx]);
+    ((T *)in.xb0)[c] = x ? (T)in.x0[c] : (T)0;
+    if (in.ref) ((T *)in.refT)[c] = (T)in.ref[c];
   }
   for (int k = t; k < N; k += gridDim.x * blockDim.x) v.binst[k] = 0;
   for (int i = t; i < nitems; i += gridDim.x * blockDim.x) {
@@ -253,18 +271,16 @@ extern "C" int pimpc_solve_static(int nx, int nu, int N, int precision, const do
                                         cudaGetErrorString(e2));
   };
   int ret;
-  static_setup_kernel<<<1, 128, 0, st>>>(v, nx, nu, N, W, item_stages, nitems);
+  const Vectors in{q, r, xmin, xmax, umin, umax, x0, ref, qd_T, lo_T, hi_T, xb0_T, ref_T};
+  if (precision == PIMPC_F32)
+    static_setup_kernel<float><<<1, 128, 0, st>>>(v, in, nx, nu, N, W, item_stages, nitems);
+  else
+    static_setup_kernel<double><<<1, 128, 0, st>>>(v, in, nx, nu, N, W, item_stages, nitems);
   if ((ret = check(cudaGetLastError(), "setup"))) return ret;
   // Everything the kernels read before writing starts from a known state on every call.
   // (The factorisation writes every word of a plain block; tiles hold stages beyond N.)
   if (!resident && (ret = check(cudaMemsetAsync(blk, 0, blk_elems * ts, st), "clear stage blocks")))
     return ret;
-  if ((ret = check(launch_gather_n64(L, q, r, n, v.qd64, st), "weights"))) return ret;
-  if ((ret = check(launch_gather_n(L, q, r, n, precision, qd_T, st), "weights"))) return ret;
-  if ((ret = check(launch_gather_n(L, xmin, umin, n, precision, lo_T, st), "bounds"))) return ret;
-  if ((ret = check(launch_gather_n(L, xmax, umax, n, precision, hi_T, st), "bounds"))) return ret;
-  if ((ret = check(launch_gather_n(L, x0, nullptr, n, precision, xb0_T, st), "x0"))) return ret;
-  if (ref && (ret = check(launch_convert(ref, n, precision, ref_T, st), "ref"))) return ret;
   if ((ret = check(launch_factorise(L, A, B, e, v.qd64, nullptr, rho, v.binst, v.off[11], N, nx, n,
                                     precision, blk, v.ferr, st), "factorise")))
     return ret;
