@@ -37,14 +37,15 @@ void reg_plan(int batch, const int *nx, const int *nu, const int *N, int precisi
 // stay within `few` threads (FP32, n 16, N 50: 1.25 us with 256 threads, 1.19 with 160, 1.18 with 96),
 // the cluster of 16 within `most`, and beyond that (FP64, whose iterations are long enough to pay for
 // an exchange through global memory, or instances that no cluster holds) the fewest CTAs within
-// `grid` (n 16, N 200, FP64: 7.15 us on a cluster of 16, 4.93 on 32 CTAs; N 100: 4.67 on the cluster).
+// `grid` (n 16, N 200, FP64: 7.15 us on a cluster of 16, 4.93 on 32 CTAs of 160 threads, 4.73 on 40 of
+// 128, 4.72 on 64; n 3, N 5000: 4.12 on 96, 3.65 on 128; n 16, N 100: 4.67 on the cluster and on 32).
 // Batches larger than the SMs take the fewest CTAs that hold an instance.
 static RegLaunch choose_reg(int item_scale, int batch, const int *nx, const int *nu, const int *N,
                             int precision, int nsm) {
   const bool f32 = precision == 0;
-  const int one = f32 ? 480 : 128, few = f32 ? 160 : 128, most = f32 ? 1024 : 160, grid = f32 ? 512 : 160;
+  const int one = f32 ? 480 : 128, few = f32 ? 160 : 128, most = f32 ? 1024 : 160, grid = f32 ? 512 : 128;
   RegLaunch best;
-  for (int cand : {1, 2, 4, 8, 16, 24, 32, 48, 64, 80, 96}) {
+  for (int cand : {1, 2, 4, 8, 16, 24, 32, 40, 48, 64, 80, 96, 112, 128, 144}) {
     if (item_scale > 0 && cand != item_scale) continue;
     RegLaunch t;
     t.C = cand;

@@ -50,7 +50,8 @@ template <typename T>
 using Args = ls::Args<T>;
 
 constexpr int kMaxN = 16;
-constexpr int kMaxC = 96;            // CTAs of one instance (grid scope)
+constexpr int kMaxC = 144;           // CTAs of one instance (grid scope)
+constexpr int kLaneShares = (kMaxC + 31) / 32;
 constexpr int kWaitPolls = 1 << 22;  // bounded waits: polls of a record in global memory ...
 constexpr long long kWaitCycles = 1ll << 31;  // ... and cycles at an mbarrier (about a second)
 
@@ -62,7 +63,8 @@ enum { kCta = 0, kCluster = 1, kGrid = 2 };
 // on the hats that a momentum step would give (latency: CTAs that have an SM each). kSolo: warp 0
 // finds c between two iterations (batches that crowd the SMs). kLazy: c is not formed before the last
 // iteration (the plain iteration with a fixed count, where no decision depends on it but that a
-// non-finite c ends the solve, so a share that is non-finite or near overflow has it formed).
+// non-finite c ends the solve, so an iterate that is not finite or so large that its squares may not
+// be has it formed).
 enum { kSpec = 0, kSolo = 1, kLazy = 2 };
 
 // Threads of one CTA by the register bound: 4 n-vectors of matrix rows per thread.
@@ -298,7 +300,8 @@ struct Lane {
   // Steps 1-4 with hats cur + f (cur - prev) (momentum) or cur: the new iterate of an owned component
   // and its share of c. sW, sY, sH, sX: the CTA's vectors (sX: row q = xbar of slot q); sync: a barrier
   // of its threads, after which earlier reads of the vectors are over.
-  template <typename Sync>
+  // kShare: whether the share is formed.
+  template <bool kShare, typename Sync>
   __device__ __forceinline__ void iterate(T *sW, T *sY, T *sH, T *sX, T f, bool momentum, Sync sync, T &zn,
                                           T &vn, T &tn, T &bn, T &cacc) {
     // ---- hats, y, w ----
@@ -347,11 +350,14 @@ struct Lane {
       tn = s - zn;
       bn = p - vn;
       // theta' - theta = xbar - z' and beta' - beta = Bbar du - v', without the duals' own rounding
-      const T d1 = xb - zn, d2 = bd - vn, d4 = zn - zh, d5 = vn - vh;
-      // d1^2 + d2^2 + d3^2 + d4^2 + d5^2 + (d4 - d5)^2 with d3 = -d2
-      const T g = d2 * d2 + (d4 * d4 + d5 * (d5 - d4));
-      cacc = (T)2 * g + d1 * d1;
+      if constexpr (kShare) cacc = share(xb - zn, bd - vn, zn - zh, vn - vh);
     }
+  }
+
+  // d1^2 + d2^2 + d3^2 + d4^2 + d5^2 + (d4 - d5)^2 with d3 = -d2.
+  static __device__ __forceinline__ T share(T d1, T d2, T d4, T d5) {
+    const T g = d2 * d2 + (d4 * d4 + d5 * (d5 - d4));
+    return (T)2 * g + d1 * d1;
   }
 
   // Cluster: the first stage's new iterate to CTA r - 1, the last one's to CTA r + 1.
@@ -561,12 +567,12 @@ __global__ void __launch_bounds__(spec_max_threads((int)sizeof(T), NM), 1) spec_
       }
       if (SC == kGrid && ok) {
         if (lane == 0) put_rec(xs + par * C + r, sum.sig, with_tag((unsigned)sum.e, tag));
-        detsum::Fx t[3];  // C <= 96 shares, three per lane, all in flight
+        detsum::Fx t[kLaneShares];  // the lane's shares, all in flight
         ok = false;
         for (int n_ = 0; n_ < kWaitPolls && !ok; ++n_) {
           bool mine = true;
 #pragma unroll
-          for (int q = 0; q < 3; ++q) {
+          for (int q = 0; q < kLaneShares; ++q) {
             unsigned long long b = with_tag((unsigned)detsum::kZero, tag);
             t[q].sig = 0;
             if (lane + 32 * q < C) get_rec(xs + par * C + lane + 32 * q, t[q].sig, b);
@@ -576,10 +582,14 @@ __global__ void __launch_bounds__(spec_max_threads((int)sizeof(T), NM), 1) spec_
           ok = __all_sync(0xffffffffu, mine);
         }
         sum = detsum::warp_sum(t[0]);
-        if (C > 32) {
-          const detsum::Fx s1 = detsum::warp_sum(t[1]), s2 = detsum::warp_sum(t[2]);
-          sum = detsum::warp_sum(lane == 0 ? sum : lane == 1 ? s1 : lane == 2 ? s2
-                                                                  : detsum::Fx{0ull, detsum::kZero});
+        if (C > 32) {  // the sums of each round of 32, on lanes 0, 1, ..
+          detsum::Fx mine = lane == 0 ? sum : detsum::Fx{0ull, detsum::kZero};
+#pragma unroll
+          for (int q = 1; q < kLaneShares; ++q) {
+            const detsum::Fx sq = detsum::warp_sum(t[q]);
+            if (lane == q) mine = sq;
+          }
+          sum = detsum::warp_sum(mine);
         }
       }
       bool take = false;
@@ -638,7 +648,7 @@ __global__ void __launch_bounds__(spec_max_threads((int)sizeof(T), NM), 1) spec_
       T fnext = (T)0;
       bool mnext = false;
       if (it < a.max_iters) {
-        L.iterate(sW, sY, sH, sX, f, momentum, sync, zn, vn, tn, bn, cacc);
+        L.template iterate<true>(sW, sY, sH, sX, f, momentum, sync, zn, vn, tn, bn, cacc);
       }
       if (it > 0) {
         named_sync<3>(all);  // the decision of it - 1
@@ -646,7 +656,7 @@ __global__ void __launch_bounds__(spec_max_threads((int)sizeof(T), NM), 1) spec_
         fnext = *(volatile T *)&sh.fnext;
         mnext = *(volatile int *)&sh.use_next != 0;
         if (momentum && !*(volatile int *)&sh.take)
-          L.iterate(sW, sY, sH, sX, (T)0, false, sync, zn, vn, tn, bn, cacc);
+          L.template iterate<true>(sW, sY, sH, sX, (T)0, false, sync, zn, vn, tn, bn, cacc);
       }
       if (SC == kCta || *(volatile int *)&sh.fail == 0) {
         if (SC == kCluster) L.push_boundary(sh, par, r, zn, vn, tn, bn);
@@ -698,12 +708,15 @@ __global__ void __launch_bounds__(reg_max_threads((int)sizeof(T), NM), kMinCtas)
     // the momentum factor this iteration's decision would take, fetched ahead
     const T fnext = lazy ? (T)0 : (T)d.factor(a, d.streak);
     T zn, vn, tn, bn, cacc;
-    L.iterate(sW, sY, sH, sX, f, !lazy && momentum, sync, zn, vn, tn, bn, cacc);
+    L.template iterate<!lazy>(sW, sY, sH, sX, f, !lazy && momentum, sync, zn, vn, tn, bn, cacc);
     if (SC != kCta && sh.fail) break;  // set before the iteration's first barrier, if at all: uniform
     if (SC == kCluster) L.push_boundary(sh, par, r, zn, vn, tn, bn);
-    if (lazy && it + 1 < a.max_iters && !__syncthreads_or(detsum::may_overflow(cacc))) {
-      L.zc = zn; L.vc = vn; L.tc = tn; L.bc = bn;
-      continue;
+    if (lazy) {
+      if (it + 1 < a.max_iters && !__syncthreads_or(detsum::large(zn, vn, tn, bn))) {
+        L.zc = zn; L.vc = vn; L.tc = tn; L.bc = bn;
+        continue;
+      }
+      cacc = L.owned ? L.share(tn - L.tc, bn - L.bc, zn - L.zc, vn - L.vc) : (T)0;
     }
     // ---- c: by warp 0, the others read it (their integer sums take longer than one more barrier) ----
     detsum::Fx sum = detsum::warp_sum(cacc);

@@ -111,11 +111,18 @@ __device__ __forceinline__ bool finite(float v) {
   return (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u;
 }
 
-// Whether a sum of v with others may leave the finite range (NaN and infinity included).
-__device__ __forceinline__ bool may_overflow(double v) {
-  return ((unsigned)__double2hiint(v) & 0x7ff00000u) >= (2047u - 16u) << 20;
+// Whether a sum of squares of differences of such values may leave the finite range (NaN and infinity
+// included): some magnitude of 2^59 (FP32) or 2^500 (FP64) and more.
+__device__ __forceinline__ bool large(double a, double b, double c, double d) {
+  const unsigned m = max(max((unsigned)__double2hiint(a) & 0x7ff00000u, (unsigned)__double2hiint(b) & 0x7ff00000u),
+                         max((unsigned)__double2hiint(c) & 0x7ff00000u, (unsigned)__double2hiint(d) & 0x7ff00000u));
+  return m >= (1023u + 500u) << 20;
 }
-__device__ __forceinline__ bool may_overflow(float v) { return !finite(v); }
+__device__ __forceinline__ bool large(float a, float b, float c, float d) {
+  const unsigned m = max(max(__float_as_uint(a) & 0x7f800000u, __float_as_uint(b) & 0x7f800000u),
+                         max(__float_as_uint(c) & 0x7f800000u, __float_as_uint(d) & 0x7f800000u));
+  return m >= (127u + 59u) << 23;
+}
 
 }  // namespace detsum
 }  // namespace pimpc
