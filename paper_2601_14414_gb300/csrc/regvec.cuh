@@ -41,10 +41,11 @@ __device__ __forceinline__ double dot(const double (&m)[NM], const double *v, in
   return a;
 }
 
-// x / 3 to within a rounding of the correctly rounded quotient: 1/3 as the sum of its rounding
-// and the rounding of what is left (two operations instead of a division; infinities pass).
+// x / 3 to within a rounding of the correctly rounded quotient: 1/3 as the sum of its value rounded
+// down and the rounding of what is left (two operations instead of a division; both parts are
+// positive, so that infinities pass).
 __device__ __forceinline__ float third(float x) {
-  constexpr float hi = 1.0f / 3.0f;
+  constexpr float hi = 0x1.555554p-2f;
   constexpr float lo = (float)(1.0 / 3.0 - (double)hi);
   return fmaf(x, hi, x * lo);
 }
