@@ -88,6 +88,14 @@ bool plan_resident(int item_scale, int batch, const int *nx, const int *nu, cons
   // what the shared-memory kernel accepts, in registers where n <= 16 allows it
   *reg = choose_reg(item_scale, batch, nx, nu, N, precision, nsm);
   if (reg->threads > 0) *smem = (size_t)4 * reg->region * ts;
+  if (reg->threads > 0 && precision == 0 && item_scale <= 1) {
+    const int mx = *std::max_element(nx, nx + batch), mu = *std::max_element(nu, nu + batch);
+    const int mN = *std::max_element(N, N + batch);
+    if (mx <= 4 && mu <= 2 && mN <= kStageThreads) {
+      reg->stage_class = mu <= 1 ? (mx <= 2 ? 0 : 1) : 2;
+      reg->stage_threads = (mN + 31) / 32 * 32;
+    }
+  }
   return true;
 }
 

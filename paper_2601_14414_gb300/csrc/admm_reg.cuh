@@ -1,5 +1,6 @@
 // admm_reg.cuh -- the resident schedule (family 3) for instances with n <= 16: the stage matrices
-// and the iterates of an instance live in the registers of one CTA, or of a cluster of C CTAs.
+// and the iterates of an instance live in the registers of one CTA, or of C CTAs: a cluster of
+// up to 16, or up to 144 that meet through global memory.
 //
 // What bounds a resident solve is the latency of one iteration: a few hundred multiply-adds per
 // stage between synchronisations, the cross-CTA exchange, and the FP64 decision of steps 5-7.
@@ -29,8 +30,8 @@
 // iteration) runs beside the next iteration, in a warp of its own (spec_kernel).
 // Per iteration, measured, against the shared-memory kernel of admm_res.cu (which keeps the
 // instances with n > 16) and, in brackets, without the deciding warp: plain LTI n 6, N 20, FP64
-// 7.9 -> 3.0 us (3.2); quadrotor n 16, N 200 FP32 6.8 -> 1.26 us (1.80), FP64 18.6 -> 4.9 us (5.6);
-// CSTR n 3, N 5000 FP32 22.8 -> 1.80 us (2.59), FP64 102 -> 4.1 us (5.9).
+// 7.9 -> 3.0 us (3.2); quadrotor n 16, N 200 FP32 6.8 -> 1.26 us (1.80), FP64 18.6 -> 4.7 us (5.6);
+// CSTR n 3, N 5000 FP32 22.8 -> 1.80 us (2.59), FP64 102 -> 3.65 us (5.9).
 #pragma once
 #include <cooperative_groups.h>
 #include <algorithm>
@@ -811,6 +812,9 @@ cudaError_t reg_launch_t(const AdmmLaunch &s, const RegLaunch &rl, cudaStream_t 
   // has other CTAs to run meanwhile.
   const bool watch = s.stall_win > 0 || s.mask != nullptr;
   const bool lazy = !s.accel && s.eps < 0.0 && !watch;
+  if constexpr (sizeof(T) == 4)  // a thread per stage is the faster one at every batch and horizon
+    if (lazy && rl.stage_class >= 0)
+      return launch_stage(s, rl.stage_class, rl.stage_threads, stream);
   const bool crowded = (int64_t)s.L.batch * rl.C > nsm || rl.threads + 32 > spec_max_threads((int)sizeof(T), cls);
   const bool spec = rl.C > 16 || (!crowded && !(lazy && rl.C == 1));
   const void *kernel = spec ? (rl.C == 1    ? pick_spec<T, kCta>(cls)

@@ -99,11 +99,15 @@ struct RegLaunch {
   int C = 0, threads = 0, region = 0, nmax = 0;  // threads == 0: the shared-memory kernel runs
   size_t xch_bytes = 0;                          // C > 16: exchange records in global memory
   void *xch = nullptr;
+  int stage_class = -1, stage_threads = 0;       // admm_stage.cu's size class (-1: it does not serve the batch)
 };
 void reg_plan(int batch, const int *nx, const int *nu, const int *N, int precision, RegLaunch *rl);
 bool plan_resident(int item_scale, int batch, const int *nx, const int *nu, const int *N,
                    const int *W, int lti, int precision, int nsm, size_t optin, int *res,
                    size_t *smem, RegLaunch *reg);
+// One thread per stage: nx <= 4, nu <= 2, up to kStageThreads stages, FP32; 3, 5 or 6 components.
+constexpr int kStageThreads = 256;
+cudaError_t launch_stage(const AdmmLaunch &s, int size_class, int threads, cudaStream_t stream);
 cudaError_t launch_reg(const AdmmLaunch &s, int precision, const RegLaunch &rl, cudaStream_t stream);
 
 // Stage-invariant instances as dense contractions (register-tiled products over stage blocks).
