@@ -325,12 +325,16 @@ static int64_t dense_words(int nx, int nu, int W, int lti, int SL, int *blk, int
 }
 
 // Slots per sub-chunk of each instance within the shared memory of three CTAs per SM (at least two
-// stages' worth, within one CTA's), the launch's regions; false if an instance does not fit.
+// stages' worth, within one CTA's), the launch's regions; false if an instance does not fit, or if a CTA's
+// threads give one fewer than five slots (n > 51): with four a quarter of them hold the next stage,
+// and the lane groups win (304 stage-invariant instances, N 200: n 48, five slots, 1.70 ms per
+// iteration in lane groups, 1.12 here; n 56 1.95 and 2.63; 256 of n 64, N 1000 11.9 and 13.7).
 bool dense_plan(int batch, const int *nx, const int *nu, const int *W, int lti, int64_t smem_sm,
                 int64_t optin, int *slots, int *plan, size_t *smem) {
   plan[0] = plan[1] = plan[2] = 0;
   for (int j = 0; j < batch; ++j) {
     int SL = kThreads / (nx[j] + nu[j]), b, h, v;
+    if (SL < 5) return false;
     while (SL > 2 && dense_words(nx[j], nu[j], W[j], lti, SL, &b, &h, &v) * 8 > smem_sm / 3 - 2048) --SL;
     dense_words(nx[j], nu[j], W[j], lti, SL, &b, &h, &v);
     slots[j] = SL;

@@ -57,6 +57,16 @@ def test_stage_invariant(dims):
         assert relerr(r["u"][j], o["u"]) <= 1e-10 and relerr(r["x"][j], o["x"]) <= 1e-10, j
 
 
+@pytest.mark.parametrize("n", [51, 52])
+def test_five_slots_and_four(n):
+    # the widest instance that gives a CTA five slots, and one more, which the lane groups take
+    insts = [W.plain_lti(9850 + j, nx, nu, N) for j, (nx, nu, N) in enumerate([(n - 11, 11, 30), (4, 2, 20)])]
+    s = pimpc.Solver(insts, precision=pimpc.F64, eps=-1.0, max_iters=60, accel=1)
+    r = s.solve()
+    for j, o in enumerate(oracle.solve_batch(insts, eps=-1.0, max_iters=60, accel=1)):
+        assert relerr(r["u"][j], o["u"]) <= 1e-10 and relerr(r["x"][j], o["x"]) <= 1e-10, j
+
+
 def test_stops_warm_starts_and_input_sets():
     insts = batch(DIMS[3:8], 9900)
     s = pimpc.Solver(insts, precision=pimpc.F64, eps=1e-6, max_iters=4000, accel=1)
