@@ -318,11 +318,14 @@ int pimpc_backward(pimpc_solver *s, const double *dL_du, const double *dL_dx, do
  * Algorithm 1 across its SMs; the arithmetic of an iteration is the same under every schedule,
  * up to the order of the sums in c).
  *   family       0: a group of lanes per stage on plain stage blocks, one component per lane
- *                   (every precision and instance kind; the default for FP64 iterations);
+ *                   (every precision and instance kind; the default for FP64 iterations, which
+ *                   on box constraints give consecutive components to consecutive threads, in
+ *                   CTAs of 256);
  *                   2: one thread per stage on halo tiles (stage-varying FP32 instances only);
- *                   3: every instance resident in the shared memory of one CTA or of a
- *                   thread-block cluster for the whole solve (no grid-wide synchronisation;
- *                   for instances that fit); 4: stage-invariant instances only, the per-stage
+ *                   3: every instance resident on chip for the whole solve (no
+ *                   synchronisation between instances; for instances that fit): for n <= 16 in
+ *                   the registers of one CTA, of a thread-block cluster or of up to 144 CTAs,
+ *                   else in the shared memory of one CTA or of a cluster; 4: stage-invariant instances only, the per-stage
  *                   products of blocks of stages as dense matrix-matrix contractions; 5: a
  *                   group of 4, 8 or 16 lanes per stage on blocked stage blocks, four
  *                   components per lane (every precision and instance kind; the default for
@@ -342,7 +345,9 @@ int pimpc_backward(pimpc_solver *s, const double *dL_du, const double *dL_dx, do
  *                active items no longer cover the grid the solve switches to items of one
  *                sub-chunk for stage-varying batches); family 2: at most
  *                this many tiles per work item (0 = 4); family 3: CTAs per instance, 1, 2, 4,
- *                8 or 16 (0 = the fewest whose shared memory holds the instance, or the most
+ *                8 or 16 (0 = chosen from the sizes: for n <= 16 the fewest whose registers
+ *                hold the instance, more for single instances where that is faster, up to
+ *                144; else the fewest whose shared memory holds it, or the most
  *                that leave each CTA four stages when the batch occupies few SMs); family 4:
  *                stages per block (0 = as many as the shared memory holds, at most 128);
  *                family 6: 127-stage tiles per work item (0 = 2); family 7: T, iterations per

@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(256) adjoint_kernel(AdjArgs a) {
 // ---- the same sweep with an instance in the registers of one CTA (n <= 16) ---------------------
 //
 // The sweep above reads every matrix element and every vector component from memory; one cart-pole
-// batch (1024 instances, N 100, 150 iterations) took it 12.5 ms. Here thread (k, c) holds component
+// batch (1024 instances, N 100, 150 iterations) took it 12.5 ms, this one 1.61. Here thread (k, c) holds component
 // c of stage k and its rows of G_k, H_k, P_k = Bbar_k M_k Bbar_k^T and its column of G_{k+1}, as in
 // the register-resident solve (admm_reg.cuh, whose reduced iteration with lambda = -beta this
 // reverses), and the vectors cross threads through shared memory. With bars for adjoints, an
@@ -507,7 +507,9 @@ __global__ void __launch_bounds__(256) adjoint_kernel(AdjArgs a) {
 // (every iteration at once when that takes no more memory than the checkpoints and states of the
 // sweep above), in place of K full states. Gradient sums run in FP64 for FP64 iterations and as
 // unevaluated float pairs (48 bits, error-free additions) for FP32 ones: three FP64 additions per
-// thread and iteration would take longer than the iteration.
+// thread and iteration would take longer than the iteration. What bounds it is the issue rate of one
+// CTA of 512 threads per SM between three barriers per iteration; two CTAs per SM (64 registers,
+// spills) took 1.87 ms, a thread per whole stage (204 registers, 8 warps per SM) 2.13.
 struct RegAdj {
   int region;       // elements of each of the four vector regions in shared memory
   int K, nck;       // iterations per segment, segments

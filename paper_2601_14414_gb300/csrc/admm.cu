@@ -1,6 +1,7 @@
 // admm.cu -- Algorithm 1 with a group of lanes per stage on plain stage blocks, one component per
-// lane (schedule family 0, the default for FP64 iterations; FP32 iterations default to the
-// blocked lane groups of admm_blk.cu).
+// lane (schedule family 0: FP32 iterations, non-box input sets, and FP64 instances that the
+// full-warp kernel of admm_dense.cu does not hold. FP32 iterations default to the blocked lane
+// groups of admm_blk.cu).
 //
 // Work decomposition. The stages of every instance are cut into items of consecutive stages
 // (item = instance j, stages [a, b)). One cooperative launch runs all iterations of all

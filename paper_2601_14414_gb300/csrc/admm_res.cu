@@ -1,5 +1,6 @@
 // admm_res.cu -- Algorithm 1 with every instance resident on chip: one CTA, or a thread-block
-// cluster of C CTAs, per instance (schedule family 3).
+// cluster of C CTAs, per instance, in shared memory (schedule family 3, batches with an instance of
+// n > 16 or one that the registers of admm_reg.cuh do not hold).
 //
 // The lock-step kernels stream the stage data from HBM every iteration and separate iterations
 // by a grid-wide barrier (global atomics); for a single instance or a small batch that barrier,

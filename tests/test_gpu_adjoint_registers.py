@@ -1,6 +1,6 @@
 """The register sweep of pimpc_backward (every instance with n <= 16 in one CTA's threads) against
-the workspace sweep, which a batch takes as soon as one of its instances is too large: the same
-instances alone and together with a large one. Sizes at the edges of the register classes and of
+the workspace sweep, which a batch takes as soon as one of its instances has n > 16: the same
+instances alone and together with such a one. Sizes at the edges of the register classes and of
 a CTA's threads (512 components in FP32, 256 for n > 8 in FP64), segments of one iteration, of some
 and of all, both reference forms, each stage layout. FP64: both sweeps differentiate the same map
 and differ by rounding only (1e-16 through a few dozen iterations: 1e-10 of the gradient allowed);
