@@ -35,7 +35,7 @@
 
 #include "launch.h"
 #include "pimpc.h"
-#include "regvec.cuh"
+#include "stage_reg.cuh"
 #include "solver.h"
 
 namespace pimpc {
@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(256) adjoint_kernel(AdjArgs a) {
 // ---- the same sweep with an instance in the registers of one CTA (n <= 16) ---------------------
 //
 // The sweep above reads every matrix element and every vector component from memory; one cart-pole
-// batch (1024 instances, N 100, 150 iterations) took it 12.5 ms, this one 1.61. Here thread (k, c) holds component
+// batch (1024 instances, N 100, 150 iterations) took it 12.5 ms, this one 1.60. Here thread (k, c) holds component
 // c of stage k and its rows of G_k, H_k, P_k = Bbar_k M_k Bbar_k^T and its column of G_{k+1}, as in
 // the register-resident solve (admm_reg.cuh, whose reduced iteration with lambda = -beta this
 // reverses), and the vectors cross threads through shared memory. With bars for adjoints, an
@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(256) adjoint_kernel(AdjArgs a) {
 // unevaluated float pairs (48 bits, error-free additions) for FP32 ones: three FP64 additions per
 // thread and iteration would take longer than the iteration. What bounds it is the issue rate of one
 // CTA of 512 threads per SM between three barriers per iteration; two CTAs per SM (64 registers,
-// spills) took 1.87 ms, a thread per whole stage (204 registers, 8 warps per SM) 2.13.
+// spills) took 1.87 ms. Batches that crowd the SMs go to adjoint_stage_kernel below.
 struct RegAdj {
   int region;       // elements of each of the four vector regions in shared memory
   int K, nck;       // iterations per segment, segments
@@ -760,10 +760,233 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
   }
 }
 
-// Plan of the register sweep: threads (0: some instance has n > 16 or more components than a CTA
-// holds threads), the segment length, and the workspace offsets.
+// ---- the same with a thread per stage (stage_reg.cuh): FP32, few states and inputs ----------------
+//
+// What adjoint_reg_kernel does per component a thread does for its whole stage, two barriers per
+// iteration instead of three and products without loads; also for horizons whose components a CTA has
+// no threads for. Only the matrices and the four vectors in hand stay in registers (128 a thread at 4 +
+// 1 components, so that four CTAs of 128 threads share an SM): the inputs of the forward iteration are
+// read again for every segment, and the gradient sums, as float pairs, live in shared memory, one
+// 16-byte access per component and iteration each way. The clamp sides take a 16-bit word per stage and
+// iteration.
+// What bounds it is instruction issue (62 % of the issue slots, the rest barriers and fixed latencies);
+// its chains are longer than those of a thread per component, so it wins where a batch takes that one
+// more than two rounds of CTAs (150 iterations, 1024 instances: n 5, N 100 1.60 -> 0.97 ms, N 60 1.38 ->
+// 0.54; n 3, N 60 0.79 -> 0.33; n 6, N 85 1.48 -> 1.20; n 5, N 20, 1.7 rounds, 0.36 and 0.44, so that one
+// stays, as do smaller batches: 152 of n 5, N 60 0.21 and 0.34) or does not fit.
+template <int NX, int NU, int kMinCtas>
+__global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(AdjArgs a, RegAdj ra) {
+  using M = stage::Mats<NX, NU>;
+  constexpr int NN = NX + NU;
+  extern __shared__ __align__(128) unsigned char adj_smem[];
+  const int j = a.order[blockIdx.x];
+  Inst<float> I;
+  make_inst(a, j, I);
+  const int nx = I.nx, nu = I.nu, N = I.N;
+  const int k = threadIdx.x, T = blockDim.x, ld = T + 1;
+  const bool on = k < N;
+  float4 *sh = reinterpret_cast<float4 *>(adj_smem);       // [NN][T]: sums of hbar and of hbar xbar
+  float2 *sb = reinterpret_cast<float2 *>(sh + NN * T);    // [NN][2][T]: of the adjoints at the two bounds
+  float2 *sx0 = sb + 2 * NN * T;                           // [NX]: of Abar_0^T qbar_0 (stage 0's thread)
+  float *sg = reinterpret_cast<float *>(sx0 + 4), *sx = sg + NN * ld;
+  M m;
+  m.setup(
+      nx, nu, on, I.rho, [&](int r, int c) { return I.Gv(k, r, c); }, [&](int r, int c) { return I.Hv(k, r, c); },
+      [&](int q, int i) { return I.Mv(k, q, i); });
+#pragma unroll
+  for (int p = 0; p < NN; ++p) {
+    sh[p * T + k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    sb[2 * p * T + k] = sb[(2 * p + 1) * T + k] = make_float2(0.0f, 0.0f);
+    sg[p * ld + k] = 0.0f;
+    if (k == 0) sg[p * ld + T] = 0.0f;
+    if (k == 0 && p < 4) sx0[p] = make_float2(0.0f, 0.0f);
+  }
+  // workspace: checkpoints [nck - 1][4][NN][nt], xb [K][NN][nt], sides [K][nt]
+  const int nt = (N + 31) & ~31;
+  const bool kept = k < nt;
+  float *ck = reinterpret_cast<float *>(ra.ws + ra.off[j]);
+  float *xbs = ck + (int64_t)(ra.nck - 1) * 4 * NN * nt;
+  unsigned short *sides = reinterpret_cast<unsigned short *>(xbs + (ra.keep_xb ? (int64_t)ra.K * NN * nt : 0));
+  auto inputs = [&](stage::Iter<NX, NU> &s) {
+    const float *rf = on ? I.refk(k) : nullptr;
+    s.inputs(
+        nx, nu, on, [&](int r) { return I.Ev(k, r); }, [&](int c) { return rf ? I.qd[c] * rf[c] : 0.0f; },
+        [&](int c) { return I.lo[c]; }, [&](int c) { return I.hi[c]; });
+#pragma unroll
+    for (int c = 0; c < NN; ++c) {
+      s.z[c] = s.v[c] = s.t[c] = s.b[c] = 0.0f;
+      const int i = stage::component<NX, NU>(c, nx, nu);
+      if (k == 0) sx[c * ld] = i >= 0 ? I.xb0[i] : 0.0f;  // only this thread reads slot 0
+    }
+  };
+  float xb[NN], share;
+  unsigned side;
+  if (ra.nck > 1) {  // forward to the start of the last segment, a checkpoint at the start of each but the first
+    stage::Iter<NX, NU> s;
+    inputs(s);
+    for (int seg = 1; seg < ra.nck; ++seg) {
+      for (int q = 0; q < ra.K; ++q) s.template step<false, false>(m, sg, sx, ld, k, on, false, xb, side, share);
+      if (!kept) continue;
+#pragma unroll
+      for (int c = 0; c < NN; ++c) {
+        float *o = ck + ((int64_t)(seg - 1) * 4 * NN + c) * nt + k;
+        o[0] = s.z[c]; o[NN * nt] = s.v[c]; o[2 * NN * nt] = s.t[c]; o[3 * NN * nt] = s.b[c];
+      }
+    }
+  }
+  // Adjoint of the last iterate: z = (x, u).
+  float zb[NN], vb[NN], tb[NN], bb[NN];
+#pragma unroll
+  for (int c = 0; c < NN; ++c) {
+    zb[c] = vb[c] = tb[c] = bb[c] = 0.0f;
+    const int i = on ? stage::component<NX, NU>(c, nx, nu) : -1;
+    if (i >= 0 && i < nx && a.dL_dx) zb[c] = (float)a.dL_dx[a.L.Nnx[j] + (int64_t)k * nx + i];
+    if (i >= nx && a.dL_du) zb[c] = (float)a.dL_du[a.L.Nnu[j] + (int64_t)k * nu + i - nx];
+  }
+  for (int seg = ra.nck - 1; seg >= 0; --seg) {
+    const int len = min(ra.K, a.iters - seg * ra.K);
+    {
+      stage::Iter<NX, NU> s;
+      inputs(s);
+      if (seg > 0 && kept) {
+#pragma unroll
+        for (int c = 0; c < NN; ++c) {
+          const float *o = ck + ((int64_t)(seg - 1) * 4 * NN + c) * nt + k;
+          s.z[c] = o[0]; s.v[c] = o[NN * nt]; s.t[c] = o[2 * NN * nt]; s.b[c] = o[3 * NN * nt];
+        }
+      }
+      for (int q = 0; q < len; ++q) {
+        s.template step<false, true>(m, sg, sx, ld, k, on, false, xb, side, share);
+        if (!kept) continue;
+        sides[(int64_t)q * nt + k] = (unsigned short)side;
+        if (ra.keep_xb) {
+#pragma unroll
+          for (int c = 0; c < NN; ++c) (xbs + (int64_t)q * NN * nt + k)[c * nt] = xb[c];
+        }
+      }
+    }
+    if (k == 0) {  // rho hbar of the stage before the first
+#pragma unroll
+      for (int c = 0; c < NN; ++c) sx[c * ld] = 0.0f;
+    }
+    for (int q = len - 1; q >= 0; --q) {
+      side = kept ? sides[(int64_t)q * nt + k] : 0u;
+      if (ra.keep_xb && kept) {  // loaded well before their use
+#pragma unroll
+        for (int c = 0; c < NN; ++c) xb[c] = (xbs + (int64_t)q * NN * nt + k)[c * nt];
+      }
+      float pb[NN], qb[NN], ab[NN];
+#pragma unroll
+      for (int c = 0; c < NN; ++c) {
+        const float half = 0.5f * (vb[c] - bb[c]);
+        const float zt = (zb[c] - tb[c]) + half;
+        float wb = third(zt);
+        const bool low = side >> c & 1u;
+        if (low || side >> (NN + c) & 1u) {
+          float2 &o = sb[(2 * c + (low ? 0 : 1)) * T + k];
+          Sum<float> sum;
+          sum.hi = o.x; sum.lo = o.y;
+          sum.add(zt);
+          o = make_float2(sum.hi, sum.lo);
+          wb = 0.0f;
+        }
+        pb[c] = (bb[c] + half) + wb;
+        qb[c] = wb - half;
+        tb[c] = fmaf(2.0f, wb, tb[c]);  // the adjoint of s = xb + theta
+      }
+#pragma unroll
+      for (int c = 0; c < NN; ++c) {
+        const float g = m.abar_t(qb, c);
+        if (on) sg[c * ld + k] = g;
+        if (k == 0 && c < NX) {
+          Sum<float> sum;
+          sum.hi = sx0[c].x; sum.lo = sx0[c].y;
+          sum.add(g);
+          sx0[c] = make_float2(sum.hi, sum.lo);
+        }
+      }
+      M::sym(m.P, pb, ab);
+      __syncthreads();
+      float hb[NN];
+      {
+        float xt[NN];
+#pragma unroll
+        for (int c = 0; c < NN; ++c) xt[c] = tb[c] + sg[c * ld + k + 1];
+        M::sym(m.H, xt, hb);
+      }
+#pragma unroll
+      for (int c = 0; c < NN; ++c) {
+        float4 &o = sh[c * T + k];
+        const float4 v = o;
+        Sum<float> h, x;
+        h.hi = v.x; h.lo = v.y; x.hi = v.z; x.lo = v.w;
+        h.add(hb[c]);
+        if (ra.keep_xb) x.add_product(hb[c], xb[c]);
+        o = make_float4(h.hi, h.lo, x.hi, x.lo);
+        hb[c] *= m.rho;
+        sx[c * ld + k + 1] = hb[c];
+      }
+      __syncthreads();
+      float xp[NN];
+#pragma unroll
+      for (int c = 0; c < NN; ++c) xp[c] = sx[c * ld + k];
+#pragma unroll
+      for (int c = 0; c < NN; ++c) {
+        const float yb = m.abar(xp, c, 0.0f);
+        zb[c] = hb[c] + yb;
+        vb[c] = ab[c] - yb;
+        tb[c] -= hb[c];
+        bb[c] = (pb[c] + qb[c]) - (yb + ab[c]);
+      }
+    }
+  }
+  // Gradients: sums over the stages, pairwise.
+  const float *rf = on ? I.refk(k) : nullptr;
+  int top = 1;
+  while (2 * top < N) top *= 2;
+  double *sd = reinterpret_cast<double *>(sg);  // over sg and sx
+  auto total = [&](double x) {
+    __syncthreads();
+    if (on) sd[k] = x;
+    for (int h = top; h > 0; h >>= 1) {
+      __syncthreads();
+      if (k < h && k + h < N) sd[k] += sd[k + h];
+    }
+    return sd[0];  // thread 0's use
+  };
+#pragma unroll
+  for (int c = 0; c < NN; ++c) {
+    const int i = stage::component<NX, NU>(c, nx, nu);  // uniform over the CTA
+    if (i < 0) continue;
+    const float4 v = sh[c * T + k];
+    const float2 l = sb[2 * c * T + k], u = sb[(2 * c + 1) * T + k];
+    const double qd = (double)I.qd[i], h = on ? (double)v.x + (double)v.y : 0.0, r = rf ? (double)rf[i] : 0.0;
+    if (on && a.g_ref && a.ref_per_stage) a.g_ref[a.L.Nn[j] + (int64_t)k * I.n + i] = qd * h;
+    const double gq = total(r * h - ((double)v.z + (double)v.w));
+    const double glo = total((double)l.x + (double)l.y);
+    const double ghi = total((double)u.x + (double)u.y);
+    const double gref = total(qd * h);
+    if (k == 0) {
+      if (a.g_ref && !a.ref_per_stage) a.g_ref[a.L.off_n[j] + i] = gref;
+      if (i < nx) {
+        if (a.g_q) a.g_q[a.L.off_nx[j] + i] = gq;
+        if (a.g_xmin) a.g_xmin[a.L.off_nx[j] + i] = glo;
+        if (a.g_xmax) a.g_xmax[a.L.off_nx[j] + i] = ghi;
+        if (a.g_x0) a.g_x0[a.L.off_nx[j] + i] = (double)sx0[c < NX ? c : 0].x + (double)sx0[c < NX ? c : 0].y;
+      } else {
+        if (a.g_r) a.g_r[a.L.off_nu[j] + i - nx] = gq;
+        if (a.g_umin) a.g_umin[a.L.off_nu[j] + i - nx] = glo;
+        if (a.g_umax) a.g_umax[a.L.off_nu[j] + i - nx] = ghi;
+      }
+    }
+  }
+}
+
+// Plan of the register sweeps: threads (0: some instance has n > 16, or more components than a CTA holds
+// threads and is not one for a thread per stage), the segment length, and the workspace offsets.
 struct RegAdjPlan {
   int threads = 0, NM = 0;
+  int stage_class = -1;  // >= 0: a thread per stage, of that size class
   RegAdj ra{};
   std::vector<int64_t> off;
   int64_t bytes = 0;
@@ -775,33 +998,77 @@ RegAdjPlan plan_reg_adjoint(const pimpc_solver *s, int Tn, int K, int nck, int s
   int nmax = 1, thr = 0, reg = 0;
   for (int j = 0; j < s->batch; ++j) nmax = std::max(nmax, s->nx[j] + s->nu[j]);
   if (nmax > 16 || Tn < 1) return p;
+  bool fits = true;
+  int nx = 1, nu = 1, N = 1;
   p.NM = nmax <= 4 ? 4 : (nmax <= 8 ? 8 : 16);
+  const int cap = adj_max_threads(ts, p.NM);
   for (int j = 0; j < s->batch; ++j) {
     const int n = s->nx[j] + s->nu[j];
-    if ((int64_t)n * s->N[j] > adj_max_threads(ts, p.NM)) return p;
-    thr = std::max(thr, n * s->N[j]);
-    reg = std::max(reg, (s->N[j] + 1) * reg_nv(n, ts));
+    fits = fits && (int64_t)n * s->N[j] <= cap;
+    thr = std::max(thr, fits ? n * s->N[j] : 0);
+    reg = std::max(reg, fits ? (s->N[j] + 1) * reg_nv(n, ts) : 0);
+    nx = std::max(nx, s->nx[j]);
+    nu = std::max(nu, s->nu[j]);
+    N = std::max(N, s->N[j]);
   }
+  // A thread per stage where a thread per component does not fit or leaves the batch more than two
+  // rounds of CTAs (adjoint_stage_kernel).
+  if (s->prec == PIMPC_F32 && N <= kStageThreads) {
+    int nsm = 0;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s->device);
+    if (!fits || s->batch > 2 * nsm * (cap / ((thr + 31) / 32 * 32))) p.stage_class = stage::size_class(nx, nu);
+  }
+  const bool stages = p.stage_class >= 0;
+  const int NN = stages ? stage::padded(p.stage_class) : 1;  // components kept per thread
+  if (!stages && !fits) return p;
+  if (stages) thr = N;
   p.threads = (thr + 31) / 32 * 32;
   p.ra.region = (reg + 3) / 4 * 4;
   p.ra.keep_xb = keep_xb;
   // words per component: what the other sweep takes, and what keeping every iteration takes
   const double theirs = 5.0 * (nck + slots + 1) + 4.0 + 32.0 / ts;
-  const double whole = 4.0 + Tn * ((keep_xb ? 1.0 : 0.0) + 0.25 / ts);
-  p.ra.K = whole <= theirs ? Tn : K;
-  p.ra.nck = whole <= theirs ? 1 : nck;
+  const double per_iter = (keep_xb ? 1.0 : 0.0) + (stages ? 0.5 / NN : 0.25 / ts);
+  p.ra.K = K;
+  p.ra.nck = nck;
+  if (stages) {  // the fewest segments (iterations run twice) within that memory
+    for (int m = 1; m < nck; ++m) {
+      const int Km = (Tn + m - 1) / m;
+      if (4.0 * (m - 1) + Km * per_iter > theirs) continue;
+      p.ra.K = Km;
+      p.ra.nck = (Tn + Km - 1) / Km;
+      break;
+    }
+  } else if (4.0 + Tn * per_iter <= theirs) {
+    p.ra.K = Tn;
+    p.ra.nck = 1;
+  }
   for (int j = 0; j < s->batch; ++j) {
-    const int64_t nt = ((int64_t)(s->nx[j] + s->nu[j]) * s->N[j] + 31) / 32 * 32;
+    const int64_t per = stages ? s->N[j] : (int64_t)(s->nx[j] + s->nu[j]) * s->N[j];
+    const int64_t nt = (per + 31) / 32 * 32;
     p.off.push_back(p.bytes);
-    p.bytes += ((int64_t)p.ra.nck * 4 + (keep_xb ? p.ra.K : 0)) * nt * ts +
-               (int64_t)p.ra.K * (nt / 32) * (int64_t)sizeof(uint2);
+    p.bytes += ((int64_t)(p.ra.nck - (stages ? 1 : 0)) * 4 + (keep_xb ? p.ra.K : 0)) * NN * nt * ts +
+               (int64_t)p.ra.K * (stages ? 2 * nt : (nt / 32) * (int64_t)sizeof(uint2));
     p.bytes = (p.bytes + 255) & ~(int64_t)255;
   }
   return p;
 }
 
+template <int NX, int NU, int kMinCtas>
+cudaError_t launch_stage_adjoint(const AdjArgs &a, const RegAdjPlan &p, int batch, cudaStream_t st) {
+  const size_t smem = (size_t)(NX + NU) * (32 * p.threads + 8 * (p.threads + 1)) + 4 * sizeof(float2);
+  auto kernel = adjoint_stage_kernel<NX, NU, kMinCtas>;
+  const cudaError_t rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (rc != cudaSuccess) return rc;
+  kernel<<<batch, p.threads, smem, st>>>(a, p.ra);
+  return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t launch_reg_adjoint(const AdjArgs &a, const RegAdjPlan &p, int batch, cudaStream_t st) {
+  if (p.stage_class >= 0)
+    return p.stage_class == 0   ? launch_stage_adjoint<2, 1, 3>(a, p, batch, st)
+           : p.stage_class == 1 ? launch_stage_adjoint<4, 1, 2>(a, p, batch, st)
+                                : launch_stage_adjoint<4, 2, 1>(a, p, batch, st);
   auto kernel = p.NM == 4 ? adjoint_reg_kernel<T, 4> : (p.NM == 8 ? adjoint_reg_kernel<T, 8> : adjoint_reg_kernel<T, 16>);
   const size_t smem = (size_t)4 * p.ra.region * sizeof(T);
   const cudaError_t rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

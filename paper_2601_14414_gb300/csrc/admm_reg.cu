@@ -1,5 +1,6 @@
 // admm_reg.cu -- planning of the register-resident schedule and its FP32 kernels (admm_reg.cuh).
 #include "admm_reg.cuh"
+#include "stage_reg.cuh"
 
 namespace pimpc {
 
@@ -91,8 +92,8 @@ bool plan_resident(int item_scale, int batch, const int *nx, const int *nu, cons
   if (reg->threads > 0 && precision == 0 && item_scale <= 1) {
     const int mx = *std::max_element(nx, nx + batch), mu = *std::max_element(nu, nu + batch);
     const int mN = *std::max_element(N, N + batch);
-    if (mx <= 4 && mu <= 2 && mN <= kStageThreads) {
-      reg->stage_class = mu <= 1 ? (mx <= 2 ? 0 : 1) : 2;
+    if (stage::size_class(mx, mu) >= 0 && mN <= kStageThreads) {
+      reg->stage_class = stage::size_class(mx, mu);
       reg->stage_threads = (mN + 31) / 32 * 32;
     }
   }
