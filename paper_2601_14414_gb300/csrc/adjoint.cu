@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
 // read again for every segment, and the gradient sums, as float pairs, live in shared memory, one
 // 16-byte access per component and iteration each way. The clamp sides take a 16-bit word per stage and
 // iteration.
-// What bounds it is instruction issue (62 % of the issue slots, the rest barriers and fixed latencies);
+// What bounds it is instruction issue (55 % of the issue slots, the rest barriers and fixed latencies);
 // its chains are longer than those of a thread per component, so it wins where a batch takes that one
 // more than two rounds of CTAs (150 iterations, 1024 instances: n 5, N 100 1.60 -> 0.97 ms, N 60 1.38 ->
 // 0.54; n 3, N 60 0.79 -> 0.33; n 6, N 85 1.48 -> 1.20; n 5, N 20, 1.7 rounds, 0.36 and 0.44, so that one

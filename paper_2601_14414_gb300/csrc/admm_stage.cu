@@ -3,11 +3,11 @@
 //
 // What bounds a batch of these is instruction issue, and a single one the latency of an iteration.
 // With a thread per component (admm_reg.cuh) every component loads each vector that it multiplies
-// from shared memory, and a CTA meets four times per iteration. A thread that owns a whole stage of n <= 6 components keeps G_k, the packed lower
-// triangles of H_k and P_k = Bbar_k M_k Bbar_k^T and the iterate in registers, multiplies without
-// loads, and exchanges two n-vectors with its neighbours: Abar_k^T y_k, formed by the thread that
-// holds G_k, to stage k - 1, and xbar_{k+1} to stage k + 1, two barriers in all. The iteration is the
-// reduced one of admm_reg.cuh (lambda = -beta throughout). What limits the warps of an SM is the
+// from shared memory, and a CTA meets four times per iteration. A thread that owns a whole stage of
+// n <= 6 components keeps G_k, the packed lower triangles of H_k and P_k = Bbar_k M_k Bbar_k^T and the
+// iterate in registers, multiplies without loads, and exchanges two n-vectors with its neighbours:
+// Abar_k^T y_k, formed by the thread that holds G_k, to stage k - 1, and xbar_{k+1} to stage k + 1, two
+// barriers in all. The iteration is the reduced one of admm_reg.cuh (lambda = -beta throughout). What limits the warps of an SM is the
 // registers of a thread: 71 at 2 + 1 components, 128 at 4 + 1, 167 at 4 + 2.
 // Per solve of 150 iterations, against a thread per component: 1024 instances of n 5, N 100 629 -> 244
 // us, N 20 139 -> 92, N 150 (more components than a CTA has threads: clusters of two CTAs) 3.68 -> 0.35
