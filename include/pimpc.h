@@ -399,10 +399,11 @@ int pimpc_autotune(pimpc_solver *s, int trial_iters, int *family, int *ctas_per_
  *   owned by the caller, read during the call's kernels only.
  *   rho, eps, max_iters, accel, eta  as in pimpc_set_options, with the same checks.
  *   u_out [N nu], x_out [N nx], iters[1], c[1], status[1]: DEVICE memory (any may be NULL).
- *   stream        cudaStream_t; the call only enqueues work on it.
+ *   stream        cudaStream_t; the call only enqueues work on it (the first one also waits).
  * The call allocates nothing (no cudaMalloc, no cudaFree, no allocating library call). Its
- * first call on a device looks up the array's address with cudaGetSymbolAddress and fills a
- * constant table of momentum factors; make that first call before any stream capture. Every call shares the array and rewrites or clears what
+ * first call on a device looks up the array's address with cudaGetSymbolAddress, fills a
+ * constant table of momentum factors and waits for that copy (not for the caller's stream); make
+ * that first call before any stream capture. Every call shares the array and rewrites or clears what
  * it reads, so consecutive calls are independent, but calls that overlap on the GPU race.
  * Capacity: the working memory is about N * (W + 15 n) * ts bytes (ts = 4 in FP32, 8 in FP64;
  * W = nx n + nx + n(n+1)/2 + nu(nu+1)/2 words of stage data, N rounded up to a multiple of 32),

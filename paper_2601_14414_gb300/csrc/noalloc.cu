@@ -26,10 +26,10 @@
 #include <cstdio>
 #include <mutex>
 #include <string>
-#include <vector>
 
 #include "launch.h"
 #include "pimpc.h"
+#include "static_arrays.h"
 
 namespace pimpc {
 void set_thread_error(const std::string &msg);
@@ -44,16 +44,26 @@ namespace {
 constexpr size_t kStaticBytes = (size_t)16 << 20;  // 16 MiB, documented in include/pimpc.h
 __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
-// Momentum factors (alpha_m - 1) / alpha_{m+1} of Algorithm 1 step 6 after m consecutive momentum
-// steps, alpha_0 = 1, alpha_{m+1} = (1 + sqrt(1 + 4 alpha_m^2)) / 2, rounded as the device rounds
-// them (multiply-adds fused).
-constexpr int kCoefs = 4096;
+constexpr int kCoefs = 4096;  // entries of the momentum table (static_arrays.h)
 __device__ double g_coef_table[kCoefs];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
-void *g_scratch_ptr[kMaxDevices] = {};
-double *g_coef_ptr[kMaxDevices] = {};
+StaticArrays g_arrays[kMaxDevices];
+
+struct Runtime {
+  int scratch(void **p) { return cudaGetSymbolAddress(p, g_static_scratch); }
+  int table(double **p) {
+    void *t = nullptr;
+    const cudaError_t rc = cudaGetSymbolAddress(&t, g_coef_table);
+    *p = (double *)t;
+    return rc;
+  }
+  int copy(double *dst, const double *src, int count) {
+    return cudaMemcpyAsync(dst, src, sizeof(double) * count, cudaMemcpyHostToDevice, cudaStreamPerThread);
+  }
+  int wait() { return cudaStreamSynchronize(cudaStreamPerThread); }
+};
 
 // Device addresses of the static array and of the momentum table on the current device (looked
 // up, and the table filled, once per device).
@@ -63,27 +73,11 @@ cudaError_t scratch_address(void **out, const double **coefs) {
   if (rc != cudaSuccess) return rc;
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(g_mu);
-  if (!g_scratch_ptr[dev]) {
-    void *p = nullptr;
-    rc = cudaGetSymbolAddress(&p, g_static_scratch);
-    if (rc != cudaSuccess) return rc;
-    void *t = nullptr;
-    rc = cudaGetSymbolAddress(&t, g_coef_table);
-    if (rc != cudaSuccess) return rc;
-    std::vector<double> tab(kCoefs);
-    double al = 1.0;
-    for (int m = 0; m < kCoefs; ++m) {
-      const double an = std::fma(0.5, std::sqrt(std::fma(4.0 * al, al, 1.0)), 0.5);
-      tab[m] = (al - 1.0) / an;
-      al = an;
-    }
-    rc = cudaMemcpy(t, tab.data(), sizeof(double) * kCoefs, cudaMemcpyHostToDevice);
-    if (rc != cudaSuccess) return rc;
-    g_coef_ptr[dev] = (double *)t;
-    g_scratch_ptr[dev] = p;
-  }
-  *out = g_scratch_ptr[dev];
-  *coefs = g_coef_ptr[dev];
+  Runtime rt;
+  rc = (cudaError_t)ensure_static_arrays(rt, g_arrays[dev], kCoefs);
+  if (rc != cudaSuccess) return rc;
+  *out = g_arrays[dev].scratch;
+  *coefs = g_arrays[dev].coefs;
   return cudaSuccess;
 }
 
