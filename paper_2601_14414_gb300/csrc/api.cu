@@ -108,8 +108,8 @@ void free_layout(pimpc_solver *s) {
   s->lay_allocs.clear();
   s->blk_T = nullptr;
   for (int b = 0; b < 3; ++b) s->it[b] = nullptr;
-  s->item_inst = s->item_a = s->item_b = s->list0 = s->list1 = s->item_first = nullptr;
-  s->list_init = s->ccount = s->pos_of = nullptr;
+  s->work = s->work_lanes = WorkList{};
+  s->list0 = s->list1 = s->ccount = s->pos_of = nullptr;
   s->cpart = nullptr;
 }
 
@@ -126,6 +126,45 @@ cudaError_t lalloc(pimpc_solver *s, P **p, size_t bytes) {
 }  // namespace
 
 namespace pimpc {
+
+// A work list on the host: items (instance, first stage, end) with an instance's items consecutive,
+// the coarse ones, then the fine ones.
+struct Items {
+  std::vector<int> inst, a, b;
+  std::vector<int> count;     // [2 batch] coarse, then fine items of each instance
+  std::vector<int> fine_len;  // [batch] stages per fine item (0: no fine items)
+  std::vector<int> first;     // [2 batch] first coarse, then first fine item of each instance
+  std::vector<int> init;      // [coarse items] starting order: longest first
+  int coarse = 0;
+  explicit Items(int batch) : count(2 * batch, 0), fine_len(batch, 0), first(2 * batch, 0) {}
+
+  // After the coarse items: the fine ones and the per-instance ranges (the finish pass of an iteration
+  // sums an instance's shares of c over [first, first + count)). volume: what a stage streams.
+  template <typename F>
+  bool finish(const std::vector<int> &order, const std::vector<int> &N, F volume) {
+    const int batch = (int)fine_len.size();
+    coarse = (int)inst.size();
+    for (int j : order)
+      for (int a0 = 0; fine_len[j] > 0 && a0 < N[j]; a0 += fine_len[j]) {
+        inst.push_back(j);
+        a.push_back(a0);
+        b.push_back(std::min(N[j], a0 + fine_len[j]));
+        count[batch + j] += 1;
+      }
+    const int all = (int)inst.size();
+    for (int i = all - 1; i >= 0; --i) first[inst[i] + (i >= coarse ? batch : 0)] = i;
+    for (int i = 0; i < all; ++i) {
+      const int j = inst[i] + (i >= coarse ? batch : 0);
+      if (i >= first[j] + count[j]) return false;
+    }
+    std::vector<double> cost(coarse);
+    for (int i = 0; i < coarse; ++i) cost[i] = volume(inst[i]) * (double)(b[i] - a[i]);
+    init.resize(coarse);
+    std::iota(init.begin(), init.end(), 0);
+    std::stable_sort(init.begin(), init.end(), [&](int x, int y) { return cost[x] > cost[y]; });
+    return true;
+  }
+};
 
 // Lays out the stage blocks and iterates for a schedule, plans the solve kernel's launch and
 // work items, and (re)allocates the buffers that depend on them. The iterates restart from zero
@@ -185,9 +224,9 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
   int64_t tot_blk = 0, tot_Ni = 0;
   AdmmLaunch P{};
   // Items: the coarse ones, then (lane-group families, stage-varying batches) the fine ones of
-  // one sub-chunk each, which the solve switches to when few instances are left.
-  std::vector<int> item_inst, item_a, item_b, nitems_inst(2 * batch, 0);
-  std::vector<int> fine_len(batch, 0);  // stages per fine item (0: no fine items)
+  // one sub-chunk each, which the solve switches to when few instances are left. `lanes`: the FP64
+  // lane groups' own where the full-warp kernel has the others (empty: not needed).
+  Items items(batch), lanes(batch);
   const int fine_sub = 1;                 // sub-chunks per fine item
   const int fine_switch = 1;              // fine items below this many coarse items per CTA
   // Instance order: largest streamed volume first.
@@ -240,10 +279,10 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
     for (int oi = 0; oi < batch; ++oi) {
       const int j = order[oi];
       for (int a0 = 0; a0 < N[j]; a0 += inner[j]) {
-        item_inst.push_back(j);
-        item_a.push_back(a0);
-        item_b.push_back(std::min(N[j], a0 + inner[j]));
-        nitems_inst[j] += 1;
+        items.inst.push_back(j);
+        items.a.push_back(a0);
+        items.b.push_back(std::min(N[j], a0 + inner[j]));
+        items.count[j] += 1;
       }
     }
     size_t smem = 0;
@@ -277,10 +316,10 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
     for (int oi = 0; oi < batch; ++oi) {
       const int j = order[oi];
       for (int a0 = 0; a0 < N[j]; a0 += 127 * tpi) {
-        item_inst.push_back(j);
-        item_a.push_back(a0);
-        item_b.push_back(std::min(N[j], a0 + 127 * tpi));
-        nitems_inst[j] += 1;
+        items.inst.push_back(j);
+        items.a.push_back(a0);
+        items.b.push_back(std::min(N[j], a0 + 127 * tpi));
+        items.count[j] += 1;
       }
     }
     P.threads = tc_threads();
@@ -317,10 +356,10 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
     for (int oi = 0; oi < batch; ++oi) {
       const int j = order[oi];
       for (int a0 = 0; a0 < N[j]; a0 += LBi * per_item) {
-        item_inst.push_back(j);
-        item_a.push_back(a0);
-        item_b.push_back(std::min(N[j], a0 + LBi * per_item));
-        nitems_inst[j] += 1;
+        items.inst.push_back(j);
+        items.a.push_back(a0);
+        items.b.push_back(std::min(N[j], a0 + LBi * per_item));
+        items.count[j] += 1;
       }
     }
     P.threads = gemm_threads();
@@ -394,12 +433,12 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
         const int P1 = grp[j] - 1;
         int is = (int)(P1 * m);
         if (lti) is = std::max(is, std::min(N[j], (256 + P1 - 1) / P1 * P1));
-        if (!lti && m > fine_sub) fine_len[j] = P1 * fine_sub;
+        if (!lti && m > fine_sub) items.fine_len[j] = P1 * fine_sub;
         for (int a0 = 0; a0 < N[j]; a0 += is) {
-          item_inst.push_back(j);
-          item_a.push_back(a0);
-          item_b.push_back(std::min(N[j], a0 + is));
-          nitems_inst[j] += 1;
+          items.inst.push_back(j);
+          items.a.push_back(a0);
+          items.b.push_back(std::min(N[j], a0 + is));
+          items.count[j] += 1;
         }
       }
     }
@@ -440,10 +479,10 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
       const int nt = halo_tiles(N[j], tw[j]);
       const int m = (int)std::max<int64_t>(1, std::min<int64_t>(max_tiles, D / tile_bytes(j, tw[j])));
       for (int t0 = 0; t0 < nt; t0 += m) {
-        item_inst.push_back(j);
-        item_a.push_back(t0);
-        item_b.push_back(std::min(nt, t0 + m));
-        nitems_inst[j] += 1;
+        items.inst.push_back(j);
+        items.a.push_back(t0);
+        items.b.push_back(std::min(nt, t0 + m));
+        items.count[j] += 1;
       }
     }
     P.threads = tile_threads();
@@ -453,7 +492,7 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
   } else {
     const int threads = admm_threads(precision);
     int nv_max = 2, W_max = 4, n5p_max = 4, scr_max = 4, xrows_max = 4;
-    int64_t capB = 0, capI = 0, total_sub = 0;
+    int64_t capB = 0, capI = 0;
     for (int j = 0; j < batch; ++j) {
       const int n = nx[j] + nu[j];
       const int n5p = admm_iter_stride(n, precision);
@@ -475,7 +514,6 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
         capB = std::max<int64_t>(capB, (int64_t)S * W[j] + ge);
       }
       capI = std::max<int64_t>(capI, (int64_t)(S + 1) * n5p);
-      total_sub += (N[j] + S - 1) / S;
     }
     P.threads = threads;
     P.capB = (int)capB;
@@ -508,28 +546,36 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
                    s->dense_plan, &s->dense_smem))
       e = dense_configure(s->dense_smem, &dense_bps);
     s->dense_grid = dense_bps * nsm;
-    if (dense_bps > 0) {
-      total_sub = 0;
-      for (int j = 0; j < batch; ++j) total_sub += (N[j] + grp[j] - 2) / (grp[j] - 1);
-    }
-    if (e == cudaSuccess && bps >= 1) {
-      const int64_t max_grid = dense_bps > 0 ? s->dense_grid : (int64_t)bps * nsm;
+    // Items of whole sub-chunks (`stages` of an instance each): the two FP64 kernels have sub-chunks of
+    // their own, and an item cut for the other one leaves SMs idle or sub-chunks part-filled.
+    auto cut = [&](Items &w, int64_t max_grid, auto stages) {
+      int64_t total = 0;
+      for (int j = 0; j < batch; ++j) total += (N[j] + stages(j) - 1) / stages(j);
       // Sub-chunks per item: enough items for about 4 per CTA, at most 16 sub-chunks per item.
-      int64_t m = sc.item_scale > 0 ? sc.item_scale : total_sub / (4 * max_grid);
+      int64_t m = sc.item_scale > 0 ? sc.item_scale : total / (4 * max_grid);
       m = std::max<int64_t>(1, std::min<int64_t>(sc.item_scale > 0 ? 64 : 16, m));
       for (int oi = 0; oi < batch; ++oi) {
         const int j = order[oi];
-        const int n = nx[j] + nu[j];
-        const int S = dense_bps > 0 ? grp[j] - 1 : threads / admm_group_size(n);
+        const int S = stages(j);
         int is = (int)(S * m);
         if (lti) is = std::max(is, std::min(N[j], (256 + S - 1) / S * S));
-        if (!lti && m > fine_sub) fine_len[j] = S * fine_sub;
+        if (!lti && m > fine_sub) w.fine_len[j] = S * fine_sub;
         for (int a0 = 0; a0 < N[j]; a0 += is) {
-          item_inst.push_back(j);
-          item_a.push_back(a0);
-          item_b.push_back(std::min(N[j], a0 + is));
-          nitems_inst[j] += 1;
+          w.inst.push_back(j);
+          w.a.push_back(a0);
+          w.b.push_back(std::min(N[j], a0 + is));
+          w.count[j] += 1;
         }
+      }
+    };
+    if (e == cudaSuccess && bps >= 1) {
+      auto in_lanes = [&](int j) { return threads / admm_group_size(nx[j] + nu[j]); };
+      const int64_t max_grid = (int64_t)bps * nsm;
+      if (dense_bps > 0) {
+        cut(items, s->dense_grid, [&](int j) { return grp[j] - 1; });
+        cut(lanes, max_grid, in_lanes);
+      } else {
+        cut(items, max_grid, in_lanes);
       }
     }
   }
@@ -538,45 +584,19 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
           (e != cudaSuccess ? cudaGetErrorString(e) : "zero occupancy");
     return PIMPC_ECUDA;
   }
-  const int nitems = (int)item_inst.size();
-  const int grid = (int)std::min<int64_t>((int64_t)bps * nsm, nitems);
+  const int nitems = (int)items.inst.size(), nitems_lanes = (int)lanes.inst.size();
+  const int grid = (int)std::min<int64_t>((int64_t)bps * nsm, nitems_lanes > 0 ? nitems_lanes : nitems);
   if (sc.family != 0) s->dense_grid = 0;
   s->dense_grid = std::min(s->dense_grid, nitems);
-  for (int oi = 0; oi < batch; ++oi) {
-    const int j = order[oi];
-    if (fine_len[j] <= 0) continue;
-    for (int a0 = 0; a0 < N[j]; a0 += fine_len[j]) {
-      item_inst.push_back(j);
-      item_a.push_back(a0);
-      item_b.push_back(std::min(N[j], a0 + fine_len[j]));
-      nitems_inst[batch + j] += 1;
-    }
-  }
-  const int nall = (int)item_inst.size();
-  // The items of an instance are consecutive (coarse ones, then fine ones): the per-iteration
-  // finish pass sums an instance's shares of c over [first, first + count).
-  std::vector<int> item_first(2 * batch, 0);
-  for (int i = nall - 1; i >= 0; --i) item_first[item_inst[i] + (i >= nitems ? batch : 0)] = i;
-  for (int i = 0; i < nall; ++i) {
-    const int j = item_inst[i], f = i >= nitems ? batch : 0;
-    if (i >= item_first[j + f] + nitems_inst[j + f]) {
+  // The active list starts with the coarse items longest first (streamed volume), so that the
+  // queue hands out the long items first and the short ones fill the end of the iteration.
+  for (Items *w : {&items, &lanes}) {
+    if (!w->finish(order, N, [&](int j) { return cost[j] / (double)N[j]; })) {
       why = "internal: the items of an instance are not consecutive";
       return PIMPC_EINVAL;
     }
   }
-  // The active list starts with the coarse items longest first (streamed volume), so that the
-  // queue hands out the long items first and the short ones fill the end of the iteration.
-  std::vector<int> list_init(nitems);
-  std::iota(list_init.begin(), list_init.end(), 0);
-  {
-    std::vector<double> icost(nitems);
-    for (int i = 0; i < nitems; ++i) {
-      const int j = item_inst[i];
-      icost[i] = cost[j] / (double)N[j] * (double)(item_b[i] - item_a[i]);
-    }
-    std::stable_sort(list_init.begin(), list_init.end(),
-                     [&](int x, int y) { return icost[x] > icost[y]; });
-  }
+  const int nall = (int)std::max(items.inst.size(), lanes.inst.size());
 
   // (Re)allocate and upload what depends on the schedule.
   cudaDeviceSynchronize();
@@ -588,14 +608,23 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
   int *d_W = nullptr, *d_tw = nullptr, *d_grp = nullptr;
   chk(lalloc(s, &s->blk_T, ts * tot_blk));
   for (int b = 0; b < 3; ++b) chk(lalloc(s, &s->it[b], ts * tot_Ni));
-  chk(lalloc(s, &s->item_inst, sizeof(int) * nall));
-  chk(lalloc(s, &s->item_a, sizeof(int) * nall));
-  chk(lalloc(s, &s->item_b, sizeof(int) * nall));
+  for (auto [w, d] : {std::pair{&items, &s->work}, std::pair{&lanes, &s->work_lanes}}) {
+    *d = WorkList{};
+    if (w->inst.empty()) continue;
+    d->nitems = w->coarse;
+    d->nfine = (int)w->inst.size() - w->coarse;
+    for (auto [h, p] : {std::pair{&w->inst, &d->item_inst}, std::pair{&w->a, &d->item_a},
+                        std::pair{&w->b, &d->item_b}, std::pair{&w->first, &d->item_first},
+                        std::pair{&w->count, &d->nitems_inst}, std::pair{&w->init, &d->list_init}}) {
+      chk(lalloc(s, p, sizeof(int) * h->size()));
+      if (e == cudaSuccess) chk(cudaMemcpy(*p, h->data(), sizeof(int) * h->size(), cudaMemcpyHostToDevice));
+    }
+  }
+  s->work.grid = s->dense_grid > 0 ? s->dense_grid : grid;
+  s->work_lanes.grid = grid;
   chk(lalloc(s, &s->list0, sizeof(int) * nall));
   chk(lalloc(s, &s->list1, sizeof(int) * nall));
-  chk(lalloc(s, &s->item_first, sizeof(int) * 2 * batch));
   chk(lalloc(s, &s->cpart, sizeof(double) * nall));
-  chk(lalloc(s, &s->list_init, sizeof(int) * std::max(nitems, 1)));
   chk(lalloc(s, &s->ccount, sizeof(int) * std::max({grid, s->dense_grid, 1})));
   chk(lalloc(s, &s->pos_of, sizeof(int) * nall));
   chk(lalloc(s, &d_blk, sizeof(int64_t) * batch));
@@ -618,13 +647,7 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
     (void)cudaGetLastError();
     return oom ? PIMPC_ENOMEM : PIMPC_ECUDA;
   }
-  chk(cudaMemcpy(s->item_inst, item_inst.data(), sizeof(int) * nall, cudaMemcpyHostToDevice));
-  chk(cudaMemcpy(s->item_a, item_a.data(), sizeof(int) * nall, cudaMemcpyHostToDevice));
-  chk(cudaMemcpy(s->item_b, item_b.data(), sizeof(int) * nall, cudaMemcpyHostToDevice));
-  chk(cudaMemcpy(s->nitems_inst, nitems_inst.data(), sizeof(int) * 2 * batch, cudaMemcpyHostToDevice));
-  chk(cudaMemcpy(s->item_first, item_first.data(), sizeof(int) * 2 * batch, cudaMemcpyHostToDevice));
   chk(cudaMemset(s->cpart, 0, sizeof(double) * nall));
-  chk(cudaMemcpy(s->list_init, list_init.data(), sizeof(int) * nitems, cudaMemcpyHostToDevice));
   chk(cudaMemcpy(d_blk, blk.data(), sizeof(int64_t) * batch, cudaMemcpyHostToDevice));
   chk(cudaMemcpy(d_Ni, Ni.data(), sizeof(int64_t) * batch, cudaMemcpyHostToDevice));
   chk(cudaMemcpy(d_W, W.data(), sizeof(int) * batch, cudaMemcpyHostToDevice));
@@ -647,12 +670,7 @@ int apply_schedule(pimpc_solver *s, const Schedule &sc_in, std::string &why) {
   s->Ni = Ni;
   s->tot_blk = tot_blk;
   s->tot_Ni = tot_Ni;
-  s->nitems = nitems;
-  s->grid_admm = grid;
-  P.grid = grid;
   P.grp = d_grp;
-  P.nfine_base = nitems;
-  P.nfine = nall - nitems;
   P.fine_switch = fine_switch;
   s->plan = P;
   s->sched = sc;
@@ -690,10 +708,13 @@ int run_solve(pimpc_solver *s, const double *dx0, const double *dup, const doubl
   a.lo = s->lo_T; a.hi = s->hi_T; a.xb0 = s->xb0_T;
   a.rho = s->rho; a.eps = s->eps; a.eta = s->eta; a.max_iters = s->max_iters; a.accel = s->accel;
   a.mask = s->mask; a.mask_len = s->mask_len;
-  a.item_inst = s->item_inst; a.item_a = s->item_a; a.item_b = s->item_b;
-  a.nitems_inst = s->nitems_inst; a.nitems = s->nitems;
-  a.item_first = s->item_first; a.cpart = s->cpart;
-  a.list_init = s->list_init; a.ccount = s->ccount; a.pos_of = s->pos_of;
+  const WorkList &w = s->active_work();
+  a.item_inst = w.item_inst; a.item_a = w.item_a; a.item_b = w.item_b;
+  a.nitems_inst = w.nitems_inst; a.nitems = w.nitems;
+  a.nfine_base = w.nitems; a.nfine = w.nfine;
+  a.item_first = w.item_first; a.list_init = w.list_init;
+  a.grid = w.grid;
+  a.cpart = s->cpart; a.ccount = s->ccount; a.pos_of = s->pos_of;
   a.list0 = s->list0; a.list1 = s->list1; a.ctl = s->ctl;
   a.base = s->base; a.old_base = s->old_base; a.st = s->st;
   a.alpha = s->alpha; a.cprev = s->cprev; a.coef = s->coef; a.cacc = s->cacc;
@@ -718,11 +739,8 @@ int run_solve(pimpc_solver *s, const double *dx0, const double *dup, const doubl
     return fail(s, PIMPC_ESTATE, "momentum table shorter than max_iters");
   if (s->sched.family == 7 && s->accel)
     return fail(s, PIMPC_ESTATE, "temporal blocking (schedule 7) runs the plain iteration: accel must be 0");
-  const bool dense = s->sched.family == 0 && s->dense_grid > 0 && !s->any_uset;
-  if (dense) {
-    a.grid = s->dense_grid;
-    a.threads = dense_threads();
-  }
+  const bool dense = s->runs_dense();
+  if (dense) a.threads = dense_threads();
   PIMPC_CHECK(s, dense ? launch_dense(a, s->dense_plan, s->dense_smem, st)
                  : s->tiled == 2 ? launch_tile(a, st)
                  : s->tiled == 3 ? launch_blk(a, s->prec, s->smem_admm, st)
@@ -1000,7 +1018,6 @@ int pimpc_create(int batch, const int *nx, const int *nu, const int *N, int lti,
   chk(dalloc(s, &s->itfirst, sizeof(int) * batch));
   chk(dalloc(s, &s->ndone, sizeof(int) * batch));
   chk(dalloc(s, &s->stop, sizeof(int) * batch));
-  chk(dalloc(s, &s->nitems_inst, sizeof(int) * 2 * batch));
   chk(dalloc(s, &s->ctl, sizeof(Ctl)));
   chk(dalloc(s, &s->binst, sizeof(int) * s->nblocks));
   chk(dalloc(s, &s->ferr, sizeof(int) * (size_t)batch));

@@ -6,6 +6,17 @@
 
 #include "launch.h"
 
+namespace pimpc {
+// The items of a solve on the device: the coarse ones, then nfine fine ones.
+struct WorkList {
+  int *item_inst = nullptr, *item_a = nullptr, *item_b = nullptr;
+  int *item_first = nullptr;   // [2 batch] first coarse / fine item of each instance
+  int *nitems_inst = nullptr;  // [2 batch] how many of them
+  int *list_init = nullptr;    // [coarse items] starting order of the active list
+  int nitems = 0, nfine = 0, grid = 0;
+};
+}  // namespace pimpc
+
 struct pimpc_solver {
   int device = 0, batch = 0, lti = 0, prec = 0, tiled = 1;
   std::vector<int> nx, nu, N, W, tw;
@@ -35,11 +46,9 @@ struct pimpc_solver {
   int *base = nullptr, *old_base = nullptr, *binst = nullptr, *ferr = nullptr;  // ferr: [batch]
   double *alpha = nullptr, *cprev = nullptr, *coef = nullptr, *cacc = nullptr;
   int *ndone = nullptr, *stop = nullptr;
-  int *item_inst = nullptr, *item_a = nullptr, *item_b = nullptr, *nitems_inst = nullptr;
+  pimpc::WorkList work, work_lanes;  // work_lanes: of the lane groups where the full-warp kernel has `work`
   int *list0 = nullptr, *list1 = nullptr;
-  int *item_first = nullptr;  // [2 batch] first coarse / fine item of each instance
   double *cpart = nullptr;    // [items] per-item share of c of the current iteration
-  int *list_init = nullptr;   // [coarse items] starting order of the active list
   int *ccount = nullptr;      // [grid] per-CTA counts of the order-keeping compaction
   int *pos_of = nullptr;      // [items] position of each item in the active list
   pimpc::Ctl *ctl = nullptr;
@@ -63,7 +72,6 @@ struct pimpc_solver {
   void *uset_r_T = nullptr, *uset_a_T = nullptr;
   std::vector<int> uset_kind_h;
   std::vector<double> uset_r_h, uset_a_h;  // r [batch], a [sum nu]
-  int nitems = 0;
   // options and state
   double rho = 1.0, eps = 1e-6, eta = 0.999;
   int max_iters = 1000, accel = 1;
@@ -71,7 +79,6 @@ struct pimpc_solver {
   int last_ref_per_stage = 0, last_ref_given = 0, last_warm = 0, last_accel = 0, last_iters_fixed = 0;
   double last_eps = 0.0;
   size_t smem_admm = 0;
-  int grid_admm = 0;
   pimpc::AdmmLaunch plan{};
   std::string err;
   // FP64 polish: FP64 bounds, options, and the FP64 solver that runs the polish iterations
@@ -97,6 +104,10 @@ struct pimpc_solver {
   // adjoint workspace (allocated by the first pimpc_backward)
   void *adj_ws = nullptr;
   size_t adj_ws_bytes = 0;
+
+  // FP64 iterations on plain blocks: the full-warp kernel, or the lane groups while an input set is on.
+  bool runs_dense() const { return sched.family == 0 && dense_grid > 0 && !any_uset; }
+  const pimpc::WorkList &active_work() const { return dense_grid > 0 && any_uset ? work_lanes : work; }
 };
 
 namespace pimpc {

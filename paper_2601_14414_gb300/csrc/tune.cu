@@ -44,10 +44,9 @@ int pimpc_get_schedule(pimpc_solver *s, int *family, int *ctas_per_sm, int *item
   if (family) *family = s->sched.family;
   if (ctas_per_sm) *ctas_per_sm = s->sched.ctas_per_sm;
   if (item_scale) *item_scale = s->sched.item_scale;
-  const bool dense = s->sched.family == 0 && s->dense_grid > 0 && !s->any_uset;
-  if (grid) *grid = dense ? s->dense_grid : s->grid_admm;
-  if (threads) *threads = dense ? dense_threads() : s->plan.threads;
-  if (items) *items = s->nitems;
+  if (grid) *grid = s->active_work().grid;
+  if (threads) *threads = s->runs_dense() ? dense_threads() : s->plan.threads;
+  if (items) *items = s->active_work().nitems;
   return PIMPC_OK;
 }
 
