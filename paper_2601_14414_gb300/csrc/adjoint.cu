@@ -505,11 +505,11 @@ __global__ void __launch_bounds__(256) adjoint_kernel(AdjArgs a) {
 // linear but for the clamp, so all it needs of the forward iteration is which side each component
 // was clamped to (two bits) and, for the weights' gradient, xb. Both are kept for a whole segment
 // (every iteration at once when that takes no more memory than the checkpoints and states of the
-// sweep above), in place of K full states. Gradient sums run in FP64 for FP64 iterations and as
-// unevaluated float pairs (48 bits, error-free additions) for FP32 ones: three FP64 additions per
-// thread and iteration would take longer than the iteration. What bounds it is the issue rate of one
-// CTA of 512 threads per SM between three barriers per iteration; two CTAs per SM (64 registers,
-// spills) took 1.87 ms. Batches that crowd the SMs go to adjoint_stage_kernel below.
+// sweep above), in place of K full states. The gradient sums run in FP64, as above: three additions per
+// thread and iteration, 4 % of an FP32 iteration here (1300 -> 1353 us, 600 instances of n 16, N 30,
+// against sums in float pairs, which lose FP64's range and its last five bits). What bounds it is the
+// issue rate of one CTA of 512 threads per SM between three barriers per iteration; two CTAs per SM (64
+// registers, spills) took 1.17 times as long. Batches that crowd the SMs go to adjoint_stage_kernel below.
 struct RegAdj {
   int region;       // elements of each of the four vector regions in shared memory
   int K, nck;       // iterations per segment, segments
@@ -518,30 +518,19 @@ struct RegAdj {
   unsigned char *ws;   // per instance: nck states of 4 vectors, K x xb, K x clamp bits
 };
 
-template <typename T>
-struct Sum;
-template <>
-struct Sum<double> {
-  double v = 0.0;
-  __device__ __forceinline__ void add(double x) { v += x; }
-  __device__ __forceinline__ void add_product(double x, double y) { v = fma(x, y, v); }
-  __device__ __forceinline__ double value() const { return v; }
-};
-template <>
-struct Sum<float> {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float x) {  // Knuth's two-sum
-    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
-    hi = s;
-  }
-  __device__ __forceinline__ void add_product(float x, float y) {
-    const float p = __fmul_rn(x, y);
-    add(p);
-    lo = __fadd_rn(lo, fmaf(x, y, -p));
-  }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
+// (double)v in integer operations: a conversion takes the FP64 pipe's issue slots as an addition does, and
+// a branch around the values that are not normal keeps the sums of a thread's components one after the
+// other (training batch below: 1.57 ms with conversions, 1.59 with a branch, 1.14 so).
+__device__ __forceinline__ double widened(float v) {
+  const bool small = fabsf(v) < 0x1p-126f;  // zero or subnormal: made normal by a power of two
+  const float f = small ? v * 0x1p25f : v;
+  const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+  unsigned bias = small ? (1023u - 127u - 25u) << 20 : (1023u - 127u) << 20;
+  if (m >= 0x7f800000u) bias = (2047u - 255u) << 20;  // infinite or NaN
+  const unsigned hi = m == 0u ? 0u : (m >> 3) + bias;
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widened(double v) { return v; }
 
 __host__ __device__ constexpr int adj_max_threads(int tsize, int NM) {
   return tsize == 4 ? 512 : (NM <= 8 ? 512 : 256);
@@ -666,7 +655,7 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
     if (c < nx) zb = a.dL_dx ? (T)a.dL_dx[a.L.Nnx[j] + (int64_t)k * nx + c] : (T)0;
     else zb = a.dL_du ? (T)a.dL_du[a.L.Nnu[j] + (int64_t)k * nu + c - nx] : (T)0;
   }
-  Sum<T> hs, hx, los, his, x0s;
+  double hs = 0.0, hx = 0.0, los = 0.0, his = 0.0, x0s = 0.0;
   for (int seg = last; seg >= 0; --seg) {
     const int len = min(ra.K, a.iters - seg * ra.K);
     if (seg < last && kept) {
@@ -682,9 +671,13 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
       const T half = (T)0.5 * (vb - bb);
       const T zt = (zb - tb) + half;
       T wb = (T)0;
-      if (below) los.add(zt);
-      else if (above) his.add(zt);
-      else wb = third(zt);
+      if (below || above) {  // one addition for both sides
+        const double sum = (below ? los : his) + widened(zt);
+        if (below) los = sum;
+        else his = sum;
+      } else {
+        wb = third(zt);
+      }
       const T pb = (bb + half) + wb, qb = wb - half, sb = tb + (T)2 * wb;
       if (on) {
         s0[at] = pb;
@@ -703,15 +696,16 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
         if (k == 0 && c < nx) {
           T g = (T)0;
           for (int r = 0; r < nx; ++r) g += sG0[r][c] * s1[r];
-          x0s.add(g);
+          x0s += widened(g);
         }
       }
       __syncthreads();
       T rh = (T)0;
       if (on) {
         const T hb = dot(Hr, s2 + row, n, (T)0);
-        hs.add(hb);
-        hx.add_product(hb, xb);
+        const double hd = widened(hb);
+        hs += hd;
+        if (ra.keep_xb) hx = fma(hd, widened(xb), hx);
         rh = rho * hb;
         s3[at + nv] = rh;  // row k + 1, read by stage k + 1
       }
@@ -726,7 +720,7 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
   }
 
   // Gradients: sums over the stages, pairwise.
-  const double qd = on ? (double)I.qd[c] : 0.0, h = hs.value();
+  const double qd = on ? (double)I.qd[c] : 0.0, h = hs;
   double *sd = reinterpret_cast<double *>(adj_smem);
   if (on && a.g_ref && a.ref_per_stage) a.g_ref[a.L.Nn[j] + (int64_t)k * n + c] = qd * h;
   int top = 1;
@@ -740,9 +734,9 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
     }
     return sd[tid < n ? tid : 0];
   };
-  const double gq = total((double)rv * h - hx.value());
-  const double glo = total(los.value());
-  const double ghi = total(his.value());
+  const double gq = total((double)rv * h - hx);
+  const double glo = total(los);
+  const double ghi = total(his);
   const double gref = total(qd * h);
   if (tid < n) {
     if (a.g_ref && !a.ref_per_stage) a.g_ref[a.L.off_n[j] + c] = gref;
@@ -750,7 +744,7 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
       if (a.g_q) a.g_q[a.L.off_nx[j] + c] = gq;
       if (a.g_xmin) a.g_xmin[a.L.off_nx[j] + c] = glo;
       if (a.g_xmax) a.g_xmax[a.L.off_nx[j] + c] = ghi;
-      if (a.g_x0) a.g_x0[a.L.off_nx[j] + c] = x0s.value();
+      if (a.g_x0) a.g_x0[a.L.off_nx[j] + c] = x0s;
     } else {
       const int q = c - nx;
       if (a.g_r) a.g_r[a.L.off_nu[j] + q] = gq;
@@ -766,14 +760,15 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
 // iteration instead of three and products without loads; also for horizons whose components a CTA has
 // no threads for. Only the matrices and the four vectors in hand stay in registers (128 a thread at 4 +
 // 1 components, so that four CTAs of 128 threads share an SM): the inputs of the forward iteration are
-// read again for every segment, and the gradient sums, as float pairs, live in shared memory, one
-// 16-byte access per component and iteration each way. The clamp sides take a 16-bit word per stage and
-// iteration.
-// What bounds it is instruction issue (55 % of the issue slots, the rest barriers and fixed latencies);
-// its chains are longer than those of a thread per component, so it wins where a batch takes that one
-// more than two rounds of CTAs (150 iterations, 1024 instances: n 5, N 100 1.60 -> 0.97 ms, N 60 1.38 ->
-// 0.54; n 3, N 60 0.79 -> 0.33; n 6, N 85 1.48 -> 1.20; n 5, N 20, 1.7 rounds, 0.36 and 0.44, so that one
-// stays, as do smaller batches: 152 of n 5, N 60 0.21 and 0.34) or does not fit.
+// read again for every segment, and the FP64 gradient sums live in shared memory, one 16-byte access per
+// component and iteration each way. The clamp sides take a 16-bit word per stage and iteration.
+// What bounds it is instruction issue, then the FP64 pipe, which ten sums per warp and iteration take for
+// 190 cycles of the SM's (training batch, 1024 of n 5, N 100, 150 iterations: 1.13 ms, 0.97 with sums in
+// float pairs); its chains are longer than those of a thread per component, so it wins where a batch takes
+// that one more than two rounds of CTAs (100 iterations, 1024 instances, thread per component and per
+// stage: n 5, N 100 1.21 and 0.79 ms, N 60 0.98 and 0.42; n 3, N 60 0.58 and 0.24; n 6, N 85 1.10 and 0.94;
+// n 5, N 20, 1.7 rounds, 0.27 and 0.33, so that one stays, as do smaller batches: 152 of n 5, N 60 0.15 and
+// 0.26; the rule's worst point is n 6 on short horizons, 2048 of N 20 0.51 and 0.57) or does not fit.
 template <int NX, int NU, int kMinCtas>
 __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(AdjArgs a, RegAdj ra) {
   using M = stage::Mats<NX, NU>;
@@ -785,9 +780,9 @@ __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(
   const int nx = I.nx, nu = I.nu, N = I.N;
   const int k = threadIdx.x, T = blockDim.x, ld = T + 1;
   const bool on = k < N;
-  float4 *sh = reinterpret_cast<float4 *>(adj_smem);       // [NN][T]: sums of hbar and of hbar xbar
-  float2 *sb = reinterpret_cast<float2 *>(sh + NN * T);    // [NN][2][T]: of the adjoints at the two bounds
-  float2 *sx0 = sb + 2 * NN * T;                           // [NX]: of Abar_0^T qbar_0 (stage 0's thread)
+  double2 *sh = reinterpret_cast<double2 *>(adj_smem);     // [NN][T]: sums of hbar and of hbar xbar
+  double *sb = reinterpret_cast<double *>(sh + NN * T);    // [NN][2][T]: of the adjoints at the two bounds
+  double *sx0 = sb + 2 * NN * T;                           // [NX]: of Abar_0^T qbar_0 (stage 0's thread)
   float *sg = reinterpret_cast<float *>(sx0 + 4), *sx = sg + NN * ld;
   M m;
   m.setup(
@@ -795,11 +790,11 @@ __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(
       [&](int q, int i) { return I.Mv(k, q, i); });
 #pragma unroll
   for (int p = 0; p < NN; ++p) {
-    sh[p * T + k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    sb[2 * p * T + k] = sb[(2 * p + 1) * T + k] = make_float2(0.0f, 0.0f);
+    sh[p * T + k] = make_double2(0.0, 0.0);
+    sb[2 * p * T + k] = sb[(2 * p + 1) * T + k] = 0.0;
     sg[p * ld + k] = 0.0f;
     if (k == 0) sg[p * ld + T] = 0.0f;
-    if (k == 0 && p < 4) sx0[p] = make_float2(0.0f, 0.0f);
+    if (k == 0 && p < 4) sx0[p] = 0.0;
   }
   // workspace: checkpoints [nck - 1][4][NN][nt], xb [K][NN][nt], sides [K][nt]
   const int nt = (N + 31) & ~31;
@@ -883,11 +878,7 @@ __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(
         float wb = third(zt);
         const bool low = side >> c & 1u;
         if (low || side >> (NN + c) & 1u) {
-          float2 &o = sb[(2 * c + (low ? 0 : 1)) * T + k];
-          Sum<float> sum;
-          sum.hi = o.x; sum.lo = o.y;
-          sum.add(zt);
-          o = make_float2(sum.hi, sum.lo);
+          sb[(2 * c + (low ? 0 : 1)) * T + k] += widened(zt);
           wb = 0.0f;
         }
         pb[c] = (bb[c] + half) + wb;
@@ -898,12 +889,7 @@ __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(
       for (int c = 0; c < NN; ++c) {
         const float g = m.abar_t(qb, c);
         if (on) sg[c * ld + k] = g;
-        if (k == 0 && c < NX) {
-          Sum<float> sum;
-          sum.hi = sx0[c].x; sum.lo = sx0[c].y;
-          sum.add(g);
-          sx0[c] = make_float2(sum.hi, sum.lo);
-        }
+        if (k == 0 && c < NX) sx0[c] += widened(g);
       }
       M::sym(m.P, pb, ab);
       __syncthreads();
@@ -916,13 +902,12 @@ __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(
       }
 #pragma unroll
       for (int c = 0; c < NN; ++c) {
-        float4 &o = sh[c * T + k];
-        const float4 v = o;
-        Sum<float> h, x;
-        h.hi = v.x; h.lo = v.y; x.hi = v.z; x.lo = v.w;
-        h.add(hb[c]);
-        if (ra.keep_xb) x.add_product(hb[c], xb[c]);
-        o = make_float4(h.hi, h.lo, x.hi, x.lo);
+        double2 &o = sh[c * T + k];
+        double2 v = o;
+        const double hd = widened(hb[c]);
+        v.x += hd;
+        if (ra.keep_xb) v.y = fma(hd, widened(xb[c]), v.y);
+        o = v;
         hb[c] *= m.rho;
         sx[c * ld + k + 1] = hb[c];
       }
@@ -958,13 +943,12 @@ __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(
   for (int c = 0; c < NN; ++c) {
     const int i = stage::component<NX, NU>(c, nx, nu);  // uniform over the CTA
     if (i < 0) continue;
-    const float4 v = sh[c * T + k];
-    const float2 l = sb[2 * c * T + k], u = sb[(2 * c + 1) * T + k];
-    const double qd = (double)I.qd[i], h = on ? (double)v.x + (double)v.y : 0.0, r = rf ? (double)rf[i] : 0.0;
+    const double2 v = sh[c * T + k];
+    const double qd = (double)I.qd[i], h = on ? v.x : 0.0, r = rf ? (double)rf[i] : 0.0;
     if (on && a.g_ref && a.ref_per_stage) a.g_ref[a.L.Nn[j] + (int64_t)k * I.n + i] = qd * h;
-    const double gq = total(r * h - ((double)v.z + (double)v.w));
-    const double glo = total((double)l.x + (double)l.y);
-    const double ghi = total((double)u.x + (double)u.y);
+    const double gq = total(r * h - v.y);
+    const double glo = total(sb[2 * c * T + k]);
+    const double ghi = total(sb[(2 * c + 1) * T + k]);
     const double gref = total(qd * h);
     if (k == 0) {
       if (a.g_ref && !a.ref_per_stage) a.g_ref[a.L.off_n[j] + i] = gref;
@@ -972,7 +956,7 @@ __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(
         if (a.g_q) a.g_q[a.L.off_nx[j] + i] = gq;
         if (a.g_xmin) a.g_xmin[a.L.off_nx[j] + i] = glo;
         if (a.g_xmax) a.g_xmax[a.L.off_nx[j] + i] = ghi;
-        if (a.g_x0) a.g_x0[a.L.off_nx[j] + i] = (double)sx0[c < NX ? c : 0].x + (double)sx0[c < NX ? c : 0].y;
+        if (a.g_x0) a.g_x0[a.L.off_nx[j] + i] = sx0[c < NX ? c : 0];
       } else {
         if (a.g_r) a.g_r[a.L.off_nu[j] + i - nx] = gq;
         if (a.g_umin) a.g_umin[a.L.off_nu[j] + i - nx] = glo;
@@ -1055,7 +1039,7 @@ RegAdjPlan plan_reg_adjoint(const pimpc_solver *s, int Tn, int K, int nck, int s
 
 template <int NX, int NU, int kMinCtas>
 cudaError_t launch_stage_adjoint(const AdjArgs &a, const RegAdjPlan &p, int batch, cudaStream_t st) {
-  const size_t smem = (size_t)(NX + NU) * (32 * p.threads + 8 * (p.threads + 1)) + 4 * sizeof(float2);
+  const size_t smem = (size_t)(NX + NU) * (32 * p.threads + 8 * (p.threads + 1)) + 4 * sizeof(double);
   auto kernel = adjoint_stage_kernel<NX, NU, kMinCtas>;
   const cudaError_t rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (rc != cudaSuccess) return rc;
