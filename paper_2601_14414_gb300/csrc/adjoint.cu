@@ -1041,7 +1041,7 @@ template <int NX, int NU, int kMinCtas>
 cudaError_t launch_stage_adjoint(const AdjArgs &a, const RegAdjPlan &p, int batch, cudaStream_t st) {
   const size_t smem = (size_t)(NX + NU) * (32 * p.threads + 8 * (p.threads + 1)) + 4 * sizeof(double);
   auto kernel = adjoint_stage_kernel<NX, NU, kMinCtas>;
-  const cudaError_t rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t rc = allow_smem((const void *)kernel, smem);
   if (rc != cudaSuccess) return rc;
   kernel<<<batch, p.threads, smem, st>>>(a, p.ra);
   return cudaGetLastError();
@@ -1055,7 +1055,7 @@ cudaError_t launch_reg_adjoint(const AdjArgs &a, const RegAdjPlan &p, int batch,
                                 : launch_stage_adjoint<4, 2, 1>(a, p, batch, st);
   auto kernel = p.NM == 4 ? adjoint_reg_kernel<T, 4> : (p.NM == 8 ? adjoint_reg_kernel<T, 8> : adjoint_reg_kernel<T, 16>);
   const size_t smem = (size_t)4 * p.ra.region * sizeof(T);
-  const cudaError_t rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t rc = allow_smem((const void *)kernel, smem);
   if (rc != cudaSuccess) return rc;
   kernel<<<batch, p.threads, smem, st>>>(a, p.ra);
   return cudaGetLastError();

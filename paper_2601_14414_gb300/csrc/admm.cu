@@ -448,11 +448,11 @@ cudaError_t admm_configure(int precision, size_t smem, int *blocks_per_sm) {
   cudaError_t rc;
   const int threads = admm_threads(precision);
   if (precision == 0) {
-    rc = cudaFuncSetAttribute(admm_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    rc = allow_smem((const void *)admm_kernel<float, false>, smem);
     if (rc != cudaSuccess) return rc;
     rc = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, admm_kernel<float, false>, threads, smem);
   } else {
-    rc = cudaFuncSetAttribute(admm_kernel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    rc = allow_smem((const void *)admm_kernel<double, false>, smem);
     if (rc != cudaSuccess) return rc;
     rc = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, admm_kernel<double, false>, threads, smem);
   }

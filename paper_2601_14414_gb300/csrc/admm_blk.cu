@@ -658,11 +658,11 @@ int64_t blk_region_words(int nx, int nu, int lti, int precision, int S) {
 cudaError_t blk_configure(int precision, size_t smem, int *blocks_per_sm) {
   cudaError_t rc;
   if (precision == 0) {
-    rc = cudaFuncSetAttribute(blk_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    rc = allow_smem((const void *)blk_kernel<float, false>, smem);
     if (rc != cudaSuccess) return rc;
     rc = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, blk_kernel<float, false>, kThreads, smem);
   } else {
-    rc = cudaFuncSetAttribute(blk_kernel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    rc = allow_smem((const void *)blk_kernel<double, false>, smem);
     if (rc != cudaSuccess) return rc;
     rc = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, blk_kernel<double, false>, kThreads, smem);
   }

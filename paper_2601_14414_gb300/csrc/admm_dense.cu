@@ -349,7 +349,7 @@ bool dense_plan(int batch, const int *nx, const int *nu, const int *W, int lti, 
 int dense_threads() { return kThreads; }
 
 cudaError_t dense_configure(size_t smem, int *blocks_per_sm) {
-  const cudaError_t rc = cudaFuncSetAttribute(dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t rc = allow_smem((const void *)dense_kernel, smem);
   if (rc != cudaSuccess) return rc;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, dense_kernel, kThreads, smem);
 }

@@ -371,11 +371,11 @@ int gemm_plan(int max_n, int max_nx, int max_nu, int precision, size_t budget, i
 cudaError_t gemm_configure(int precision, size_t smem, int *blocks_per_sm) {
   cudaError_t rc;
   if (precision == 0) {
-    rc = cudaFuncSetAttribute(gemm_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    rc = allow_smem((const void *)gemm_kernel<float>, smem);
     if (rc != cudaSuccess) return rc;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, gemm_kernel<float>, kGemmThreads, smem);
   }
-  rc = cudaFuncSetAttribute(gemm_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  rc = allow_smem((const void *)gemm_kernel<double>, smem);
   if (rc != cudaSuccess) return rc;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, gemm_kernel<double>, kGemmThreads, smem);
 }

@@ -824,7 +824,7 @@ cudaError_t reg_launch_t(const AdmmLaunch &s, const RegLaunch &rl, cudaStream_t 
                        : lazy     ? pick_kernel<T, kCta, kLazy>(cls, crowded)
                                   : pick_kernel<T, kCta, kSolo>(cls, crowded);
   const size_t smem = (size_t)4 * rl.region * sizeof(T);
-  rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  rc = allow_smem(kernel, smem);
   if (rc != cudaSuccess) return rc;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(s.L.batch * rl.C);

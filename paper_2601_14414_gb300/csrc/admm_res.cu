@@ -345,7 +345,7 @@ cudaError_t launch_t(const AdmmLaunch &s, const ResPlan &pl, size_t smem, cudaSt
       if ((rc = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return rc;
       if ((int64_t)s.L.batch * pl.C > 2 * (int64_t)nsm) kernel = (const void *)resident_kernel<T, 4>;
     }
-    rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    rc = allow_smem(kernel, smem);
     if (rc != cudaSuccess) return rc;
     if (pl.C > 8) {
       rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);

@@ -303,11 +303,11 @@ size_t tb_static_smem(int precision) {
 cudaError_t tb_configure(int precision, size_t smem, int *blocks_per_sm) {
   cudaError_t rc;
   if (precision == 0) {
-    rc = cudaFuncSetAttribute(tb_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    rc = allow_smem((const void *)tb_kernel<float>, smem);
     if (rc != cudaSuccess) return rc;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, tb_kernel<float>, kTbThreads, smem);
   }
-  rc = cudaFuncSetAttribute(tb_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  rc = allow_smem((const void *)tb_kernel<double>, smem);
   if (rc != cudaSuccess) return rc;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, tb_kernel<double>, kTbThreads, smem);
 }

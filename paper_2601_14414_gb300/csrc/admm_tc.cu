@@ -612,7 +612,7 @@ size_t tc_smem_bytes(int nx, int nu) {
 }
 
 cudaError_t tc_configure(size_t smem, int *blocks_per_sm) {
-  cudaError_t rc = cudaFuncSetAttribute(tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t rc = allow_smem((const void *)tc_kernel, smem);
   if (rc != cudaSuccess) return rc;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, tc_kernel, kThreads, smem);
 }

@@ -405,8 +405,7 @@ int tile_threads() { return kTileThreads; }
 int tile_warps() { return kTileWarps; }
 
 cudaError_t tile_configure(size_t smem, int *blocks_per_sm) {
-  cudaError_t rc = cudaFuncSetAttribute(tile_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)smem);
+  cudaError_t rc = allow_smem((const void *)tile_kernel<float>, smem);
   if (rc != cudaSuccess) return rc;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, tile_kernel<float>,
                                                        kTileThreads, smem);

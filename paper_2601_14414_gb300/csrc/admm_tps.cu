@@ -350,11 +350,11 @@ size_t tps_smem_bytes(int nn_max, int precision) {
 cudaError_t tps_configure(int precision, size_t smem, int *blocks_per_sm) {
   cudaError_t rc;
   if (precision == 0) {
-    rc = cudaFuncSetAttribute(tps_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    rc = allow_smem((const void *)tps_kernel<float>, smem);
     if (rc != cudaSuccess) return rc;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, tps_kernel<float>, kThreads, smem);
   }
-  rc = cudaFuncSetAttribute(tps_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  rc = allow_smem((const void *)tps_kernel<double>, smem);
   if (rc != cudaSuccess) return rc;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, tps_kernel<double>, kThreads, smem);
 }

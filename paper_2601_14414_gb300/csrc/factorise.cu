@@ -334,8 +334,7 @@ template <typename T, int kLanes, int kParts>
 cudaError_t launch_lanes(const FactArgs &a, T *blk, int warps, size_t per_group, cudaStream_t stream) {
   const int groups = warps * 32 / kLanes, stages = groups / kParts;
   const size_t smem = per_group * groups + sizeof(double) * a.tab_words;
-  cudaError_t rc = cudaFuncSetAttribute(factorise_kernel<T, kLanes, kParts>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t rc = allow_smem((const void *)factorise_kernel<T, kLanes, kParts>, smem);
   if (rc != cudaSuccess) return rc;
   factorise_kernel<T, kLanes, kParts>
       <<<(unsigned)((a.nblocks + stages - 1) / stages), 32 * warps, smem, stream>>>(a, blk);

@@ -4,6 +4,9 @@
 
 namespace pimpc {
 
+// A launch of `kernel` on the current device may take `bytes` of dynamic shared memory (see smem_limit.h).
+cudaError_t allow_smem(const void *kernel, size_t bytes);
+
 cudaError_t launch_factorise(const Layout &L, const double *A, const double *B, const double *e,
                              const double *qd, const double *rdu, double rho, const int *binst,
                              const int64_t *bbase, int64_t nblocks, int max_nx, int max_n,

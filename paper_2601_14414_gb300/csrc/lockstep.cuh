@@ -521,7 +521,7 @@ cudaError_t launch_sequence(const AdmmLaunch &s, Args<T> &a, const void *kernel,
   set_control_kernel<<<1, 1, 0, stream>>>(s.ctl, s.nitems, s.L.batch, s.bar_limit);
   if ((rc = cudaGetLastError()) != cudaSuccess) return rc;
   if (s.max_iters > 0) {
-    rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    rc = allow_smem(kernel, smem);
     if (rc != cudaSuccess) return rc;
     // Cooperative launch (all CTAs co-resident: the grid barrier relies on it), issued through
     // cudaLaunchKernelExC so that it can also be recorded into a CUDA graph.

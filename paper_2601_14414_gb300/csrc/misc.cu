@@ -1,7 +1,28 @@
 // misc.cu -- elementwise marshalling kernels: FP64 ABI arrays <-> the solver's internal layout.
 #include "lockstep.cuh"
+#include "smem_limit.h"
 
 namespace pimpc {
+
+namespace {
+struct SmemLimit {
+  const void *kernel;
+  int get(std::size_t *bytes) const {
+    cudaFuncAttributes at;
+    const cudaError_t rc = cudaFuncGetAttributes(&at, kernel);
+    *bytes = rc == cudaSuccess ? (std::size_t)at.maxDynamicSharedSizeBytes : 0;
+    return rc;
+  }
+  int set(std::size_t bytes) const {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  }
+};
+std::mutex g_smem_mu;
+}  // namespace
+
+cudaError_t allow_smem(const void *kernel, size_t bytes) {
+  return (cudaError_t)raise_smem_limit(SmemLimit{kernel}, g_smem_mu, bytes);
+}
 
 namespace {
 
