@@ -232,7 +232,7 @@ def profiled_traffic(family):
 def oracle_sample(insts, cfg, seconds_hint, rng_seed=0, keep=False):
     """The FP64 oracle (Algorithm 1, same eps and iteration cap) on random instances of the
     workload, all host cores, grown until about `seconds_hint` seconds. Returns (count, seconds,
-    threads, indices[, results])."""
+    threads, indices, results); the results only with `keep` (else none are held)."""
     import oracle
     threads = os.cpu_count() or 1
     rng = np.random.default_rng(rng_seed)
@@ -253,9 +253,7 @@ def oracle_sample(insts, cfg, seconds_hint, rng_seed=0, keep=False):
         if time.perf_counter() - t0 >= seconds_hint:
             break
     dt = time.perf_counter() - t0
-    if keep:
-        return done, dt, threads, order[:done], results
-    return done, dt, threads, order[:done]
+    return done, dt, threads, order[:done], results
 
 
 def oracle_converged(insts, idx):
@@ -918,7 +916,7 @@ def run_ours(args):
         cpu = None
         oracle_score = None
         if not args.no_cpu_baseline:
-            n_cpu, dt_cpu, cores, idx_cpu = oracle_sample(insts, cfg, 20.0)
+            n_cpu, dt_cpu, cores, idx_cpu, _ = oracle_sample(insts, cfg, 20.0)
             cpu = dict(value=n_cpu / dt_cpu, unit="solves/s", cores=cores, kind="oracle",
                        sample=f"{n_cpu} random instances of the {batch}-instance workload "
                               f"(all iterations to the same eps), {dt_cpu:.1f} s")
