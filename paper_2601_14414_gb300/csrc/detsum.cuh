@@ -3,10 +3,14 @@
 // butterfly with its shuffles about 570), and the sum of c^{i+1} sits on the critical path of
 // every iteration of a single-instance solve. Here the lanes agree on the largest exponent, shift
 // their significands to it and add them as integers (redux.sync on limbs): no FP64 instruction,
-// and a result that does not depend on the order of the lanes. What the shifts cut off is below
-// 2^-56 of the largest value per summand, less than the rounding of a chain of double additions.
+// and a result that does not depend on the order of the lanes. What the shifts cut off of a summand is
+// below 2^-53 of the largest value's leading bit for floats (limbs.cuh), 2^-57 for doubles and for the
+// sums of warps: no more than a double addition may round off, and nothing where the values are within
+// 2^30 of each other.
 #pragma once
 #include <cuda_runtime.h>
+
+#include "limbs.cuh"
 
 namespace pimpc {
 namespace detsum {
@@ -33,13 +37,10 @@ __device__ __forceinline__ Fx warp_sum(float v) {
   const int e = x == 0xff ? 1 << 10 : (x ? x : 1);
   const int em = __reduce_max_sync(0xffffffffu, e);
   if (em == 1 << 10) return special_sum(Fx{m ? 1ull : 0ull, x == 0xff ? kSpecial : 0});
-  const int sh = em - e;
-  const unsigned long long q =
-      sh < 64 ? ((unsigned long long)(x ? (m | 0x800000u) : m) << 27) >> sh : 0ull;
-  const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)q & 0x3ffffffu);
-  const unsigned l1 = __reduce_add_sync(0xffffffffu, (unsigned)(q >> 26));
-  // v = (24-bit m) 2^(x - 150), q = m 2^27
-  return Fx{(unsigned long long)l0 + ((unsigned long long)l1 << 26), em - 177 + kBias};
+  const Limbs q = split(x ? m | 0x800000u : m, em - e);
+  const unsigned l0 = __reduce_add_sync(0xffffffffu, q.lo);
+  const unsigned l1 = __reduce_add_sync(0xffffffffu, q.hi);
+  return Fx{join(l0, l1), exponent(em) + kBias};
 }
 
 __device__ __forceinline__ Fx add_limbs(unsigned long long q, int e) {
