@@ -40,14 +40,19 @@ void reg_plan(int batch, const int *nx, const int *nu, const int *N, int precisi
 // an exchange through global memory, or instances that no cluster holds) the fewest CTAs within
 // `grid` (n 16, N 200, FP64: 7.15 us on a cluster of 16, 4.93 on 32 CTAs of 160 threads, 4.73 on 40 of
 // 128, 4.72 on 64; n 3, N 5000: 4.12 on 96, 3.65 on 128; n 16, N 100: 4.67 on the cluster and on 32).
-// Batches larger than the SMs take the fewest CTAs that hold an instance.
+// Batches larger than the SMs take the fewest CTAs that hold an instance; clusters of 5 and 6 only where
+// they make two and a half rounds of CTAs or more, because the GPCs hold them unevenly (FP64, n 16, 30
+// iterations, the shared-memory kernel / 8 / 5 or 6 CTAs: N 60, 76 instances 908 / 1051 / 667 us, 304 3557 /
+// 3664 / 2425; N 80, 76 1120 / 1176 / 981; FP32, n 16, N 121, 76 369 / 389 / 215; N 70, 60 instances 1102 /
+// 709 / 737).
 static RegLaunch choose_reg(int item_scale, int batch, const int *nx, const int *nu, const int *N,
                             int precision, int nsm) {
   const bool f32 = precision == 0;
   const int one = f32 ? 480 : 128, few = f32 ? 160 : 128, most = f32 ? 1024 : 160, grid = f32 ? 512 : 128;
   RegLaunch best;
-  for (int cand : {1, 2, 4, 8, 16, 24, 32, 40, 48, 64, 80, 96, 112, 128, 144}) {
+  for (int cand : {1, 2, 4, 5, 6, 8, 16, 24, 32, 40, 48, 64, 80, 96, 112, 128, 144}) {
     if (item_scale > 0 && cand != item_scale) continue;
+    if ((cand == 5 || cand == 6) && (item_scale > 0 || 2 * (int64_t)batch * cand < 5 * (int64_t)nsm)) continue;
     RegLaunch t;
     t.C = cand;
     reg_plan(batch, nx, nu, N, precision, &t);

@@ -126,3 +126,26 @@ def test_fp32_stall_stop(cls):
         err = max(np.max(np.abs(r["u"][j] - o["u"])), np.max(np.abs(r["x"][j] - o["x"])))
         assert err <= 1e-4 * scale, j
     s.close()
+
+
+@pytest.mark.parametrize("precision,dims", [
+    (pimpc.F64, [(12, 4, 60), (11, 4, 43)]), (pimpc.F64, [(12, 4, 83), (9, 5, 80)]),
+    (pimpc.F32, [(12, 4, 121), (13, 3, 33)]), (pimpc.F32, [(14, 2, 150)]),
+])
+def test_clusters_of_five_and_six(precision, dims):
+    # batches of two and a half rounds of CTAs or more whose largest instance needs more than four CTAs
+    some = [W.random_ltv(8900 + j, *dims[j % len(dims)]) for j in range(4)]
+    count = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    K = 60
+    ora = oracle.solve_batch(some, eps=-1.0, max_iters=K, accel=1, history=True)
+    mask = np.ascontiguousarray(np.stack([ora[j % 4]["mask"] for j in range(count)]).astype(np.uint8))
+    s = pimpc.Solver([some[j % 4] for j in range(count)], precision=precision, eps=-1.0, max_iters=K, accel=1)
+    s.set_schedule(pimpc.FAMILY_RESIDENT)
+    pimpc.pimpc_set_restart_mask(s.h, mask, K)
+    r = s.solve()
+    tol = 1e-10 if precision == pimpc.F64 else 1e-4
+    for j in range(count):
+        o = ora[j % 4]
+        assert r["iters"][j] == K
+        assert relerr(r["u"][j], o["u"]) <= tol and relerr(r["x"][j], o["x"]) <= tol, j
+    s.close()
