@@ -324,8 +324,10 @@ static int64_t dense_words(int nx, int nu, int W, int lti, int SL, int *blk, int
   return (int64_t)*blk + *halo + 6 * (int64_t)*vec;
 }
 
-// Slots per sub-chunk of each instance within the shared memory of three CTAs per SM (at least two
-// stages' worth, within one CTA's), the launch's regions; false if an instance does not fit, or if a CTA's
+// Slots per sub-chunk of each instance, at least two stages' worth, within a third of an SM's shared
+// memory, and the launch's regions. Each region is the largest over the instances, so that a batch of
+// one size runs three CTAs per SM, as the kernel is compiled for, and one of many sizes may run two (the
+// 256 uneven instances: 82,688 bytes, two CTAs). False if an instance does not fit, or if a CTA's
 // threads give one fewer than five slots (n > 51): with four a quarter of them hold the next stage,
 // and the lane groups win (304 stage-invariant instances, N 200: n 48, five slots, 1.70 ms per
 // iteration in lane groups, 1.12 here; n 56 1.95 and 2.63; 256 of n 64, N 1000 11.9 and 13.7).

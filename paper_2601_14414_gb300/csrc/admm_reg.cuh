@@ -20,8 +20,8 @@
 // arithmetic (detsum.cuh) off the 64-cycle FP64 pipe. Within a cluster the data go by st.async
 // into the others' shared memory and complete on their mbarriers (520-660 cycles per exchange,
 // measured; remote stores and a cluster barrier 890 and more); beyond 16 CTAs they go through
-// global memory as 16-byte records that carry their iteration number (1400-1600 cycles for up
-// to 96 CTAs; a barrier on an atomic counter takes 2500 before any data are read).
+// global memory as 16-byte records that carry their iteration number (1400-1600 cycles, measured with
+// 16 to 96 CTAs; a barrier on an atomic counter takes 2500 before any data are read).
 // The launch also makes the starting iterates and the outputs: one kernel per solve.
 // FP64 is bound by its pipe (a warp issues one FP64 instruction per 64 cycles, an SM one per 19),
 // so the FP64 code counts instructions: one chain per dot product, with the sums around it folded

@@ -97,7 +97,7 @@ cudaError_t launch_resident(const AdmmLaunch &s, int precision, const int *plan,
                             cudaStream_t stream);
 
 // The same for n <= 16 with the stage data in registers: threads (0: does not fit) and vector
-// region of one CTA for C CTAs per instance.
+// region of one CTA for C CTAs per instance (up to 16 a cluster, beyond that a cooperative launch).
 struct RegLaunch {
   int C = 0, threads = 0, region = 0, nmax = 0;  // threads == 0: the shared-memory kernel runs
   size_t xch_bytes = 0;                          // C > 16: exchange records in global memory
@@ -145,9 +145,10 @@ cudaError_t launch_tb(const AdmmLaunch &s, int precision, int T, size_t smem, cu
 // Schedule of the batched solve: which kernel family and how its work is cut.
 struct Schedule {
   int family = -1;       // 0: lane groups on plain stage blocks; 2: one thread per stage on halo
-                         // tiles (stage-varying FP32 only); 3: every instance resident in the
-                         // shared memory of one CTA or a cluster (item_scale = CTAs per
-                         // instance, 0: the fewest that fit); 4: stage-invariant instances as
+                         // tiles (stage-varying FP32 only); 3: every instance resident on chip,
+                         // in registers (n <= 16) or shared memory of one CTA, a cluster or more
+                         // CTAs (item_scale = CTAs per instance, 0: by the sizes, see
+                         // plan_resident); 4: stage-invariant instances as
                          // dense contractions over blocks of stages; 5: lane groups owning
                          // 4-column blocks on blocked stage blocks; 6: stage-invariant FP32
                          // instances with the stage products on the tensor cores; 7: temporal

@@ -16,11 +16,12 @@
 //
 // The arithmetic is that of pimpc_solve: the same factorisation, solve and output kernels run
 // on the same memory layout, with their buffers carved out of the static array. An instance that
-// the resident schedule holds (registers or shared memory of one CTA, a cluster or a few dozen
-// CTAs; see plan_resident) runs on it: one instance leaves the lock-step frame waiting on its grid
-// barrier (n 16, N 200, 100 FP32 iterations: 8.81 ms there, 0.17 ms resident, all launches counted). Its momentum factors
-// come from a constant table, filled once per device together with the array's address; longer
-// runs, and instances too long for a cluster, use one thread per stage on tiles.
+// the resident schedule holds (registers of one CTA, a cluster or up to 144 CTAs, shared memory of
+// a CTA or a cluster; see plan_resident) runs on it: one instance leaves the lock-step frame waiting
+// on its grid barrier (n 16, N 200, 100 FP32 iterations: 8.81 ms there, 0.17 ms resident, all launches
+// counted). Its momentum factors come from a constant table, filled and waited for once per device
+// together with the array's address (static_arrays.h); longer runs, and instances too long for a
+// cluster, use one thread per stage on tiles.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
