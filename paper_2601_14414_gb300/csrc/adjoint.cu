@@ -506,10 +506,11 @@ __global__ void __launch_bounds__(256) adjoint_kernel(AdjArgs a) {
 // was clamped to (two bits) and, for the weights' gradient, xb. Both are kept for a whole segment
 // (every iteration at once when that takes no more memory than the checkpoints and states of the
 // sweep above), in place of K full states. The gradient sums run in FP64, as above: three additions per
-// thread and iteration, 4 % of an FP32 iteration here (1300 -> 1353 us, 600 instances of n 16, N 30,
-// against sums in float pairs, which lose FP64's range and its last five bits). What bounds it is the
-// issue rate of one CTA of 512 threads per SM between three barriers per iteration; two CTAs per SM (64
-// registers, spills) took 1.17 times as long. Batches that crowd the SMs go to adjoint_stage_kernel below.
+// thread and iteration, taken at the start of the next one, 3 % of an FP32 iteration (600 instances of n
+// 16, N 30: 1300 us with sums in float pairs, which lose FP64's range and its last five bits, 1354 with
+// FP64 sums where their terms arise, 1340 so). What bounds it is the issue rate of one CTA of 512 threads
+// per SM between three barriers per iteration; two CTAs per SM (64 registers, spills) took 1.17 times as
+// long. Batches that crowd the SMs go to adjoint_stage_kernel below.
 struct RegAdj {
   int region;       // elements of each of the four vector regions in shared memory
   int K, nck;       // iterations per segment, segments
@@ -664,9 +665,16 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
     }
     for (int m = 0; m < len; ++m) forward(m);
     __syncthreads();  // the bits of this segment (written by lane 0), and the regions' last reads
+    T hb = 0, xb = 0;
+    auto sums = [&]() {
+      const double hd = widened(hb);
+      hs += hd;
+      if (ra.keep_xb) hx = fma(hd, widened(xb), hx);
+    };
     for (int m = len - 1; m >= 0; --m) {
       const uint2 side = kept ? bits[(int64_t)m * nw + warp] : make_uint2(0u, 0u);
-      const T xb = ra.keep_xb && kept ? xbs[(int64_t)m * nt + tid] : (T)0;
+      sums();
+      if (ra.keep_xb && kept) xb = xbs[(int64_t)m * nt + tid];
       const bool below = side.x >> lane & 1u, above = side.y >> lane & 1u;
       const T half = (T)0.5 * (vb - bb);
       const T zt = (zb - tb) + half;
@@ -702,10 +710,7 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
       __syncthreads();
       T rh = (T)0;
       if (on) {
-        const T hb = dot(Hr, s2 + row, n, (T)0);
-        const double hd = widened(hb);
-        hs += hd;
-        if (ra.keep_xb) hx = fma(hd, widened(xb), hx);
+        hb = dot(Hr, s2 + row, n, (T)0);
         rh = rho * hb;
         s3[at + nv] = rh;  // row k + 1, read by stage k + 1
       }
@@ -717,6 +722,7 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
       tb = sb - rh;
       bb = (pb + qb) - (yb + ab);
     }
+    sums();
   }
 
   // Gradients: sums over the stages, pairwise.
@@ -763,12 +769,13 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
 // read again for every segment, and the FP64 gradient sums live in shared memory, one 16-byte access per
 // component and iteration each way. The clamp sides take a 16-bit word per stage and iteration.
 // What bounds it is instruction issue, then the FP64 pipe, which ten sums per warp and iteration take for
-// 190 cycles of the SM's (training batch, 1024 of n 5, N 100, 150 iterations: 1.13 ms, 0.97 with sums in
-// float pairs); its chains are longer than those of a thread per component, so it wins where a batch takes
-// that one more than two rounds of CTAs (100 iterations, 1024 instances, thread per component and per
-// stage: n 5, N 100 1.21 and 0.79 ms, N 60 0.98 and 0.42; n 3, N 60 0.58 and 0.24; n 6, N 85 1.10 and 0.94;
-// n 5, N 20, 1.7 rounds, 0.27 and 0.33, so that one stays, as do smaller batches: 152 of n 5, N 60 0.15 and
-// 0.26; the rule's worst point is n 6 on short horizons, 2048 of N 20 0.51 and 0.57) or does not fit.
+// 190 cycles of the SM's (training batch, 1024 of n 5, N 100, 150 iterations: 1.04 ms; 0.97 with sums in
+// float pairs; 1.13 with each sum where its term arises, where its warp has nothing else to issue). Its
+// chains are longer than those of a thread per component, so it wins where a batch takes that one more
+// than two rounds of CTAs (100 iterations, 1024 instances, thread per component and per stage: n 5, N 100
+// 1.17 and 0.71 ms, N 60 0.95 and 0.38; n 3, N 60 0.54 and 0.22; n 6, N 85 1.05 and 0.93; n 5, N 20, 1.7
+// rounds, 0.26 and 0.30, so that one stays, as do smaller batches: 152 of n 5, N 60 0.14 and 0.24; the
+// rule's worst points are n 6 on short horizons, 2048 of N 20 0.51 and 0.56) or does not fit.
 template <int NX, int NU, int kMinCtas>
 __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(AdjArgs a, RegAdj ra) {
   using M = stage::Mats<NX, NU>;
@@ -864,12 +871,23 @@ __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(
 #pragma unroll
       for (int c = 0; c < NN; ++c) sx[c * ld] = 0.0f;
     }
+    // The sums of an iteration are added at the start of the next, where there is work to run beside them.
+    float hb[NN];
+#pragma unroll
+    for (int c = 0; c < NN; ++c) hb[c] = xb[c] = 0.0f;
+    auto sums = [&]() {
+#pragma unroll
+      for (int c = 0; c < NN; ++c) {
+        double2 v = sh[c * T + k];
+        const double hd = widened(hb[c]);
+        v.x += hd;
+        if (ra.keep_xb) v.y = fma(hd, widened(xb[c]), v.y);
+        sh[c * T + k] = v;
+      }
+    };
     for (int q = len - 1; q >= 0; --q) {
       side = kept ? sides[(int64_t)q * nt + k] : 0u;
-      if (ra.keep_xb && kept) {  // loaded well before their use
-#pragma unroll
-        for (int c = 0; c < NN; ++c) xb[c] = (xbs + (int64_t)q * NN * nt + k)[c * nt];
-      }
+      sums();
       float pb[NN], qb[NN], ab[NN];
 #pragma unroll
       for (int c = 0; c < NN; ++c) {
@@ -885,6 +903,10 @@ __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(
         qb[c] = wb - half;
         tb[c] = fmaf(2.0f, wb, tb[c]);  // the adjoint of s = xb + theta
       }
+      if (ra.keep_xb && kept) {
+#pragma unroll
+        for (int c = 0; c < NN; ++c) xb[c] = (xbs + (int64_t)q * NN * nt + k)[c * nt];
+      }
 #pragma unroll
       for (int c = 0; c < NN; ++c) {
         const float g = m.abar_t(qb, c);
@@ -893,7 +915,6 @@ __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(
       }
       M::sym(m.P, pb, ab);
       __syncthreads();
-      float hb[NN];
       {
         float xt[NN];
 #pragma unroll
@@ -901,29 +922,21 @@ __global__ void __launch_bounds__(kStageThreads, kMinCtas) adjoint_stage_kernel(
         M::sym(m.H, xt, hb);
       }
 #pragma unroll
-      for (int c = 0; c < NN; ++c) {
-        double2 &o = sh[c * T + k];
-        double2 v = o;
-        const double hd = widened(hb[c]);
-        v.x += hd;
-        if (ra.keep_xb) v.y = fma(hd, widened(xb[c]), v.y);
-        o = v;
-        hb[c] *= m.rho;
-        sx[c * ld + k + 1] = hb[c];
-      }
+      for (int c = 0; c < NN; ++c) sx[c * ld + k + 1] = m.rho * hb[c];
       __syncthreads();
       float xp[NN];
 #pragma unroll
       for (int c = 0; c < NN; ++c) xp[c] = sx[c * ld + k];
 #pragma unroll
       for (int c = 0; c < NN; ++c) {
-        const float yb = m.abar(xp, c, 0.0f);
-        zb[c] = hb[c] + yb;
+        const float yb = m.abar(xp, c, 0.0f), rh = m.rho * hb[c];
+        zb[c] = rh + yb;
         vb[c] = ab[c] - yb;
-        tb[c] -= hb[c];
+        tb[c] -= rh;
         bb[c] = (pb[c] + qb[c]) - (yb + ab[c]);
       }
     }
+    sums();
   }
   // Gradients: sums over the stages, pairwise.
   const float *rf = on ? I.refk(k) : nullptr;
