@@ -595,14 +595,13 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
   T z = 0, v = 0, t = 0, b = 0;
   // One forward iteration; m >= 0: keep its clamp bits and xb as the segment's m-th.
   auto forward = [&](int m) {
-    const T be = b + ee;
     if (on) {
       s0[at] = v - b;
-      s1[at] = (z - v) - be;
+      s1[at] = (z - v) - (b + ee);
     }
     if (tid < n) s3[tid] = x0;  // row 0: xbar_0; row k + 1: xbar_{k+1}
     __syncthreads();
-    T p = (T)0;
+    T bd = (T)0;
     if (on) {
       T acc = z - t;
       if (more) {
@@ -610,7 +609,7 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
         acc = dot(Gn, s1 + row + nv, nx, acc);
       }
       s2[at] = qref + rho * acc;
-      p = dot(Pr, s0 + row, n, b);
+      bd = dot(Pr, s0 + row, n, (T)0);
     }
     __syncthreads();
     T xb = (T)0;
@@ -621,15 +620,13 @@ __global__ void __launch_bounds__(adj_max_threads((int)sizeof(T), NM)) adjoint_r
     __syncthreads();
     bool below = false, above = false;
     if (on) {
-      const T q = dot(Gr, s3 + row, n, be);
-      const T s = xb + t;
-      const T w = third((T)2 * s + (p + q));
-      below = w <= lo;
-      above = !below && w >= hi;
-      z = w < lo ? lo : (w > hi ? hi : w);
-      v = (T)0.5 * (z + (p - q));
-      t = s - z;
-      b = p - v;
+      const Step<T> r = steps23(xb, bd, dot(Gr, s3 + row, n, ee), t, b, lo, hi);
+      below = r.w <= lo;
+      above = !below && r.w >= hi;
+      z = r.z;
+      v = r.v;
+      t = r.t;
+      b = r.b;
     }
     if (m >= 0) {
       const unsigned bl = __ballot_sync(0xffffffffu, below), ab = __ballot_sync(0xffffffffu, above);

@@ -216,11 +216,9 @@ __global__ void __launch_bounds__(kThreads, 3) dense_kernel(ls::Args<double> a, 
         const double *Gk1 = lti ? rHalo : rB + (slot + 1) * W;       // G_{k+1}
         const double *Hk = (lti ? rHalo + ((k < N - 1) ? 0 : W) : Gk) + oH;
         // ---- w = v - beta, y = z - v - beta - ebar ----
-        double be = 0.0;  // ebar - lambda
         if (owned || next) {
-          be = bh + (c < nx ? Gk[oE + c] : 0.0);
           if (owned) sW[slot * nv + c] = vh - bh;
-          sY[slot * nv + c] = (zh - vh) - be;
+          sY[slot * nv + c] = (zh - vh) - (bh + (c < nx ? Gk[oE + c] : 0.0));
         }
         if (tid < n) sX[tid] = sc > 0 ? sX[S * nv + tid] : (ka == 0 ? a.xb0[a.L.off_n[j] + tid] : 0.0);
         __syncthreads();
@@ -257,27 +255,24 @@ __global__ void __launch_bounds__(kThreads, 3) dense_kernel(ls::Args<double> a, 
         // ---- steps 2-4 ----
         if (owned) {
           const double *xk = sX + slot * nv, *du = sD + slot * nuv;
-          double bd, qv;  // Bbar du, Abar xbar + ebar - lambda
+          double bd, ax;  // Bbar du, Abar xbar + ebar
           if (c < nx) {
             const double *row = Gk + c * ldg;  // odd stride: the lanes' rows hit distinct banks
-            qv = dot_strided(row, 1, xk, n, be);
+            ax = dot_strided(row, 1, xk, n, Gk[oE + c]);
             bd = dot_strided(row + nx, 1, du, nu, 0.0);
           } else {
-            qv = be + xk[c];
+            ax = xk[c];
             bd = du[c - nx];
           }
-          const double s = xb + th, p = bh + bd;
-          const double z = clamp(third(2.0 * s + (p + qv)), lo, hi);
-          const double v = 0.5 * (z + (p - qv));
-          const double t = s - z, b = p - v;
+          const Step<double> r = steps23(xb, bd, ax, th, bh, lo, hi);
           double *o = In + (int64_t)k * n5p + c;
-          o[0] = z;
-          o[n] = v;
-          o[2 * n] = t;
-          o[3 * n] = b;
-          o[4 * n] = negated(b);
+          o[0] = r.z;
+          o[n] = r.v;
+          o[2 * n] = r.t;
+          o[3 * n] = r.b;
+          o[4 * n] = negated(r.b);
           // theta' - theta = xbar - z' and beta' - beta = Bbar du - v', without the duals' own rounding
-          const double d1 = xb - z, d2 = bd - v, d4 = z - zh, d5 = v - vh;
+          const double d1 = xb - r.z, d2 = bd - r.v, d4 = r.z - zh, d5 = r.v - vh;
           // d1^2 + d2^2 + d3^2 + d4^2 + d5^2 + (d4 - d5)^2 with d3 = -d2
           const double g = d2 * d2 + (d4 * d4 + d5 * (d5 - d4));
           cacc = fma(d1, d1, fma(2.0, g, cacc));

@@ -313,10 +313,9 @@ struct Lane {
       th = tc + f * (tc - tp);
       bh = bc + f * (bc - bp);
     }
-    const T be = bh + ee;  // ebar - lambda
     if (active) {
       sW[slot * nv + c] = vh - bh;
-      sY[slot * nv + c] = (zh - vh) - be;
+      sY[slot * nv + c] = (zh - vh) - (bh + ee);
     }
     sync();
     // ---- Abar_{k+1}^T y_{k+1}, h_k; Bbar du = P_k w_k ----
@@ -343,13 +342,11 @@ struct Lane {
     cacc = (T)0;
     zn = vn = tn = bn = (T)0;
     if (owned) {
-      const T q = dot(Gr, sX + slot * nv, n, be);  // Abar xbar + ebar - lambda
-      const T s = xb + th, p = bh + bd;
-      const T w = third((T)2 * s + (p + q));
-      zn = clamp(w, lo, hi);
-      vn = (T)0.5 * (zn + (p - q));
-      tn = s - zn;
-      bn = p - vn;
+      const Step<T> r = steps23(xb, bd, dot(Gr, sX + slot * nv, n, ee), th, bh, lo, hi);
+      zn = r.z;
+      vn = r.v;
+      tn = r.t;
+      bn = r.b;
       // theta' - theta = xbar - z' and beta' - beta = Bbar du - v', without the duals' own rounding
       if constexpr (kShare) cacc = share(xb - zn, bd - vn, zn - zh, vn - vh);
     }

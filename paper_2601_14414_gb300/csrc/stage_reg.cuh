@@ -155,21 +155,18 @@ struct Iter {
     side = 0u;
 #pragma unroll
     for (int r = 0; r < NN; ++r) {
-      const float q = m.abar(xp, r, r < NX ? b[r] + e[r < NX ? r : 0] : b[r]);  // Abar xbar + ebar - lambda
-      const float s = xb[r] + t[r], p = b[r] + bd[r];
-      const float w = third(2.0f * s + (p + q));
-      if (kSide) side |= w <= lo[r] ? 1u << r : (w >= hi[r] ? 1u << (NN + r) : 0u);
-      const float zn = clamp(w, lo[r], hi[r]);
-      const float vn = 0.5f * (zn + (p - q));
+      const float ax = m.abar(xp, r, r < NX ? e[r < NX ? r : 0] : 0.0f);  // Abar xbar + ebar
+      const Step<float> o = steps23(xb[r], bd[r], ax, t[r], b[r], lo[r], hi[r]);
+      if (kSide) side |= o.w <= lo[r] ? 1u << r : (o.w >= hi[r] ? 1u << (NN + r) : 0u);
       if (kShare) {  // the duals' differences without their own rounding, as in admm_reg.cuh
-        const float d1 = xb[r] - zn, d2 = bd[r] - vn, d4 = zn - z[r], d5 = vn - v[r];
+        const float d1 = xb[r] - o.z, d2 = bd[r] - o.v, d4 = o.z - z[r], d5 = o.v - v[r];
         g += d2 * d2 + (d4 * d4 + d5 * (d5 - d4));
         d += d1 * d1;
       }
-      z[r] = zn;
-      v[r] = vn;
-      t[r] = s - zn;
-      b[r] = p - vn;
+      z[r] = o.z;
+      v[r] = o.v;
+      t[r] = o.t;
+      b[r] = o.b;
     }
     if (kShare) share = on ? 2.0f * g + d : 0.0f;
     return false;
