@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(256) adjoint_kernel(AdjArgs a) {
 //   w = v - beta, y = z - v - beta - ebar, h = Qbar ref + rho (z - theta + Abar_{k+1}^T y_{k+1}),
 //   xb = H h, p = beta + P w, q = Abar xb_{k-1} + beta + ebar, s = xb + theta,
 //   z' = clamp((2 s + p + q) / 3), v' = (z' + p - q) / 2, theta' = s - z', beta' = p - v'
-// reverses to
+// (computed with the beta of p + q and of p - q taken together, steps23 in regvec.cuh) reverses to
 //   vt = v'bar - beta'bar, zt = z'bar - theta'bar + vt / 2, wb = zt / 3 where w was inside the box,
 //   pb = beta'bar + vt / 2 + wb, qb = wb - vt / 2, sb = theta'bar + 2 wb,
 //   xbbar = sb + Abar_{k+1}^T qb_{k+1}, hbar = H xbbar, yb = Abar_k rho hbar_{k-1},

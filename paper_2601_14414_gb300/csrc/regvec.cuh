@@ -72,10 +72,10 @@ __device__ __forceinline__ double clamp(double w, double lo, double hi) {
 }
 
 // Steps 2-3 of one component in the reduced form (lambda = -beta): xb = xbar, bd = Bbar du, ax = Abar xbar
-// + ebar, th and b the duals' hats. gamma = bd + beta - ax + lambda is bd - ax, without the duals: summed
-// as (beta + bd) - (beta + ax), two operations fewer where beta starts ax's dot product, it carried
-// beta's rounding into v, and the iterates' error against wider arithmetic was up to 1.6 times as large
-// (stage-invariant n 8 and n 5, FP32 and FP64).
+// + ebar, th and b the duals' hats. gamma = bd + beta - ax + lambda is bd - ax, without the duals. Summed
+// as (beta + bd) - (beta + ax), one operation fewer where beta starts ax's dot product, it carries beta's
+// rounding into v: the rms error of x against FP64 then is 1.25 times that of the unreduced iteration
+// for the cart-poles (FP32 and FP64 alike), and 0.73 and 0.94 times so.
 template <typename T>
 struct Step {
   T w, z, v, t, b;
