@@ -8,11 +8,11 @@
 // iterate in registers, multiplies without loads, and exchanges two n-vectors with its neighbours:
 // Abar_k^T y_k, formed by the thread that holds G_k, to stage k - 1, and xbar_{k+1} to stage k + 1, two
 // barriers in all. The iteration is the reduced one of admm_reg.cuh (lambda = -beta throughout). What limits the warps of an SM is the
-// registers of a thread: 71 at 2 + 1 components, 128 at 4 + 1, 167 at 4 + 2.
-// Per solve of 150 iterations, against a thread per component: 1024 instances of n 5, N 100 629 -> 244
-// us, N 20 139 -> 92, N 150 (more components than a CTA has threads: clusters of two CTAs) 3.68 -> 0.35
-// ms; 153 instances of N 100 176 -> 89; one instance of n 5, N 60 82 -> 62, N 256 160 -> 90; n 3, N 20
-// 59 -> 33; slower by 4 % at most (n 5, one stage, 53 -> 55), so that the batch does not matter.
+// registers of a thread: 69 at 2 + 1 components, 125 at 4 + 1, 167 at 4 + 2.
+// Per solve of 150 iterations, against a thread per component: 1024 instances of n 5, N 100 629 -> 217
+// us, N 20 139 -> 76, N 150 (more components than a CTA has threads: clusters of two CTAs) 3.68 -> 0.32
+// ms; 153 instances of N 100 176 -> 76; one instance of n 5, N 60 82 -> 55, N 256 160 -> 79; n 3, N 20
+// 59 -> 37; slower by 4 % at most (n 5, one stage, 53 -> 55), so that the batch does not matter.
 #include <math.h>
 
 #include "detsum.cuh"
